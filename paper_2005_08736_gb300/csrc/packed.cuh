@@ -178,50 +178,54 @@ __device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas
   }
 }
 
-// WENO5 end values with nonlinear weights (weno5_pair, WENO-JS or WENO-Z) of
-// two columns at once: the candidate polynomials, smoothness indicators,
-// weights and combinations in pair arithmetic; |beta0 - beta2| and the
-// reciprocals per half.
+// Nonlinear WENO5 end values of two columns at once, as six times their
+// deviations from the centre averages (weno5_dev in recon.cuh, the same
+// differences, candidates and weights in pair arithmetic; |beta0 - beta2| and
+// the reciprocals per half).
+template <int MODE>
+HGKS_HD void weno5_dev_x2(float2 q0, float2 q1, float2 q2, float2 q3, float2 q4, float2& rL, float2& rR) {
+  const float2 one = bc2(1.f), two = bc2(2.f);
+  const float2 D1 = sub2(q1, q0), D2 = sub2(q2, q1), D3 = sub2(q3, q2), D4 = sub2(q4, q3);
+  const float2 s0 = sub2(D2, D1), s1 = sub2(D3, D2), s2 = sub2(D4, D3);
+  const float2 t0 = fma2(two, D2, s0), t1 = add2(D2, D3), t2 = sub2(add2(D3, D3), s2);
+  const float2 w = add2(t0, D2), z = add2(t2, D3);
+  const float2 c0 = add2(w, s0), c1 = add2(t1, D3), e0 = sub2(z, s2), e1 = add2(t1, D2);
+  const float2 k = bc2(3.f / 13.f);
+  const float2 b0 = fma2(mul2(k, t0), t0, mul2(s0, s0));
+  const float2 b1 = fma2(mul2(k, t1), t1, mul2(s1, s1));
+  const float2 b2 = fma2(mul2(k, t2), t2, mul2(s2, s2));
+  float2 f0, f1, f2;
+  if constexpr (MODE == RECON_WENO_JS) {
+    const float2 e = bc2(12e-6f / 13.f);
+    const float2 B0 = add2(b0, e), B1 = add2(b1, e), B2 = add2(b2, e);
+    f0 = rcp2(mul2(B0, B0));
+    f1 = rcp2(mul2(B1, B1));
+    f2 = rcp2(mul2(B2, B2));
+  } else {
+    const float2 e = bc2(12e-20f / 13.f);
+    const float2 d02 = sub2(b0, b2);
+    const float2 tau5 = make_float2(fabsf(d02.x), fabsf(d02.y));
+    f0 = fma2(tau5, rcp2(add2(b0, e)), one);
+    f1 = fma2(tau5, rcp2(add2(b1, e)), one);
+    f2 = fma2(tau5, rcp2(add2(b2, e)), one);
+  }
+  const float2 g0 = mul2(bc2(3.f), f0), g1 = mul2(bc2(6.f), f1), g2 = mul2(bc2(3.f), f2);
+  const float2 nR = fma2(f0, c0, fma2(g1, c1, mul2(g2, z))), SR = add2(add2(f0, g1), g2);
+  const float2 nL = fma2(f2, e0, fma2(g1, e1, mul2(g0, w))), SL = add2(add2(f2, g1), g0);
+  const float2 iL = rcp2(SL);
+  rR = mul2(nR, rcp2(SR));
+  rL = mul2(nL, make_float2(-iL.x, -iL.y));
+}
+
+// WENO5 end values with nonlinear weights (weno5_pair) of two columns at once.
 template <int MODE>
 HGKS_HD void weno5_pair_x2(float2 q0, float2 q1, float2 q2, float2 q3, float2 q4,
                                               float2& qL, float2& qR) {
+  float2 rL, rR;
+  weno5_dev_x2<MODE>(q0, q1, q2, q3, q4, rL, rR);
   const float2 c6 = bc2(1.f / 6.f);
-  const float2 pR0 = mul2(fma2(bc2(2.f), q0, fma2(bc2(-7.f), q1, mul2(bc2(11.f), q2))), c6);
-  const float2 pR1 = mul2(fma2(bc2(-1.f), q1, fma2(bc2(5.f), q2, mul2(bc2(2.f), q3))), c6);
-  const float2 pR2 = mul2(fma2(bc2(2.f), q2, fma2(bc2(5.f), q3, mul2(bc2(-1.f), q4))), c6);
-  const float2 pL0 = mul2(fma2(bc2(2.f), q4, fma2(bc2(-7.f), q3, mul2(bc2(11.f), q2))), c6);
-  const float2 pL1 = mul2(fma2(bc2(-1.f), q3, fma2(bc2(5.f), q2, mul2(bc2(2.f), q1))), c6);
-  const float2 pL2 = mul2(fma2(bc2(2.f), q2, fma2(bc2(5.f), q1, mul2(bc2(-1.f), q0))), c6);
-  const float2 s0 = fma2(bc2(-2.f), q1, add2(q0, q2)), t0 = fma2(bc2(-4.f), q1, fma2(bc2(3.f), q2, q0));
-  const float2 s1 = fma2(bc2(-2.f), q2, add2(q1, q3)), t1 = sub2(q1, q3);
-  const float2 s2 = fma2(bc2(-2.f), q3, add2(q2, q4)), t2 = fma2(bc2(3.f), q2, fma2(bc2(-4.f), q3, q4));
-  const float2 c13 = bc2(13.f / 12.f), qt = bc2(0.25f);
-  const float2 b0 = fma2(mul2(c13, s0), s0, mul2(mul2(qt, t0), t0));
-  const float2 b1 = fma2(mul2(c13, s1), s1, mul2(mul2(qt, t1), t1));
-  const float2 b2 = fma2(mul2(c13, s2), s2, mul2(mul2(qt, t2), t2));
-  float2 f0, f1, f2;  // weight factors of beta0, beta1, beta2
-  if constexpr (MODE == RECON_WENO_JS) {
-    const float2 e = bc2(1e-6f);
-    const float2 e0 = add2(e, b0), e1 = add2(e, b1), e2 = add2(e, b2);
-    f0 = rcp2(mul2(e0, e0));
-    f1 = rcp2(mul2(e1, e1));
-    f2 = rcp2(mul2(e2, e2));
-  } else {
-    const float2 e = bc2(1e-20f);
-    const float2 d02 = sub2(b0, b2);
-    const float2 tau5 = make_float2(fabsf(d02.x), fabsf(d02.y));
-    f0 = fma2(tau5, rcp2(add2(b0, e)), bc2(1.f));
-    f1 = fma2(tau5, rcp2(add2(b1, e)), bc2(1.f));
-    f2 = fma2(tau5, rcp2(add2(b2, e)), bc2(1.f));
-  }
-  {
-    const float2 a0 = mul2(bc2(0.1f), f0), a1 = mul2(bc2(0.6f), f1), a2 = mul2(bc2(0.3f), f2);
-    qR = mul2(fma2(a0, pR0, fma2(a1, pR1, mul2(a2, pR2))), rcp2(add2(add2(a0, a1), a2)));
-  }
-  {
-    const float2 a0 = mul2(bc2(0.1f), f2), a1 = mul2(bc2(0.6f), f1), a2 = mul2(bc2(0.3f), f0);
-    qL = mul2(fma2(a0, pL0, fma2(a1, pL1, mul2(a2, pL2))), rcp2(add2(add2(a0, a1), a2)));
-  }
+  qR = fma2(rR, c6, q2);
+  qL = fma2(rL, c6, q2);
 }
 
 // Tangential reconstruction with nonlinear weights (tangential, WENO modes)
@@ -230,16 +234,15 @@ HGKS_HD void weno5_pair_x2(float2 q0, float2 q1, float2 q2, float2 q3, float2 q4
 template <int MODE>
 HGKS_HD void tangential_weno_x2(float2 f0, float2 f1, float2 f2, float2 f3, float2 f4,
                                                    float2 v[2], float2 d[2]) {
-  float2 qL, qR;
-  weno5_pair_x2<MODE>(f0, f1, f2, f3, f4, qL, qR);
-  const float2 gs = bc2(0.5f / 1.7320508075688772f);
-  const float2 b = sub2(qR, qL);
-  const float2 c = fma2(bc2(3.f), add2(qL, qR), mul2(bc2(-6.f), f2));
-  v[0] = fma2(mul2(b, bc2(-1.f)), gs, f2);
-  v[1] = fma2(b, gs, f2);
-  const float2 c2 = mul2(mul2(bc2(2.f), c), gs);
-  d[0] = sub2(b, c2);
-  d[1] = add2(b, c2);
+  float2 rL, rR;
+  weno5_dev_x2<MODE>(f0, f1, f2, f3, f4, rL, rR);
+  const float gs = 0.5f / 1.7320508075688772f, c6 = 1.f / 6.f;
+  const float2 b = sub2(rR, rL), r = add2(rL, rR);
+  v[0] = fma2(b, bc2(-gs * c6), f2);
+  v[1] = fma2(b, bc2(gs * c6), f2);
+  const float2 cs = mul2(r, bc2(gs)), b6 = mul2(b, bc2(c6));
+  d[0] = sub2(b6, cs);
+  d[1] = add2(b6, cs);
 }
 
 }  // namespace hgks

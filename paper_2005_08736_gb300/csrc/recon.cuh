@@ -12,6 +12,8 @@
 
 #include "physics.cuh"
 
+#include <type_traits>
+
 namespace hgks {
 
 enum Recon { RECON_LINEAR = 0, RECON_WENO_JS = 1, RECON_WENO_Z = 2 };
@@ -23,56 +25,98 @@ enum FluxKind { FLUX_SMOOTH = 0, FLUX_FULL = 1 };
 template <int MODE> __host__ __device__ constexpr int recon_of() { return MODE >= 3 ? MODE - 2 : MODE; }
 template <int MODE> __host__ __device__ constexpr bool is_char_mode() { return MODE >= 3; }
 
-// Both end values of the centre cell: qL at x_{i-1/2}, qR at x_{i+1/2}.
+// Nonlinear WENO5 end values of the centre cell, as six times their
+// deviation from its average: rL = 6 (q(x_{i-1/2}) - q2), rR = 6 (q(x_{i+1/2}) - q2).
 // Candidate quadratics on {i-2,i-1,i}, {i-1,i,i+1}, {i,i+1,i+2} with optimal
 // weights (1/10, 6/10, 3/10) for the right end; the left end uses the mirrored
 // stencils, whose smoothness indicators are the same three in reverse order.
 // WENO-JS: alpha = d/(1e-6 + beta)^2.  WENO-Z: alpha = d (1 + |beta0 - beta2|/(beta + 1e-20)).
+//
+// Everything is formed from the differences D_k = q_k - q_{k-1} and their
+// differences s_k: the candidates' deviations then take one addition each
+// and the indicators three operations (12/13 beta = s^2 + 3/13 t^2, the factor
+// moved into the epsilons), 54 operations per tangential reconstruction
+// against 81 from the averages themselves.  The kernels that call this spend
+// most of their time here and are bound by instruction issue (FP32) or the
+// FP64 pipe.
+// Measured with the flux's primitive form (physics.cuh), GB300: WENO-JS +
+// smooth flux FP32 100x83x77, two steps 2.88 -> 2.42 ms; WENO-Z + full flux
+// FP32 256^3 83.5 -> 71.4 ms a step, FP64 64^3 127 -> 78 ms.
+// FP64: a division costs as much as ten multiplications there, so the
+// weights are multiplied through by the product of the denominators (WENO-Z:
+// B0 B1 B2; WENO-JS: its square), which leaves one (WENO-Z) or two divisions
+// of the five; the products stay in range for |q| up to 1e25 (WENO-Z) and
+// 1e38 (WENO-JS).  FP32's range does not allow the products.
+template <int MODE, class T>
+HGKS_HD void weno5_dev(T q0, T q1, T q2, T q3, T q4, T& rL, T& rR) {
+  static_assert(MODE == RECON_WENO_JS || MODE == RECON_WENO_Z, "nonlinear weights");
+  const T D1 = q1 - q0, D2 = q2 - q1, D3 = q3 - q2, D4 = q4 - q3;
+  const T s0 = D2 - D1, s1 = D3 - D2, s2 = D4 - D3;
+  const T t0 = T(2) * D2 + s0, t1 = D2 + D3, t2 = T(2) * D3 - s2;
+  // candidates: right c0, c1, z (stencils 0, 1, 2); left -e0, -e1, -w (stencils 2, 1, 0)
+  const T w = t0 + D2, z = t2 + D3;
+  const T c0 = w + s0, c1 = t1 + D3, e0 = z - s2, e1 = t1 + D2;
+  const T k = T(3) / T(13);
+  const T b0 = k * t0 * t0 + s0 * s0;
+  const T b1 = k * t1 * t1 + s1 * s1;
+  const T b2 = k * t2 * t2 + s2 * s2;
+  T f0, f1, f2;  // weight factors of beta0, beta1, beta2 (up to a common factor)
+  if (MODE == RECON_WENO_JS) {
+    const T e = T(12e-6 / 13);
+    const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+    if constexpr (std::is_same<T, double>::value) {
+      const T p12 = B1 * B2, p02 = B0 * B2, p01 = B0 * B1;
+      f0 = p12 * p12;
+      f1 = p02 * p02;
+      f2 = p01 * p01;
+    } else {
+      f0 = T(1) / (B0 * B0);
+      f1 = T(1) / (B1 * B1);
+      f2 = T(1) / (B2 * B2);
+    }
+  } else {
+    const T e = T(12e-20 / 13);
+    const T tau5 = tabs(b0 - b2);
+    const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+    if constexpr (std::is_same<T, double>::value) {
+      f0 = (B0 + tau5) * (B1 * B2);
+      f1 = (B1 + tau5) * (B0 * B2);
+      f2 = (B2 + tau5) * (B0 * B1);
+    } else {
+      f0 = tau5 * (T(1) / B0) + T(1);
+      f1 = tau5 * (T(1) / B1) + T(1);
+      f2 = tau5 * (T(1) / B2) + T(1);
+    }
+  }
+  const T g0 = T(3) * f0, g1 = T(6) * f1, g2 = T(3) * f2;
+  const T nR = f0 * c0 + g1 * c1 + g2 * z, SR = f0 + g1 + g2;
+  const T nL = f2 * e0 + g1 * e1 + g0 * w, SL = f2 + g1 + g0;
+  if constexpr (std::is_same<T, double>::value && MODE == RECON_WENO_Z) {
+    const T inv = T(1) / (SR * SL);
+    rR = nR * SL * inv;
+    rL = -(nL * SR * inv);
+  } else {
+    rR = nR * (T(1) / SR);
+    rL = -(nL * (T(1) / SL));
+  }
+}
+
+// Both end values of the centre cell: qL at x_{i-1/2}, qR at x_{i+1/2}.
 template <int MODE_, class T>
 HGKS_HD void weno5_pair(T q0, T q1, T q2, T q3, T q4, T& qL, T& qR) {
   constexpr int MODE = recon_of<MODE_>();
-  if (MODE == RECON_LINEAR) {
+  if constexpr (MODE == RECON_LINEAR) {
     // The optimal-weight combination of the three candidates is the
     // fifth-degree reconstruction (2, -13, 47, 27, -3)/60 of the five averages.
     const T c60 = T(1) / T(60);
     qR = (T(2) * q0 - T(13) * q1 + T(47) * q2 + T(27) * q3 - T(3) * q4) * c60;
     qL = (T(2) * q4 - T(13) * q3 + T(47) * q2 + T(27) * q1 - T(3) * q0) * c60;
-    return;
-  }
-  const T c6 = T(1) / T(6);
-  const T pR0 = (T(2) * q0 - T(7) * q1 + T(11) * q2) * c6;
-  const T pR1 = (-q1 + T(5) * q2 + T(2) * q3) * c6;
-  const T pR2 = (T(2) * q2 + T(5) * q3 - q4) * c6;
-  const T pL0 = (T(2) * q4 - T(7) * q3 + T(11) * q2) * c6;
-  const T pL1 = (-q3 + T(5) * q2 + T(2) * q1) * c6;
-  const T pL2 = (T(2) * q2 + T(5) * q1 - q0) * c6;
-  const T s0 = q0 - T(2) * q1 + q2, t0 = q0 - T(4) * q1 + T(3) * q2;
-  const T s1 = q1 - T(2) * q2 + q3, t1 = q1 - q3;
-  const T s2 = q2 - T(2) * q3 + q4, t2 = T(3) * q2 - T(4) * q3 + q4;
-  const T c13 = T(13) / T(12);
-  const T b0 = c13 * s0 * s0 + T(0.25) * t0 * t0;
-  const T b1 = c13 * s1 * s1 + T(0.25) * t1 * t1;
-  const T b2 = c13 * s2 * s2 + T(0.25) * t2 * t2;
-  T f0, f1, f2;  // weight factors of beta0, beta1, beta2
-  if (MODE == RECON_WENO_JS) {
-    const T e = T(1e-6);
-    f0 = T(1) / ((e + b0) * (e + b0));
-    f1 = T(1) / ((e + b1) * (e + b1));
-    f2 = T(1) / ((e + b2) * (e + b2));
   } else {
-    const T e = T(1e-20);
-    const T tau5 = tabs(b0 - b2);
-    f0 = T(1) + tau5 / (b0 + e);
-    f1 = T(1) + tau5 / (b1 + e);
-    f2 = T(1) + tau5 / (b2 + e);
-  }
-  {
-    const T a0 = T(0.1) * f0, a1 = T(0.6) * f1, a2 = T(0.3) * f2;
-    qR = (a0 * pR0 + a1 * pR1 + a2 * pR2) / (a0 + a1 + a2);
-  }
-  {
-    const T a0 = T(0.1) * f2, a1 = T(0.6) * f1, a2 = T(0.3) * f0;
-    qL = (a0 * pL0 + a1 * pL1 + a2 * pL2) / (a0 + a1 + a2);
+    T rL, rR;
+    weno5_dev<MODE>(q0, q1, q2, q3, q4, rL, rR);
+    const T c6 = T(1) / T(6);
+    qR = rR * c6 + q2;
+    qL = rL * c6 + q2;
   }
 }
 
@@ -89,7 +133,7 @@ template <int MODE_, class T>
 HGKS_HD void tangential(T f0, T f1, T f2, T f3, T f4, T v[2], T d[2]) {
   constexpr int MODE = recon_of<MODE_>();
   const T sq3 = T(1.7320508075688772);
-  if (MODE == RECON_LINEAR) {
+  if constexpr (MODE == RECON_LINEAR) {
     const T E = T(719) / T(720) * f2 + (f1 + f3) * (T(1) / T(1080)) - (f0 + f4) * (T(1) / T(4320));
     const T O = sq3 * (T(7) / T(432) * (f0 - f4) + T(25) / T(216) * (f3 - f1));
     const T A = (f0 - f4) * (T(1) / T(12)) + T(2) / T(3) * (f3 - f1);
@@ -99,15 +143,16 @@ HGKS_HD void tangential(T f0, T f1, T f2, T f3, T f4, T v[2], T d[2]) {
     d[0] = A - B;
     d[1] = A + B;
   } else {
-    T qL, qR;
-    weno5_pair<MODE>(f0, f1, f2, f3, f4, qL, qR);
-    const T gs = T(0.5) / sq3;
-    const T b = qR - qL;
-    const T c = T(3) * (qL + qR) - T(6) * f2;
-    v[0] = f2 - b * gs;
-    v[1] = f2 + b * gs;
-    d[0] = b - T(2) * c * gs;
-    d[1] = b + T(2) * c * gs;
+    // b = (rR - rL)/6, c = (rL + rR)/2
+    T rL, rR;
+    weno5_dev<MODE>(f0, f1, f2, f3, f4, rL, rR);
+    const T b = rR - rL, r = rL + rR;
+    const T gs = T(0.5) / sq3, c6 = T(1) / T(6);
+    v[0] = f2 - b * (gs * c6);
+    v[1] = f2 + b * (gs * c6);
+    const T cs = r * gs;
+    d[0] = b * c6 - cs;
+    d[1] = b * c6 + cs;
   }
 }
 
