@@ -88,18 +88,11 @@ struct PointStateX2 {
   float2 dq[3][5];
 };
 
-// Velocity gradient and pressure derivative of the state along one axis:
-// du[k] = d u_k, dp = d p for the conservative derivative dQ (the pieces the
-// Euler Jacobian-vector product and the viscous flux share).
-struct DirDeriv {
-  float2 du[3], dp;
-};
-
-// Smooth BGK flux at two points (physics.cuh, flux_smooth): F - E(Q_ref)
-// (want_F) and -dF are accumulated into Fs[0..4] and Fs[5..9] summed over the
-// halves: Fs[i] += F_i(.x) + F_i(.y), Fs[5+i] += dF_i(.x) + dF_i(.y).
-// dF = J_n(Q0) Q_t with Q_t = -sum_d J_d(Q0) dQ0/dx_d; F = Euler flux + the
-// BGK Navier-Stokes viscous flux with the heat flux scaled by 1/Pr.
+// Smooth BGK flux at two points (physics.cuh, flux_smooth, through the
+// primitive derivatives and their time derivatives): F - E(Q_ref) (WANT_F)
+// and dF are accumulated into Fs[0..4] and Fs[5..9] summed over the halves:
+// Fs[i] += F_i(.x) + F_i(.y), Fs[5+i] += dF_i(.x) + dF_i(.y).  The time
+// derivatives are formed with the opposite sign (they enter dF linearly).
 template <bool WANT_F>
 __device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas<float>& g, float Fs[10]) {
   // Primitive state (prim_of).
@@ -107,70 +100,65 @@ __device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas
   const float2 inv = rcp2(rho);
   const float2 U[3] = {mul2(st.q[1], inv), mul2(st.q[2], inv), mul2(st.q[3], inv)};
   const float2 nU[3] = {mul2(U[0], bc2(-1.f)), mul2(U[1], bc2(-1.f)), mul2(U[2], bc2(-1.f))};
-  const float2 ke2 = fma2(st.q[1], U[0], fma2(st.q[2], U[1], mul2(st.q[3], U[2])));  // |m|^2/rho
-  const float2 dp = mul2(bc2(g.gm1), fma2(ke2, bc2(-0.5f), st.q[4]));
-  const float2 H = add2(add2(bc2(g.h_r), st.q[4]), dp);
   const float2 hq2 = mul2(bc2(0.5f), fma2(U[0], U[0], fma2(U[1], U[1], mul2(U[2], U[2]))));
-  const float2 m[3] = {mul2(rho, U[0]), mul2(rho, U[1]), mul2(rho, U[2])};
+  const float2 dp = mul2(bc2(g.gm1), fma2(mul2(hq2, bc2(-1.f)), rho, st.q[4]));
+  const float2 p = add2(bc2(g.p_r), dp);
+  const float2 H = add2(add2(bc2(g.h_r), st.q[4]), dp);
 
-  auto deriv = [&](const float2 dQ[5]) {
-    DirDeriv r;
+  // Derivatives along n, t1, t2 (prim_rates).
+  float2 du[3][3], dpd[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) r.du[k] = mul2(fma2(nU[k], dQ[0], dQ[1 + k]), inv);
+  for (int d = 0; d < 3; ++d) {
+    const float2* dQ = st.dq[d];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) du[d][k] = mul2(fma2(nU[k], dQ[0], dQ[1 + k]), inv);
     float2 t = fma2(nU[0], dQ[1], dQ[4]);
     t = fma2(nU[1], dQ[2], t);
     t = fma2(nU[2], dQ[3], t);
     t = fma2(hq2, dQ[0], t);
-    r.dp = mul2(bc2(g.gm1), t);
-    return r;
-  };
-  // J_J(Q) dQ (euler_jvp) from the shared pieces.
-  auto jvp = [&](int J, const float2 dQ[5], const DirDeriv& r, float2 out[5]) {
-    out[0] = dQ[1 + J];
+    dpd[d] = mul2(bc2(g.gm1), t);
+  }
+  const float2 div = add2(add2(du[0][0], du[1][1]), du[2][2]);
+  // minus the time derivatives of density, velocity and pressure
+  const float2 rt = fma2(U[0], st.dq[0][0], fma2(U[1], st.dq[1][0], fma2(U[2], st.dq[2][0], mul2(rho, div))));
+  float2 ut[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) out[1 + i] = fma2(dQ[1 + J], U[i], mul2(m[J], r.du[i]));
-    out[1 + J] = add2(out[1 + J], r.dp);
-    out[4] = fma2(r.du[J], H, mul2(U[J], add2(dQ[4], r.dp)));
-  };
-
-  const DirDeriv r0 = deriv(st.dq[0]), r1 = deriv(st.dq[1]), r2 = deriv(st.dq[2]);
-  // S = sum_d J_d dQ/dx_d = -Q_t.
-  float2 S[5], j[5];
-  jvp(0, st.dq[0], r0, S);
-  jvp(1, st.dq[1], r1, j);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) S[i] = add2(S[i], j[i]);
-  jvp(2, st.dq[2], r2, j);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) S[i] = add2(S[i], j[i]);
-  // dF = J_n Q_t = -J_n S.
-  const DirDeriv rs = deriv(S);
+  for (int i = 0; i < 3; ++i)
+    ut[i] = fma2(U[0], du[0][i], fma2(U[1], du[1][i], fma2(U[2], du[2][i], mul2(dpd[i], inv))));
+  const float2 pt = fma2(U[0], dpd[0], fma2(U[1], dpd[1], fma2(U[2], dpd[2], mul2(mul2(bc2(g.gamma), p), div))));
+  // minus the time derivative of the Euler flux (euler_flux_rate)
+  const float2 m = st.q[1];
+  const float2 mt = fma2(rt, U[0], mul2(rho, ut[0]));
+  const float2 uu = fma2(U[0], ut[0], fma2(U[1], ut[1], mul2(U[2], ut[2])));
+  const float2 Ht = fma2(bc2(g.gamma / g.gm1), pt, fma2(hq2, rt, mul2(rho, uu)));
   float2 dF[5];
-  jvp(0, S, rs, dF);
+  dF[0] = mt;
+  dF[1] = fma2(mt, U[0], fma2(m, ut[0], pt));
+  dF[2] = fma2(mt, U[1], mul2(m, ut[1]));
+  dF[3] = fma2(mt, U[2], mul2(m, ut[2]));
+  dF[4] = fma2(ut[0], H, mul2(U[0], Ht));
 #pragma unroll
   for (int i = 0; i < 5; ++i) Fs[5 + i] -= dF[i].x + dF[i].y;
   if constexpr (WANT_F) {
     // Viscosity mu(T) of the gas law at T = p/rho.
+    const float2 theta = mul2(p, inv);
     float2 mu = bc2(g.mu_ref);
     if (g.visc_law == 1) {
-      const float2 th = mul2(add2(bc2(g.p_r), dp), inv);
-      mu = make_float2(g.mu_ref * tpow(th.x * g.T_ref_inv, g.visc_exp),
-                       g.mu_ref * tpow(th.y * g.T_ref_inv, g.visc_exp));
+      mu = make_float2(g.mu_ref * tpow(theta.x * g.T_ref_inv, g.visc_exp),
+                       g.mu_ref * tpow(theta.y * g.T_ref_inv, g.visc_exp));
     }
     // Viscous stress row of the normal direction and the heat flux
-    // (ns_viscous_flux) from the gradients of the three directions.
-    const float2 theta = mul2(add2(bc2(g.p_r), dp), inv);
-    const float2 divU = add2(add2(r0.du[0], r1.du[1]), r2.du[2]);
-    const float2 dT0 = mul2(fma2(theta, mul2(st.dq[0][0], bc2(-1.f)), r0.dp), inv);
-    const float2 s00 = mul2(mu, fma2(divU, bc2(-2.f / (g.K + 3.f)), mul2(bc2(2.f), r0.du[0])));
-    const float2 s01 = mul2(mu, add2(r0.du[1], r1.du[0]));
-    const float2 s02 = mul2(mu, add2(r0.du[2], r2.du[0]));
+    // (ns_viscous_rates).
+    const float2 dT0 = mul2(fma2(theta, mul2(st.dq[0][0], bc2(-1.f)), dpd[0]), inv);
+    const float2 s00 = mul2(mu, fma2(div, bc2(-2.f / (g.K + 3.f)), mul2(bc2(2.f), du[0][0])));
+    const float2 s01 = mul2(mu, add2(du[0][1], du[1][0]));
+    const float2 s02 = mul2(mu, add2(du[0][2], du[2][0]));
     const float hc = -(g.pr_fix + 1.f) * 0.5f * (g.K + 5.f);
     float2 F[5];
-    F[0] = m[0];
-    F[1] = sub2(fma2(m[0], U[0], dp), s00);
-    F[2] = sub2(mul2(m[0], U[1]), s01);
-    F[3] = sub2(mul2(m[0], U[2]), s02);
+    F[0] = m;
+    F[1] = sub2(fma2(m, U[0], dp), s00);
+    F[2] = sub2(mul2(m, U[1]), s01);
+    F[3] = sub2(mul2(m, U[2]), s02);
     const float2 work = fma2(s00, U[0], fma2(s01, U[1], mul2(s02, U[2])));
     F[4] = fma2(mul2(mu, bc2(hc)), dT0, sub2(mul2(U[0], H), work));
 #pragma unroll
