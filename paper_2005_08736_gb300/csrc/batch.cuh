@@ -1,6 +1,6 @@
 // Batched launches of an ensemble step: ONE grid per phase of the S2O4 step
-// (CFL reduction, dt, ghost fills, transposed copy, the three sweeps and the
-// update of each stage, time) covering every instance of the ensemble.  The
+// (CFL reduction and dt; ghost fill with the transposed copy, the three sweeps
+// and the update of each stage) covering every instance of the ensemble.  The
 // instance table is a kernel parameter (__grid_constant__: it stays in the
 // constant bank, no copy): instance m owns the blocks [start[m], start[m+1])
 // of the grid, and each block runs the same body as the single-instance
@@ -10,6 +10,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "march.cuh"
 #include "sweep.cuh"
 
 namespace hgks {
@@ -48,110 +49,37 @@ __global__ void __launch_bounds__(Job::kThreads, Job::kMinBlocks)
 template <class T>
 struct CflJob {
   static constexpr int kThreads = 256, kMinBlocks = 1;
-  const T* q;
-  GridDev g;
-  const T *wx, *wy, *wz;
-  double rho_r, p_r, gamma;
-  unsigned long long* dtmin;
-  int* flag;
+  CflArgs<T> a;
   int nblocks;
-  __device__ __forceinline__ void run(int b) const {
-    cfl_block(q, g, wx, wy, wz, rho_r, p_r, gamma, dtmin, flag, b, nblocks);
-  }
-};
-
-struct SetDtJob {
-  static constexpr int kThreads = 32, kMinBlocks = 1;
-  double* scal;
-  unsigned long long* dtmin;
-  double cfl, dt_fixed;
-  const int* flag;
-  __device__ __forceinline__ void run(int) const {
-    if (threadIdx.x != 0) return;
-    if (flag && *flag) return;
-    scal[0] = dt_fixed > 0.0 ? dt_fixed : cfl * __longlong_as_double((long long)*dtmin);
-    *dtmin = (unsigned long long)__double_as_longlong(1e300);
-  }
-};
-
-struct AdvanceJob {
-  static constexpr int kThreads = 32, kMinBlocks = 1;
-  double* scal;
-  const int* flag;
-  __device__ __forceinline__ void run(int) const {
-    if (threadIdx.x != 0) return;
-    if (flag && *flag) return;
-    scal[1] += scal[0];
-    scal[2] += 1.0;
-  }
+  __device__ __forceinline__ void run(int b) const { cfl_block(a, b, nblocks); }
 };
 
 template <class T>
-struct GhostXJob {
+struct PadJob {
   static constexpr int kThreads = 256, kMinBlocks = 1;
-  T* q;
-  GridDev g;
-  __device__ __forceinline__ void run(int b) const {
-    ghost_x_cells(q, g, b * (long long)kThreads + threadIdx.x);
-  }
-};
-
-template <class T>
-struct GhostYJob {
-  static constexpr int kThreads = 256, kMinBlocks = 1;
-  T* q;
-  GridDev g;
-  int wall;
-  Gas<T> gas;
-  T T_wall;
-  __device__ __forceinline__ void run(int b) const {
-    ghost_y_cells(q, g, wall, gas, T_wall, b * (long long)kThreads + threadIdx.x);
-  }
-};
-
-template <class T>
-struct GhostZJob {
-  static constexpr int kThreads = 256, kMinBlocks = 1;
-  T* q;
-  GridDev g;
-  __device__ __forceinline__ void run(int b) const {
-    ghost_z_cells(q, g, b * (long long)kThreads + threadIdx.x);
-  }
-};
-
-template <class T>
-struct TransposeJob {
-  static constexpr int kThreads = 256, kMinBlocks = 1;
-  const T* q;
-  T* qx;
-  GridDev g;
+  PadArgs<T> a;
   int gx, gy;
-  __device__ __forceinline__ void run(int b) const {
-#define HGKS_TR_BX (b % gx)
-#define HGKS_TR_BY ((b / gx) % gy)
-#define HGKS_TR_BZ (b / (gx * gy))
-#include "transpose_body.inc"
-#undef HGKS_TR_BX
-#undef HGKS_TR_BY
-#undef HGKS_TR_BZ
-  }
+  __device__ __forceinline__ void run(int b) const { pad_block(a, b % gx, (b / gx) % gy, b / (gx * gy)); }
 };
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL, bool PK>
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
 struct SweepJob {
   static constexpr int kThreads = sweep_threads(TP, TS);
-  static constexpr int kMinBlocks = PK ? 2 : sweep_min_blocks<T, MODE, FLUX, TP, TS>();
-  SweepArgs<T> a;
-  int gx, gy;
+  static constexpr int kMinBlocks = sweep_min_blocks<T, MODE, FLUX, TP, TS>();
+  SweepArgs3<T> a;
   __device__ __forceinline__ void run(int b) const {
-#define HGKS_SW_BX (b % gx)
-#define HGKS_SW_BY ((b / gx) % gy)
-#define HGKS_SW_BZ (b / (gx * gy))
+    const SweepArgs3<T>& sweeps = a;
+#define HGKS_SW_B b
 #include "sweep_body.inc"
-#undef HGKS_SW_BX
-#undef HGKS_SW_BY
-#undef HGKS_SW_BZ
+#undef HGKS_SW_B
   }
+};
+
+template <int STAGE>
+struct MarchJob {
+  static constexpr int kThreads = March::THREADS, kMinBlocks = 1;
+  SweepArgs3<float> a;
+  __device__ __forceinline__ void run(int b) const { march_block<STAGE>(a, b); }
 };
 
 template <class T, int STAGE>

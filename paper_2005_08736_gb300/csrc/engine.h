@@ -37,7 +37,7 @@ struct Engine {
   void* w[3] = {nullptr, nullptr, nullptr};   // cell widths incl. ghosts, n + 6
   double* scal = nullptr;                      // [0] dt, [1] t, [2] step
   unsigned long long* dtmin = nullptr;
-  int* flag = nullptr;
+  int* flag = nullptr;         // [0] non-physical flag, [1] block counter of the CFL reduction
   double* part = nullptr;      // diagnostic partials
   double* diag_out = nullptr;  // 8 doubles
   double* io = nullptr;        // FP64 staging buffer, 5 * N
@@ -59,10 +59,9 @@ struct Engine {
   int diag_blocks = 0;
   int cfl_blocks = 0;
   int sms = 152;  // multiprocessors of the device
-  // Sweep launch choices (set by hgks_autotune): tile variant (0: the default
-  // tile; 1, 2: wider tiles of the linear-weight smooth FP32 sweep; 3: the
-  // 32x8 tile in packed FP32 pairs) and the number of face layers each CTA
-  // marches through (0: automatic).
+  // Sweep launch choices (set by hgks_autotune): the variant of a stored
+  // choice (it no longer selects a kernel) and the length of each CTA's march,
+  // in rows (k_march) or face layers (k_sweep); 0: automatic.
   int sweep_variant = 0;
   int sweep_chunk = 0;
 };
@@ -127,16 +126,18 @@ struct Probe {
 };
 
 // Kernel sequences, implemented per floating type in kernels_f32.cu / kernels_f64.cu.
-template <class T> cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, Probe* probe = nullptr);
+// Ghost cells of qbuf; with `copy` also its copy with x slowest into e.qx.
+template <class T> cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe = nullptr);
 template <class T> cudaError_t enqueue_turbulence(const Engine& e);
 // Append a history record of the state in qbuf (gated: only if the step
 // count is a multiple of e.hist_every and the non-physical flag is clear).
 template <class T> cudaError_t enqueue_history_record(const Engine& e, const void* qbuf, bool gated);
 template <class T> cudaError_t enqueue_channel_rows(const Engine& e);
 template <class T> cudaError_t enqueue_rhs_and_update(const Engine& e, int stage, Probe* probe = nullptr);
-template <class T> cudaError_t enqueue_cfl(const Engine& e, const void* qbuf);
-// The stage-1 sweep of direction d on e.q alone (tuning).
-template <class T> cudaError_t enqueue_sweep_only(const Engine& e, int d);
+// CFL reduction and check of the state in qbuf; with_dt also sets the step's dt.
+template <class T> cudaError_t enqueue_cfl(const Engine& e, const void* qbuf, bool with_dt, double dt_fixed);
+// The stage-1 sweeps on e.q alone (tuning).
+template <class T> cudaError_t enqueue_sweep_only(const Engine& e);
 template <class T> cudaError_t enqueue_diag(const Engine& e);
 template <class T> cudaError_t enqueue_from_fp64(const Engine& e, const double* src, int conservative);
 template <class T> cudaError_t enqueue_to_fp64(const Engine& e, double* dst);
@@ -164,7 +165,6 @@ inline void swap_state_buffers(Engine& e) {
   e.comp2 = t;
 }
 cudaError_t enqueue_set_dt(const Engine& e, double dt_fixed);
-cudaError_t enqueue_advance_time(const Engine& e);
 
 // Empty string if cfg is a valid problem statement, else the reason.
 std::string validate_config(const hgks_config& cfg);

@@ -5,6 +5,7 @@
 #include "engine.h"
 #include "kernels.cuh"
 #include "sweep.cuh"
+#include "march.cuh"
 #include "adjoint.cuh"
 #include "turbulence.cuh"
 #include "batch.cuh"
@@ -55,16 +56,17 @@ inline unsigned blocks_for(long long n, int threads) {
   return unsigned((n + threads - 1) / threads);
 }
 
+// Ghost fill of q; with `copy` also the copy with x slowest for the x sweep.
 template <class T>
-cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, Probe* probe) {
-  T* q = static_cast<T*>(qbuf);
-  const GridDev g = grid_of(e);
-  const int th = 256;
+PadArgs<T> pad_args(const Engine& e, void* q, bool copy) {
+  return {static_cast<T*>(q), copy ? static_cast<T*>(e.qx) : nullptr, grid_of(e),
+          e.cfg.bc_y == HGKS_BC_WALL_ISOTHERMAL ? 1 : 0, gas_of<T>(e.cfg), T(e.cfg.T_wall)};
+}
+
+template <class T>
+cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe) {
   if (probe) probe->begin(e.stream, KC_GHOST);
-  k_ghost_x<T><<<blocks_for(6LL * g.n[1] * g.n[2], th), th, 0, e.stream>>>(q, g);
-  k_ghost_y<T><<<blocks_for(6LL * g.p[0] * g.n[2], th), th, 0, e.stream>>>(
-      q, g, e.cfg.bc_y == HGKS_BC_WALL_ISOTHERMAL, gas_of<T>(e.cfg), T(e.cfg.T_wall));
-  k_ghost_z<T><<<blocks_for(6LL * g.p[0] * g.p[1], th), th, 0, e.stream>>>(q, g);
+  k_pad<T><<<dim3((e.p[0] + 31) / 32, (e.p[1] + 31) / 32, e.p[2]), 256, 0, e.stream>>>(pad_args<T>(e, qbuf, copy));
   if (probe) probe->end(e.stream);
   return cudaGetLastError();
 }
@@ -78,83 +80,108 @@ template <> struct SweepTile<float, FLUX_FULL> { static constexpr int TP = 16, T
 template <> struct SweepTile<double, FLUX_SMOOTH> { static constexpr int TP = 16, TS = 8, NL = 2; };
 template <> struct SweepTile<double, FLUX_FULL> { static constexpr int TP = 8, TS = 8, NL = 2; };
 
-// Arguments and grid (gx, gy, gz) of the sweep of direction d on the padded
-// state q with a TP x TS tile and NL layers per face-field pass.
-template <class T, int TP, int TS, int NL>
-SweepArgs<T> sweep_args(const Engine& e, const T* q, int d, int& gx, int& gy, int& gz) {
-  const GridDev g = grid_of(e);
-  SweepArgs<T> a;
-  // The x sweep reads the copy of the state with x slowest (k_transpose_x).
-  const bool xt = d == 0 && e.qx != nullptr;
-  a.q = xt ? static_cast<const T*>(e.qx) : q;
-  a.xt = xt ? 1 : 0;
-  a.fd = static_cast<T*>(e.fd[d]);
-  a.wn = static_cast<const T*>(e.w[d]);
-  a.wt1 = static_cast<const T*>(e.w[(d + 1) % 3]);
-  a.wt2 = static_cast<const T*>(e.w[(d + 2) % 3]);
-  a.scal = e.scal;
-  a.g = g;
-  a.d = d;
-  a.gas = gas_of<T>(e.cfg);
-  const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
-  gx = (g.n[P] + TP - 1) / TP;
-  gy = (g.n[S] + TS - 1) / TS;
-  // Chunk the march along d so that the grid holds several waves of CTAs.
-  const int layers = g.n[d] + 1;
-  int chunk = e.sweep_chunk;
-  if (chunk <= 0) {
-    const int want_chunks = (4 * e.sms + gx * gy - 1) / (gx * gy);
-    chunk = (layers + want_chunks - 1) / want_chunks;
-    if (chunk < 2 * NL) chunk = 2 * NL;
+// What the three sweeps of a stage on the padded state q share.
+template <class T>
+SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
+  SweepArgs3<T> a;
+  a.q = q;
+  // The x sweep reads the copy of the state with x slowest (k_pad).
+  a.qx = static_cast<const T*>(e.qx);
+  for (int d = 0; d < 3; ++d) {
+    a.fd[d] = static_cast<T*>(e.fd[d]);
+    a.w[d] = static_cast<const T*>(e.w[d]);
+    a.layers[d] = e.n[d] + 1;
   }
-  chunk = (chunk + NL - 1) / NL * NL;
-  a.chunk = chunk;
-  gz = (layers + chunk - 1) / chunk;
+  a.scal = e.scal;
+  a.g = grid_of(e);
+  a.gas = gas_of<T>(e.cfg);
+  a.start[0] = 0;
   return a;
 }
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL, bool PK = false>
-cudaError_t launch_sweep_tile(const Engine& e, const T* q, int d) {
-  const GridDev g = grid_of(e);
-  if (d == 0 && e.qx != nullptr) {
-    const dim3 tgrid((g.p[0] + 31) / 32, (g.p[1] + 31) / 32, g.p[2]);
-    k_transpose_x<T><<<tgrid, 256, 0, e.stream>>>(q, static_cast<T*>(e.qx), g);
+// k_sweep with a TP x TS tile and NL layers per face-field pass.  The march
+// along the normal carries nothing from one pass to the next, so its length
+// only sets the number of CTAs: four per SM, down to one pass each on small
+// grids.
+template <class T, int TP, int TS, int NL>
+SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
+  SweepArgs3<T> a = sweep_common(e, q);
+  int tiles = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
+    a.gx[d] = (e.n[P] + TP - 1) / TP;
+    a.gy[d] = (e.n[S] + TS - 1) / TS;
+    tiles += a.gx[d] * a.gy[d];
   }
-  int gx, gy, gz;
-  const SweepArgs<T> a = sweep_args<T, TP, TS, NL>(e, q, d, gx, gy, gz);
+  for (int d = 0; d < 3; ++d) {
+    int chunk = e.sweep_chunk;
+    if (chunk <= 0) {
+      const int want_chunks = (12 * e.sms + tiles - 1) / tiles;
+      chunk = (a.layers[d] + want_chunks - 1) / want_chunks;
+    }
+    chunk = (chunk + NL - 1) / NL * NL;
+    a.chunk[d] = chunk;
+    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * ((a.layers[d] + chunk - 1) / chunk);
+  }
+  return a;
+}
+
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
+cudaError_t launch_sweep_tile(const Engine& e, const T* q) {
+  const SweepArgs3<T> a = sweep_args<T, TP, TS, NL>(e, q);
   constexpr size_t smem = sweep_smem_bytes<T, MODE, FLUX, TP, TS, NL>();
-  auto kern = k_sweep<T, MODE, FLUX, STAGE, TP, TS, NL, PK>;
+  auto kern = k_sweep<T, MODE, FLUX, STAGE, TP, TS, NL>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<dim3(gx, gy, gz), sweep_threads(TP, TS), smem, e.stream>>>(a);
+  kern<<<a.start[3], sweep_threads(TP, TS), smem, e.stream>>>(a);
   return cudaGetLastError();
 }
 
-// Tile variants: 0 is SweepTile; the linear-weight smooth FP32 sweep also has
-// 32x8 and 16x16 tiles with two layers per face-field pass (1, 2) and the
-// 32x8 tile with the packed FP32-pair last phase (3).
-template <class T, int MODE, int FLUX, int STAGE>
-cudaError_t launch_sweep(const Engine& e, const T* q, int d) {
-  if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
-    if (e.sweep_variant == 1) return launch_sweep_tile<T, MODE, FLUX, STAGE, 32, 8, 2>(e, q, d);
-    if (e.sweep_variant == 2) return launch_sweep_tile<T, MODE, FLUX, STAGE, 16, 16, 2>(e, q, d);
-    if (e.sweep_variant == 3) return launch_sweep_tile<T, MODE, FLUX, STAGE, 32, 8, 2, true>(e, q, d);
-
+// k_march: every block takes the same number of rows of the sequence of all
+// tiles' rows (march_block), so that the blocks, one per SM, finish together;
+// at least two rows, since each stretch repeats four rows of face fields (a
+// quarter of a row's work each).
+inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks) {
+  SweepArgs3<float> a = sweep_common(e, q);
+  for (int d = 0; d < 3; ++d) {
+    // Face n of a periodic direction is face 0.
+    if (d != 1 || e.cfg.bc_y == HGKS_BC_PERIODIC) a.layers[d] = e.n[d];
+    const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
+    a.gx[d] = (e.n[P] + March::TP - 1) / March::TP;
+    a.gy[d] = (a.layers[d] + March::LAYERS - 1) / March::LAYERS;
+    a.chunk[d] = 0;
+    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[S];
   }
-  return launch_sweep_tile<T, MODE, FLUX, STAGE, SweepTile<T, FLUX>::TP, SweepTile<T, FLUX>::TS,
-                           SweepTile<T, FLUX>::NL>(e, q, d);
+  const int rows = a.start[3];
+  a.share = e.sweep_chunk > 0 ? e.sweep_chunk : std::max(2, (rows + e.sms - 1) / e.sms);
+  blocks = (rows + a.share - 1) / a.share;
+  return a;
 }
 
+template <class T, int MODE, int FLUX, int STAGE>
+cudaError_t launch_sweep(const Engine& e, const T* q) {
+  if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
+    int blocks;
+    const SweepArgs3<float> a = march_args(e, q, blocks);
+    const cudaError_t err = cudaFuncSetAttribute(k_march<STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)March::SMEM);
+    if (err != cudaSuccess) return err;
+    k_march<STAGE><<<blocks, March::THREADS, March::SMEM, e.stream>>>(a);
+    return cudaGetLastError();
+  } else {
+    return launch_sweep_tile<T, MODE, FLUX, STAGE, SweepTile<T, FLUX>::TP, SweepTile<T, FLUX>::TS,
+                             SweepTile<T, FLUX>::NL>(e, q);
+  }
+}
+
+// The three sweeps of a stage.
 template <class T, int MODE, int FLUX>
 cudaError_t launch_all_directions(const Engine& e, const T* q, int stage, Probe* probe) {
-  for (int d = 0; d < 3; ++d) {
-    if (probe) probe->begin(e.stream, stage == 1 ? KC_FLUX1 : KC_FLUX2);
-    const cudaError_t err = stage == 1 ? launch_sweep<T, MODE, FLUX, 1>(e, q, d)
-                                       : launch_sweep<T, MODE, FLUX, 2>(e, q, d);
-    if (probe) probe->end(e.stream);
-    if (err != cudaSuccess) return err;
-  }
-  return cudaSuccess;
+  if (probe) probe->begin(e.stream, stage == 1 ? KC_FLUX1 : KC_FLUX2);
+  const cudaError_t err = stage == 1 ? launch_sweep<T, MODE, FLUX, 1>(e, q)
+                                     : launch_sweep<T, MODE, FLUX, 2>(e, q);
+  if (probe) probe->end(e.stream);
+  return err;
 }
 
 // Arguments of the update kernel on the context's current buffers.
@@ -174,6 +201,7 @@ UpdateArgs<T> update_args(const Engine& e) {
   ua.wy = static_cast<const T*>(e.w[1]);
   ua.wz = static_cast<const T*>(e.w[2]);
   ua.scal = e.scal;
+  ua.time = e.scal;
   ua.g = grid_of(e);
   const bool mass_flux = e.cfg.force_mode == HGKS_FORCE_MASS_FLUX;
   ua.force_x = mass_flux ? T(0) : T(e.cfg.force_x);
@@ -184,7 +212,7 @@ UpdateArgs<T> update_args(const Engine& e) {
 template <class T>
 cudaError_t enqueue_rhs_and_update(const Engine& e, int stage, Probe* probe) {
   T* qin = static_cast<T*>(stage == 1 ? e.q : e.qs);
-  cudaError_t err = enqueue_ghosts<T>(e, qin, probe);
+  cudaError_t err = enqueue_ghosts<T>(e, qin, e.qx != nullptr, probe);
   if (err != cudaSuccess) return err;
   const int mode = sweep_mode(e.cfg), flux = e.cfg.flux;
 #define HGKS_DISPATCH(M, F) \
@@ -217,23 +245,30 @@ cudaError_t enqueue_rhs_and_update(const Engine& e, int stage, Probe* probe) {
 }
 
 template <class T>
-cudaError_t enqueue_sweep_only(const Engine& e, int d) {
+cudaError_t enqueue_sweep_only(const Engine& e) {
   const T* q = static_cast<const T*>(e.q);
   const int mode = sweep_mode(e.cfg), flux = e.cfg.flux;
 #define HGKS_SW(M, F) \
-  if (mode == M && flux == F) return launch_sweep<T, M, F, 1>(e, q, d);
+  if (mode == M && flux == F) return launch_sweep<T, M, F, 1>(e, q);
   HGKS_SW(0, 0) HGKS_SW(1, 0) HGKS_SW(2, 0) HGKS_SW(3, 0) HGKS_SW(4, 0)
   HGKS_SW(0, 1) HGKS_SW(1, 1) HGKS_SW(2, 1) HGKS_SW(3, 1) HGKS_SW(4, 1)
 #undef HGKS_SW
   return cudaErrorInvalidValue;
 }
 
+// CFL reduction and check of the state in qbuf; with_dt also sets the step's
+// dt (dt_fixed > 0 overrides the CFL step).
 template <class T>
-cudaError_t enqueue_cfl(const Engine& e, const void* qbuf) {
-  k_cfl<T><<<e.cfl_blocks, 256, 0, e.stream>>>(
-      static_cast<const T*>(qbuf), grid_of(e), static_cast<const T*>(e.w[0]),
-      static_cast<const T*>(e.w[1]), static_cast<const T*>(e.w[2]), e.cfg.rho_ref, e.cfg.p_ref,
-      e.cfg.gamma, e.dtmin, e.flag);
+CflArgs<T> cfl_args(const Engine& e, const void* qbuf, bool with_dt, double dt_fixed) {
+  return {static_cast<const T*>(qbuf), grid_of(e), static_cast<const T*>(e.w[0]),
+          static_cast<const T*>(e.w[1]), static_cast<const T*>(e.w[2]), e.cfg.rho_ref, e.cfg.p_ref,
+          e.cfg.gamma, e.dtmin, e.flag, reinterpret_cast<unsigned*>(e.flag + 1),
+          with_dt ? e.scal : nullptr, e.cfg.cfl, dt_fixed, e.guard ? 1 : 0};
+}
+
+template <class T>
+cudaError_t enqueue_cfl(const Engine& e, const void* qbuf, bool with_dt, double dt_fixed) {
+  k_cfl<T><<<e.cfl_blocks, 256, 0, e.stream>>>(cfl_args<T>(e, qbuf, with_dt, dt_fixed));
   return cudaGetLastError();
 }
 
@@ -391,7 +426,7 @@ cudaError_t enqueue_adjoint_step(const Engine& e, const double* adj_in, double* 
   ea.guard = false;
   cudaError_t err = enqueue_rhs_and_update<T>(ea, 1);
   if (err != cudaSuccess) return err;
-  err = enqueue_ghosts<T>(e, e.qs);
+  err = enqueue_ghosts<T>(e, e.qs, false);
   if (err != cudaSuccess) return err;
   // mu* = (d dL(Q*)/dQ*)^T (dt^2/3 lam).
   err = cudaMemsetAsync(acc, 0, accb, e.stream);
@@ -445,50 +480,26 @@ cudaError_t launch_batched(const std::vector<Job>& jobs, const std::vector<int>&
   return cudaSuccess;
 }
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL, bool PK>
-cudaError_t batched_sweeps(const std::vector<Engine*>& ms, int stage, cudaStream_t s) {
-  for (int d = 0; d < 3; ++d) {
-    if (d == 0) {
-      std::vector<TransposeJob<T>> tj;
-      std::vector<int> tb;
-      for (Engine* e : ms) {
-        if (!e->qx) continue;
-        const GridDev g = grid_of(*e);
-        const int gx = (g.p[0] + 31) / 32, gy = (g.p[1] + 31) / 32;
-        tj.push_back({static_cast<const T*>(stage == 1 ? e->q : e->qs), static_cast<T*>(e->qx), g, gx, gy});
-        tb.push_back(gx * gy * g.p[2]);
-      }
-      const cudaError_t err = launch_batched(tj, tb, 0, s);
-      if (err != cudaSuccess) return err;
-    }
-    using Job = SweepJob<T, MODE, FLUX, STAGE, TP, TS, NL, PK>;
-    std::vector<Job> jobs;
-    std::vector<int> blocks;
-    for (Engine* e : ms) {
-      int gx, gy, gz;
-      Job j;
-      j.a = sweep_args<T, TP, TS, NL>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs), d, gx, gy, gz);
-      j.gx = gx;
-      j.gy = gy;
-      jobs.push_back(j);
-      blocks.push_back(gx * gy * gz);
-    }
-    const cudaError_t err = launch_batched(jobs, blocks, sweep_smem_bytes<T, MODE, FLUX, TP, TS, NL>(), s);
-    if (err != cudaSuccess) return err;
-  }
-  return cudaSuccess;
-}
-
 template <class T, int MODE, int FLUX, int STAGE>
-cudaError_t batched_sweeps_variant(const std::vector<Engine*>& ms, int stage, cudaStream_t s) {
+cudaError_t batched_sweeps(const std::vector<Engine*>& ms, int stage, cudaStream_t s) {
+  std::vector<int> blocks;
   if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
-    const int v = ms[0]->sweep_variant;
-    if (v == 1) return batched_sweeps<T, MODE, FLUX, STAGE, 32, 8, 2, false>(ms, stage, s);
-    if (v == 2) return batched_sweeps<T, MODE, FLUX, STAGE, 16, 16, 2, false>(ms, stage, s);
-    if (v == 3) return batched_sweeps<T, MODE, FLUX, STAGE, 32, 8, 2, true>(ms, stage, s);
+    std::vector<MarchJob<STAGE>> jobs;
+    for (Engine* e : ms) {
+      int nb;
+      jobs.push_back({march_args(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs), nb)});
+      blocks.push_back(nb);
+    }
+    return launch_batched(jobs, blocks, March::SMEM, s);
+  } else {
+    constexpr int TP = SweepTile<T, FLUX>::TP, TS = SweepTile<T, FLUX>::TS, NL = SweepTile<T, FLUX>::NL;
+    std::vector<SweepJob<T, MODE, FLUX, STAGE, TP, TS, NL>> jobs;
+    for (Engine* e : ms) {
+      jobs.push_back({sweep_args<T, TP, TS, NL>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
+      blocks.push_back(jobs.back().a.start[3]);
+    }
+    return launch_batched(jobs, blocks, sweep_smem_bytes<T, MODE, FLUX, TP, TS, NL>(), s);
   }
-  return batched_sweeps<T, MODE, FLUX, STAGE, SweepTile<T, FLUX>::TP, SweepTile<T, FLUX>::TS,
-                        SweepTile<T, FLUX>::NL, false>(ms, stage, s);
 }
 
 template <class T>
@@ -498,46 +509,26 @@ cudaError_t enqueue_batched_step(const std::vector<Engine*>& ms, double dt_fixed
     std::vector<CflJob<T>> jobs;
     std::vector<int> blocks;
     for (Engine* e : ms) {
-      jobs.push_back({static_cast<const T*>(e->q), grid_of(*e), static_cast<const T*>(e->w[0]),
-                      static_cast<const T*>(e->w[1]), static_cast<const T*>(e->w[2]), e->cfg.rho_ref,
-                      e->cfg.p_ref, e->cfg.gamma, e->dtmin, e->flag, e->cfl_blocks});
+      jobs.push_back({cfl_args<T>(*e, e->q, true, dt_fixed), e->cfl_blocks});
       blocks.push_back(e->cfl_blocks);
-    }
-    if ((err = launch_batched(jobs, blocks, 0, s)) != cudaSuccess) return err;
-  }
-  {
-    std::vector<SetDtJob> jobs;
-    std::vector<int> blocks;
-    for (Engine* e : ms) {
-      jobs.push_back({e->scal, e->dtmin, e->cfg.cfl, dt_fixed, e->guard ? e->flag : nullptr});
-      blocks.push_back(1);
     }
     if ((err = launch_batched(jobs, blocks, 0, s)) != cudaSuccess) return err;
   }
   const int mode = sweep_mode(ms[0]->cfg), flux = ms[0]->cfg.flux;
   for (int stage = 1; stage <= 2; ++stage) {
-    std::vector<GhostXJob<T>> gxj;
-    std::vector<GhostYJob<T>> gyj;
-    std::vector<GhostZJob<T>> gzj;
-    std::vector<int> bx, by, bz;
+    std::vector<PadJob<T>> pj;
+    std::vector<int> pb;
     for (Engine* e : ms) {
-      T* q = static_cast<T*>(stage == 1 ? e->q : e->qs);
-      const GridDev g = grid_of(*e);
-      gxj.push_back({q, g});
-      bx.push_back(blocks_for(6LL * g.n[1] * g.n[2], 256));
-      gyj.push_back({q, g, e->cfg.bc_y == HGKS_BC_WALL_ISOTHERMAL ? 1 : 0, gas_of<T>(e->cfg), T(e->cfg.T_wall)});
-      by.push_back(blocks_for(6LL * g.p[0] * g.n[2], 256));
-      gzj.push_back({q, g});
-      bz.push_back(blocks_for(6LL * g.p[0] * g.p[1], 256));
+      const int gx = (e->p[0] + 31) / 32, gy = (e->p[1] + 31) / 32;
+      pj.push_back({pad_args<T>(*e, stage == 1 ? e->q : e->qs, e->qx != nullptr), gx, gy});
+      pb.push_back(gx * gy * e->p[2]);
     }
-    if ((err = launch_batched(gxj, bx, 0, s)) != cudaSuccess) return err;
-    if ((err = launch_batched(gyj, by, 0, s)) != cudaSuccess) return err;
-    if ((err = launch_batched(gzj, bz, 0, s)) != cudaSuccess) return err;
+    if ((err = launch_batched(pj, pb, 0, s)) != cudaSuccess) return err;
     err = cudaErrorInvalidValue;
 #define HGKS_BSW(M, F)                                                                           \
     if (mode == M && flux == F)                                                                  \
-      err = stage == 1 ? batched_sweeps_variant<T, M, F, 1>(ms, stage, s)                        \
-                       : batched_sweeps_variant<T, M, F, 2>(ms, stage, s);
+      err = stage == 1 ? batched_sweeps<T, M, F, 1>(ms, stage, s)                        \
+                       : batched_sweeps<T, M, F, 2>(ms, stage, s);
     HGKS_BSW(0, 0) HGKS_BSW(1, 0) HGKS_BSW(2, 0) HGKS_BSW(3, 0) HGKS_BSW(4, 0)
     HGKS_BSW(0, 1) HGKS_BSW(1, 1) HGKS_BSW(2, 1) HGKS_BSW(3, 1) HGKS_BSW(4, 1)
 #undef HGKS_BSW
@@ -562,20 +553,14 @@ cudaError_t enqueue_batched_step(const std::vector<Engine*>& ms, double dt_fixed
     }
     if (err != cudaSuccess) return err;
   }
-  std::vector<AdvanceJob> aj;
-  std::vector<int> ab;
-  for (Engine* e : ms) {
-    aj.push_back({e->scal, e->guard ? e->flag : nullptr});
-    ab.push_back(1);
-  }
-  return launch_batched(aj, ab, 0, s);
+  return cudaSuccess;
 }
 
 #define HGKS_INSTANTIATE(T)                                                  \
-  template cudaError_t enqueue_ghosts<T>(const Engine&, void*, Probe*);      \
+  template cudaError_t enqueue_ghosts<T>(const Engine&, void*, bool, Probe*); \
   template cudaError_t enqueue_rhs_and_update<T>(const Engine&, int, Probe*); \
-  template cudaError_t enqueue_cfl<T>(const Engine&, const void*);           \
-  template cudaError_t enqueue_sweep_only<T>(const Engine&, int);            \
+  template cudaError_t enqueue_cfl<T>(const Engine&, const void*, bool, double); \
+  template cudaError_t enqueue_sweep_only<T>(const Engine&);                 \
   template cudaError_t enqueue_diag<T>(const Engine&);                       \
   template cudaError_t enqueue_turbulence<T>(const Engine&);                 \
   template cudaError_t enqueue_history_record<T>(const Engine&, const void*, bool); \

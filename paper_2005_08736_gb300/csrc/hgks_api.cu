@@ -125,9 +125,8 @@ cudaError_t enqueue_stage_pair(hgks::Engine& e, double dt_fixed, hgks::Probe* pr
   cudaError_t err;
   const bool f32 = e.cfg.prec == HGKS_FP32;
   if (probe) probe->begin(e.stream, hgks::KC_CFL);
-  err = f32 ? hgks::enqueue_cfl<float>(e, e.q) : hgks::enqueue_cfl<double>(e, e.q);
-  if (err != cudaSuccess) return err;
-  err = hgks::enqueue_set_dt(e, dt_fixed);
+  err = f32 ? hgks::enqueue_cfl<float>(e, e.q, true, dt_fixed)
+            : hgks::enqueue_cfl<double>(e, e.q, true, dt_fixed);
   if (probe) probe->end(e.stream);
   if (err != cudaSuccess) return err;
   for (int stage = 1; stage <= 2; ++stage) {
@@ -135,8 +134,7 @@ cudaError_t enqueue_stage_pair(hgks::Engine& e, double dt_fixed, hgks::Probe* pr
               : hgks::enqueue_rhs_and_update<double>(e, stage, probe);
     if (err != cudaSuccess) return err;
   }
-  err = hgks::enqueue_advance_time(e);
-  if (err != cudaSuccess || e.hist_every <= 0) return err;
+  if (e.hist_every <= 0) return cudaSuccess;
   // Statistics history: a record of Q^{n+1} (in qs) every hist_every steps.
   return f32 ? hgks::enqueue_history_record<float>(e, e.qs, true)
              : hgks::enqueue_history_record<double>(e, e.qs, true);
@@ -184,7 +182,7 @@ static __global__ void k_reset_scalars(double* scal, unsigned long long* dtmin, 
   scal[2] = 0.0;
   scal[3] = 0.0;
   *dtmin = (unsigned long long)__double_as_longlong(1e300);
-  *flag = 0;
+  flag[0] = flag[1] = 0;
 }
 
 static __global__ void k_reset_flag(unsigned long long* dtmin, int* flag) {
@@ -267,10 +265,6 @@ cudaError_t enqueue_set_dt(const Engine& e, double dt_fixed) {
   k_set_dt<<<1, 32, 0, e.stream>>>(e.scal, e.dtmin, e.cfg.cfl, dt_fixed, e.guard ? e.flag : nullptr);
   return cudaGetLastError();
 }
-cudaError_t enqueue_advance_time(const Engine& e) {
-  k_advance_time<<<1, 32, 0, e.stream>>>(e.scal, e.guard ? e.flag : nullptr);
-  return cudaGetLastError();
-}
 
 }  // namespace hgks
 
@@ -346,7 +340,7 @@ hgks_status hgks_create(const hgks_config* cfg, void* stream, hgks_ctx** out) {
   for (int d = 0; d < 3 && err == cudaSuccess; ++d) err = alloc(&e.w[d], (e.n[d] + 6) * es);
   if (err == cudaSuccess) err = alloc((void**)&e.scal, 4 * sizeof(double));
   if (err == cudaSuccess) err = alloc((void**)&e.dtmin, sizeof(unsigned long long));
-  if (err == cudaSuccess) err = alloc((void**)&e.flag, sizeof(int));
+  if (err == cudaSuccess) err = alloc((void**)&e.flag, 2 * sizeof(int));
   if (err == cudaSuccess) err = alloc((void**)&e.part, 8 * sizeof(double) * e.diag_blocks);
   if (err == cudaSuccess) err = alloc((void**)&e.diag_out, 8 * sizeof(double));
   if (err == cudaSuccess) err = alloc((void**)&e.io, 5 * e.N * sizeof(double));
@@ -461,7 +455,7 @@ hgks_status hgks_step(hgks_ctx* c, int nsteps, double dt, int sync, double* t_ou
   // later one from writing, so the state before the first non-physical one
   // is still in one of the two buffers.
   const bool f32 = e.cfg.prec == HGKS_FP32;
-  HGKS_CHECK(c, f32 ? hgks::enqueue_cfl<float>(e, e.q) : hgks::enqueue_cfl<double>(e, e.q));
+  HGKS_CHECK(c, f32 ? hgks::enqueue_cfl<float>(e, e.q, false, 0.0) : hgks::enqueue_cfl<double>(e, e.q, false, 0.0));
   double scal[3];
   int flag = 0;
   HGKS_CHECK(c, cudaMemcpyAsync(scal, e.scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, e.stream));
@@ -1120,7 +1114,7 @@ hgks_status hgks_autotune(hgks_ctx* c, int* variant_out, int* chunk_out, double*
   const bool f32 = e.cfg.prec == HGKS_FP32;
   // The state is not changed: only the stage-1 ghost fill and sweeps run (they
   // write the ghost layers and the face-flux buffers).
-  HGKS_CHECK(c, f32 ? hgks::enqueue_ghosts<float>(e, e.q) : hgks::enqueue_ghosts<double>(e, e.q));
+  HGKS_CHECK(c, f32 ? hgks::enqueue_ghosts<float>(e, e.q, true) : hgks::enqueue_ghosts<double>(e, e.q, true));
   HGKS_CHECK(c, hgks::enqueue_set_dt(e, 1e-3));
   cudaEvent_t t0, t1;
   HGKS_CHECK(c, cudaEventCreate(&t0));
@@ -1128,36 +1122,32 @@ hgks_status hgks_autotune(hgks_ctx* c, int* variant_out, int* chunk_out, double*
   const int nmax = std::max(e.n[0], std::max(e.n[1], e.n[2])) + 1;
   const int chunks[] = {0, 8, 16, 32, 64, 128};
   float best = 1e30f;
-  int best_v = 0, best_c = 0;
+  int best_c = 0;
   cudaError_t err = cudaSuccess;
-  for (int v = 0; v < hgks::sweep_variant_count(e) && err == cudaSuccess; ++v) {
-    for (int ci = 0; ci < 6 && err == cudaSuccess; ++ci) {
-      if (chunks[ci] > 2 * nmax) continue;
-      e.sweep_variant = v;
-      e.sweep_chunk = chunks[ci];
-      float ms = 0.f;
-      for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {  // rep 0 warms up
-        if (rep == 1) err = cudaEventRecord(t0, e.stream);
-        for (int d = 0; d < 3 && err == cudaSuccess; ++d)
-          err = f32 ? hgks::enqueue_sweep_only<float>(e, d) : hgks::enqueue_sweep_only<double>(e, d);
-      }
-      if (err == cudaSuccess) err = cudaEventRecord(t1, e.stream);
-      if (err == cudaSuccess) err = cudaEventSynchronize(t1);
-      if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, t0, t1);
-      if (err == cudaSuccess && ms < best) {
-        best = ms;
-        best_v = v;
-        best_c = chunks[ci];
-      }
+  for (int ci = 0; ci < 6 && err == cudaSuccess; ++ci) {
+    if (chunks[ci] > 2 * nmax) continue;
+    e.sweep_variant = 0;
+    e.sweep_chunk = chunks[ci];
+    float ms = 0.f;
+    for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {  // rep 0 warms up
+      if (rep == 1) err = cudaEventRecord(t0, e.stream);
+      if (err == cudaSuccess) err = f32 ? hgks::enqueue_sweep_only<float>(e) : hgks::enqueue_sweep_only<double>(e);
+    }
+    if (err == cudaSuccess) err = cudaEventRecord(t1, e.stream);
+    if (err == cudaSuccess) err = cudaEventSynchronize(t1);
+    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, t0, t1);
+    if (err == cudaSuccess && ms < best) {
+      best = ms;
+      best_c = chunks[ci];
     }
   }
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
   HGKS_CHECK(c, err);
-  e.sweep_variant = best_v;
+  e.sweep_variant = 0;
   e.sweep_chunk = best_c;
   drop_graphs(c);  // the captured steps hold the old launch shapes
-  if (variant_out) *variant_out = best_v;
+  if (variant_out) *variant_out = 0;
   if (chunk_out) *chunk_out = best_c;
   if (ms_out) *ms_out = best / 2.0;
   return HGKS_OK;
@@ -1210,6 +1200,8 @@ const char* hgks_last_error(const hgks_ctx* c) {
 
 namespace hgks {
 
+// Variants a stored launch shape may name: linear weights + smooth flux in
+// FP32 had four tiles once, all of which run k_march now.
 int sweep_variant_count(const Engine& e) {
   return (e.cfg.prec == HGKS_FP32 && e.cfg.recon == HGKS_RECON_LINEAR &&
           e.cfg.flux == HGKS_FLUX_SMOOTH) ? 4 : 1;

@@ -53,109 +53,99 @@ __host__ __device__ __forceinline__ FaceBox face_box(const GridDev& g, int d, in
 
 // ------------------------------------------------------------- ghost cells ---
 
-// The ghost fills and the CFL reduction are bodies over explicit block
-// coordinates (device functions) with thin __global__ wrappers; the update,
-// the transposed copy and the sweep keep their bodies in the kernels, as
-// included texts (update_body.inc, transpose_body.inc, sweep_body.inc).  The
-// ensemble's batched launches (batch.cuh) run the same bodies for many
-// instances in one grid.
+// The ghost fill and the CFL reduction are bodies over explicit block
+// coordinates (device functions) with thin __global__ wrappers; the update
+// and the sweep keep their bodies in the kernels, as included texts
+// (update_body.inc, sweep_body.inc).  The ensemble's batched launches
+// (batch.cuh) run the same bodies for many instances in one grid.
 
-// x ghosts (periodic) for interior y, z; tid indexes the ghost cells.
+// Ghost cells of the padded state q and, if qx is not null, the copy of the
+// padded state with x slowest, qx[v][x][z][y] (ghosts included), that the x
+// sweep reads like the y and z sweeps read q: consecutive threads along y,
+// the normal axis strided.  x and z are periodic; y is periodic or has the
+// isothermal no-slip walls of Sec. 3.3: the ghost mirrors interior cell m
+// with velocity negated, equal pressure and T_g = 2 T_w - T_m (floored at
+// T_w/2).  Every ghost cell (edges and corners too) is formed from the
+// interior cell it wraps to, so one launch does what separate fills in x, y
+// and z and a transposed copy did in four: blocks read interior cells and
+// write ghost cells only.  One CTA per 32 x 32 tile of a padded x-y plane,
+// block (bx, by, bz) of grid (ceil(p0/32), ceil(p1/32), p2), 256 threads.
+// At 32^3 the launches and their gaps cost more than the copies (two stages,
+// four launches each, were 30 us of a 197 us step); at 256^3 the fused copy
+// moves the same bytes.
 template <class T>
-__device__ __forceinline__ void ghost_x_cells(T* __restrict__ q, const GridDev& g, long long tid) {
-  const long long total = 6LL * g.n[1] * g.n[2];
-  if (tid >= total) return;
-  const int m = int(tid % 6);
-  const long long r = tid / 6;
-  const int y = int(r % g.n[1]), z = int(r / g.n[1]);
-  const int x = m < 3 ? -1 - m : g.n[0] + (m - 3);
-  const int src = m < 3 ? g.n[0] - 1 - m : m - 3;
-  const long long dst = pad_index(g, x, y, z), s = pad_index(g, src, y, z);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) q[v * g.P + dst] = q[v * g.P + s];
-}
-template <class T>
-__global__ void k_ghost_x(T* __restrict__ q, GridDev g) {
-  ghost_x_cells(q, g, blockIdx.x * (long long)blockDim.x + threadIdx.x);
-}
+struct PadArgs {
+  T* q;
+  T* qx;  // or null: ghost cells only
+  GridDev g;
+  int wall;
+  Gas<T> gas;
+  T T_wall;
+};
 
-// y ghosts for all x (ghosts included) and interior z: periodic, or the
-// isothermal no-slip wall (Sec. 3.3): the ghost mirrors interior cell m with
-// velocity negated, equal pressure and T_g = 2 T_w - T_m (floored at T_w/2).
 template <class T>
-__device__ __forceinline__ void ghost_y_cells(T* __restrict__ q, const GridDev& g, int wall,
-                                              const Gas<T>& gas, T T_wall, long long tid) {
-  const long long total = 6LL * g.p[0] * g.n[2];
-  if (tid >= total) return;
-  const int x = int(tid % g.p[0]) - kGhost;
-  const long long r = tid / g.p[0];
-  const int m = int(r % 6), z = int(r / 6);
-  const int y = m < 3 ? -1 - m : g.n[1] + (m - 3);
-  const long long dst = pad_index(g, x, y, z);
-  if (!wall) {
-    const int src = m < 3 ? g.n[1] - 1 - m : m - 3;
-    const long long s = pad_index(g, x, src, z);
+__device__ __forceinline__ void pad_block(const PadArgs<T>& a, int bx, int by, int z) {
+  __shared__ T tile[5][32][33];
+  const GridDev& g = a.g;
+  const int p0 = g.p[0], p1 = g.p[1], p2 = g.p[2];
+  const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
+  const int x0 = bx * 32, y0 = by * 32;
+  const bool zin = z >= kGhost && z < n2 + kGhost;
+  if (!a.qx && zin && x0 >= kGhost && x0 + 32 <= n0 + kGhost && y0 >= kGhost && y0 + 32 <= n1 + kGhost)
+    return;  // interior cells only
+  const int zs = z < kGhost ? z + n2 : (z >= n2 + kGhost ? z - n2 : z);
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const int x = x0 + tx;
+  const int xs = x < kGhost ? x + n0 : (x >= n0 + kGhost ? x - n0 : x);
+  const bool xin = xs == x;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) q[v * g.P + dst] = q[v * g.P + s];
-    return;
+  for (int j = ty; j < 32; j += 8) {
+    const int y = y0 + j;
+    if (x >= p0 || y >= p1) continue;
+    const bool yin = y >= kGhost && y < n1 + kGhost;
+    const bool ghost = !(xin && yin && zin);
+    if (!ghost && !a.qx) continue;
+    int ys = y;
+    if (!yin) ys = a.wall ? (y < kGhost ? 2 * kGhost - 1 - y : 2 * (n1 + kGhost) - 1 - y)
+                          : (y < kGhost ? y + n1 : y - n1);
+    const long long s = ((long long)zs * p1 + ys) * p0 + xs;
+    T v[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] = a.q[k * g.P + s];
+    if (!yin && a.wall) {
+      const Prim<T> st = prim_of(v, a.gas);
+      T Tg = T(2) * a.T_wall - st.theta;
+      if (Tg < T(0.5) * a.T_wall) Tg = T(0.5) * a.T_wall;
+      const T rg = st.p / Tg;
+      const T ke = T(0.5) * rg * (st.U * st.U + st.V * st.V + st.W * st.W);
+      v[0] = rg - a.gas.rho_r;
+      v[1] = -rg * st.U;
+      v[2] = -rg * st.V;
+      v[3] = -rg * st.W;
+      v[4] = st.dp / a.gas.gm1 + ke;
+    }
+    if (ghost) {
+      const long long d = ((long long)z * p1 + y) * p0 + x;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) a.q[k * g.P + d] = v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) tile[k][j][tx] = v[k];
   }
-  const int src = m < 3 ? m : g.n[1] - 1 - (m - 3);
-  const long long s = pad_index(g, x, src, z);
-  T dq[5];
+  if (!a.qx) return;
+  __syncthreads();
+  T* dst = a.qx + (long long)z * p1;
 #pragma unroll
-  for (int v = 0; v < 5; ++v) dq[v] = q[v * g.P + s];
-  const Prim<T> st = prim_of(dq, gas);
-  T Tg = T(2) * T_wall - st.theta;
-  if (Tg < T(0.5) * T_wall) Tg = T(0.5) * T_wall;
-  const T rg = st.p / Tg;
-  const T ke = T(0.5) * rg * (st.U * st.U + st.V * st.V + st.W * st.W);
-  q[0 * g.P + dst] = rg - gas.rho_r;
-  q[1 * g.P + dst] = -rg * st.U;
-  q[2 * g.P + dst] = -rg * st.V;
-  q[3 * g.P + dst] = -rg * st.W;
-  q[4 * g.P + dst] = st.dp / gas.gm1 + ke;
-}
-template <class T>
-__global__ void k_ghost_y(T* __restrict__ q, GridDev g, int wall, Gas<T> gas, T T_wall) {
-  ghost_y_cells(q, g, wall, gas, T_wall, blockIdx.x * (long long)blockDim.x + threadIdx.x);
-}
-
-// z ghosts (periodic) for all x, y including ghosts.
-template <class T>
-__device__ __forceinline__ void ghost_z_cells(T* __restrict__ q, const GridDev& g, long long tid) {
-  const long long plane = (long long)g.p[0] * g.p[1];
-  const long long total = 6LL * plane;
-  if (tid >= total) return;
-  const long long xy = tid % plane;
-  const int m = int(tid / plane);
-  const int z = m < 3 ? -1 - m : g.n[2] + (m - 3);
-  const int src = m < 3 ? g.n[2] - 1 - m : m - 3;
-  const long long dst = (long long)(z + kGhost) * plane + xy;
-  const long long s = (long long)(src + kGhost) * plane + xy;
+  for (int v = 0; v < 5; ++v)
 #pragma unroll
-  for (int v = 0; v < 5; ++v) q[v * g.P + dst] = q[v * g.P + s];
+    for (int j = ty; j < 32; j += 8) {
+      const int xo = x0 + j, y = y0 + tx;
+      if (xo < p0 && y < p1) dst[v * g.P + (long long)xo * p2 * p1 + y] = tile[v][tx][j];
+    }
 }
 template <class T>
-__global__ void k_ghost_z(T* __restrict__ q, GridDev g) {
-  ghost_z_cells(q, g, blockIdx.x * (long long)blockDim.x + threadIdx.x);
-}
-
-// Copy of the padded state with x slowest, qx[v][x][z][y] = q[v][z][y][x]
-// (padded coordinates, ghosts included), so that the x sweep reads its cells
-// like the y and z sweeps read q: consecutive threads along y, the normal
-// axis strided.  One CTA per 32 x 32 tile of an x-y plane, all five
-// variables through shared memory (the 20 loads of a thread are in flight
-// together); grid (ceil(p0/32), ceil(p1/32), p2), 256 threads.
-template <class T>
-__global__ void __launch_bounds__(256) k_transpose_x(const T* __restrict__ q, T* __restrict__ qx,
-                                                     GridDev g) {
-#define HGKS_TR_BX blockIdx.x
-#define HGKS_TR_BY blockIdx.y
-#define HGKS_TR_BZ blockIdx.z
-#include "transpose_body.inc"
-#undef HGKS_TR_BX
-#undef HGKS_TR_BY
-#undef HGKS_TR_BZ
+__global__ void __launch_bounds__(256) k_pad(PadArgs<T> a) {
+  pad_block(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Global conservative-variable index of local-frame component i for sweep
@@ -184,6 +174,8 @@ struct UpdateArgs {
   const T* __restrict__ wy;
   const T* __restrict__ wz;
   const double* __restrict__ scal;
+  double* time;               // stage 2: the scalars, whose time and step count the first
+                              // block advances (nothing in this kernel reads them)
   GridDev g;
   T force_x;
   T rho_r;
@@ -228,20 +220,48 @@ __device__ __forceinline__ double warp_sum(double v) {
 // with a flag for non-physical states (rho <= 0, p <= 0, NaN).  The per-cell
 // arithmetic runs in T; the minimum is combined in FP64: positive doubles
 // order like their bit patterns, so block minima meet in a 64-bit atomicMin.
+// With a.scal set, the last block to finish (a counter at a.ticket) forms the
+// step's dt from the minimum and resets it, which saves the step a launch.
 template <class T>
-__device__ __forceinline__ void cfl_block(const T* __restrict__ q, const GridDev& g,
-                                          const T* __restrict__ wx, const T* __restrict__ wy,
-                                          const T* __restrict__ wz, double rho_r, double p_r,
-                                          double gamma, unsigned long long* __restrict__ dtmin,
-                                          int* __restrict__ flag, int block, int nblocks) {
+struct CflArgs {
+  const T* q;
+  GridDev g;
+  const T *wx, *wy, *wz;
+  double rho_r, p_r, gamma;
+  unsigned long long* dtmin;
+  int* flag;
+  unsigned* ticket;
+  double* scal;  // null: check the state and form the minimum only
+  double cfl, dt_fixed;
+  int guard;     // dt is left as it is once the flag is set
+};
+
+// dt of the step: dt_fixed > 0 overrides the CFL step.  With the
+// non-physical flag set (flag may be null: no guard) the step's scalars are
+// left as they are.  Scalars: [0] dt, [1] t, [2] steps taken.
+__device__ __forceinline__ void set_dt(double* scal, unsigned long long* dtmin, double cfl, double dt_fixed,
+                                       const int* flag) {
+  if (flag && *(volatile const int*)flag) return;
+  scal[0] = dt_fixed > 0.0 ? dt_fixed
+                           : cfl * __longlong_as_double((long long)*(volatile unsigned long long*)dtmin);
+  *dtmin = (unsigned long long)__double_as_longlong(1e300);
+}
+
+template <class T>
+__device__ __forceinline__ void cfl_block(const CflArgs<T>& a, int block, int nblocks) {
+  const GridDev& g = a.g;
+  const T* __restrict__ q = a.q;
   T best = T(1e30);
   int bad = 0;
   const int nx = g.n[0], ny = g.n[1];
-  const T tr = T(rho_r), tp = T(p_r), tg = T(gamma), tg1 = T(gamma - 1.0);
-  // Rows (y, z) of the interior, four per block and pass, x over the threads
-  // (coalesced, no 64-bit division per cell); the loads of the four rows are
-  // issued before any of them is used.
+  const T tr = T(a.rho_r), tp = T(a.p_r), tg = T(a.gamma), tg1 = T(a.gamma - 1.0);
+  // Rows (y, z) of the interior over the blocks, x over W threads (a power of
+  // two, so that short rows leave no thread idle): 4 R rows per block and
+  // pass, the loads of a thread's four rows issued before any is used.
   const int rows = ny * g.n[2];
+  int W = 32;
+  while (W < nx && W < (int)blockDim.x) W *= 2;
+  const int R = blockDim.x / W, tx = threadIdx.x & (W - 1), tr_ = threadIdx.x / W;
   auto cell = [&](T rho, T mx, T my, T mz, T E, int x, int y, int z) {
     const T inv = T(1) / rho;
     const T ke = T(0.5) * (mx * mx + my * my + mz * mz) * inv;
@@ -249,17 +269,17 @@ __device__ __forceinline__ void cfl_block(const T* __restrict__ q, const GridDev
     const bool ok = rho > T(0) && p > T(0);  // false for NaN too
     bad |= !ok;
     const T cs = tsqrt(ok ? tg * p * inv : T(1));
-    T b = fmin(wx[x + kGhost] / (tabs(mx * inv) + cs), wy[y + kGhost] / (tabs(my * inv) + cs));
-    b = fmin(b, wz[z + kGhost] / (tabs(mz * inv) + cs));
+    T b = fmin(a.wx[x + kGhost] / (tabs(mx * inv) + cs), a.wy[y + kGhost] / (tabs(my * inv) + cs));
+    b = fmin(b, a.wz[z + kGhost] / (tabs(mz * inv) + cs));
     if (ok) best = fmin(best, b);
   };
-  for (int row0 = 4 * block; row0 < rows; row0 += 4 * nblocks) {
-    for (int x0 = 0; x0 < nx; x0 += blockDim.x) {
-      const int x = x0 + threadIdx.x;
+  for (int row0 = 4 * R * block; row0 < rows; row0 += 4 * R * nblocks) {
+    for (int x0 = 0; x0 < nx; x0 += W) {
+      const int x = x0 + tx;
       T v[4][5];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int row = row0 + k;
+        const int row = row0 + k * R + tr_;
         if (row < rows && x < nx) {
           const long long pi = pad_index(g, x, row % ny, row / ny);
 #pragma unroll
@@ -268,7 +288,7 @@ __device__ __forceinline__ void cfl_block(const T* __restrict__ q, const GridDev
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int row = row0 + k;
+        const int row = row0 + k * R + tr_;
         if (row < rows && x < nx)
           cell(tr + v[k][0], v[k][1], v[k][2], v[k][3], v[k][4], x, row % ny, row / ny);
       }
@@ -286,35 +306,28 @@ __device__ __forceinline__ void cfl_block(const T* __restrict__ q, const GridDev
     double v = threadIdx.x < (blockDim.x >> 5) ? sm[threadIdx.x] : 1e300;
     v = warp_min(v);
     if (threadIdx.x == 0) {
-      atomicMin(dtmin, (unsigned long long)__double_as_longlong(v));
-      if (sbad) atomicOr(flag, 1);
+      atomicMin(a.dtmin, (unsigned long long)__double_as_longlong(v));
+      if (sbad) atomicOr(a.flag, 1);
+      if (a.scal) {
+        __threadfence();
+        if (atomicAdd(a.ticket, 1u) == unsigned(nblocks - 1)) {
+          __threadfence();
+          *a.ticket = 0;
+          set_dt(a.scal, a.dtmin, a.cfl, a.dt_fixed, a.guard ? a.flag : nullptr);
+        }
+      }
     }
   }
 }
 template <class T>
-__global__ void __launch_bounds__(256) k_cfl(const T* __restrict__ q, GridDev g,
-                                             const T* __restrict__ wx, const T* __restrict__ wy,
-                                             const T* __restrict__ wz, double rho_r, double p_r,
-                                             double gamma, unsigned long long* __restrict__ dtmin,
-                                             int* __restrict__ flag) {
-  cfl_block(q, g, wx, wy, wz, rho_r, p_r, gamma, dtmin, flag, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(256) k_cfl(CflArgs<T> a) {
+  cfl_block(a, blockIdx.x, gridDim.x);
 }
 
-// Scalars: [0] dt, [1] t, [2] steps taken.  dt_fixed > 0 overrides the CFL step.
-// With the non-physical flag set (flag may be null: no guard) the step's
-// scalars are left as they are.
+// dt alone (steps that take no CFL reduction: the adjoint, tuning).
 static __global__ void k_set_dt(double* scal, unsigned long long* dtmin, double cfl, double dt_fixed,
                                 const int* flag) {
-  if (threadIdx.x != 0) return;
-  if (flag && *flag) return;
-  scal[0] = dt_fixed > 0.0 ? dt_fixed : cfl * __longlong_as_double((long long)*dtmin);
-  *dtmin = (unsigned long long)__double_as_longlong(1e300);
-}
-static __global__ void k_advance_time(double* scal, const int* flag) {
-  if (threadIdx.x != 0) return;
-  if (flag && *flag) return;
-  scal[1] += scal[0];
-  scal[2] += 1.0;
+  if (threadIdx.x == 0) set_dt(scal, dtmin, cfl, dt_fixed, flag);
 }
 
 // FP64 partial sums per block: mass, momentum (3), energy, kinetic energy,

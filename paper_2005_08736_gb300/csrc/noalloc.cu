@@ -23,7 +23,7 @@ constexpr size_t kQBytes = align_up(5ull * kMaxP * kMaxP * kMaxP * 8);
 constexpr size_t kIncBytes = align_up(5ull * kMaxN * kMaxN * kMaxN * 8);
 constexpr size_t kFdBytes = align_up(10ull * (kMaxN + 1) * kMaxN * kMaxN * 8);
 constexpr size_t kWBytes = align_up(kMaxP * 8);
-constexpr size_t kScalBytes = align_up(4 * 8 + 8 + 4);
+constexpr size_t kScalBytes = align_up(4 * 8 + 8 + 2 * 4);
 constexpr size_t kScratchBytes =
     2 * kQBytes + 3 * kIncBytes + 3 * kFdBytes + 3 * kWBytes + kScalBytes;  // ~16 MiB
 
@@ -133,12 +133,11 @@ extern "C" hgks_status hgks_step_noalloc(const hgks_config* cfg, double* cons_in
               : hgks::enqueue_from_fp64<double>(e, cons_inout, 1);
   const double dt_fixed = dt > 0.0 ? dt : 0.0;
   for (int n = 0; n < nsteps && err == cudaSuccess; ++n) {
-    err = f32 ? hgks::enqueue_cfl<float>(e, e.q) : hgks::enqueue_cfl<double>(e, e.q);
-    if (err == cudaSuccess) err = hgks::enqueue_set_dt(e, dt_fixed);
+    err = f32 ? hgks::enqueue_cfl<float>(e, e.q, true, dt_fixed)
+              : hgks::enqueue_cfl<double>(e, e.q, true, dt_fixed);
     for (int stage = 1; stage <= 2 && err == cudaSuccess; ++stage)
       err = f32 ? hgks::enqueue_rhs_and_update<float>(e, stage)
                 : hgks::enqueue_rhs_and_update<double>(e, stage);
-    if (err == cudaSuccess) err = hgks::enqueue_advance_time(e);
     hgks::swap_state_buffers(e);  // Q^{n+1} was written into qs
   }
   if (err == cudaSuccess)

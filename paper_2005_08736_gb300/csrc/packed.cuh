@@ -51,7 +51,8 @@ HGKS_HD float2 rcp2(float2 a) { return make_float2(1.f / a.x, 1.f / a.y); }
 // averages) of two columns at once: values v[m] and derivatives d[m] (per
 // unit cell length) at the Gauss abscissae s_m = -+1/(2 sqrt 3):
 //   P(+-g) = E +- O,  P'(+-g) = A +- B  with
-//   E = 719/720 f2 + (f1+f3)/1080 - (f0+f4)/4320,
+//   E = f2 + (-f2/720 + (f1+f3)/1080 - (f0+f4)/4320), in this grouping: a
+//   rounded 719/720 would scale every face value,
 //   O = sqrt3 (7/432 (f0-f4) + 25/216 (f3-f1)),
 //   A = (f0-f4)/12 + 2(f3-f1)/3,  B = sqrt3/54 (13 (f1+f3) - 24 f2 - (f0+f4)).
 HGKS_HD void tangential_linear_x2(float2 f0, float2 f1, float2 f2, float2 f3,
@@ -59,7 +60,7 @@ HGKS_HD void tangential_linear_x2(float2 f0, float2 f1, float2 f2, float2 f3,
   const float sq3 = 1.7320508075688772f;
   const float2 s13 = add2(f1, f3), s04 = add2(f0, f4);
   const float2 d04 = sub2(f0, f4), d31 = sub2(f3, f1);
-  const float2 E = fma2(f2, bc2(719.f / 720.f), fma2(s13, bc2(1.f / 1080.f), mul2(s04, bc2(-1.f / 4320.f))));
+  const float2 E = add2(f2, fma2(f2, bc2(-1.f / 720.f), fma2(s13, bc2(1.f / 1080.f), mul2(s04, bc2(-1.f / 4320.f)))));
   const float2 O = fma2(d04, bc2(sq3 * 7.f / 432.f), mul2(d31, bc2(sq3 * 25.f / 216.f)));
   const float2 A = fma2(d04, bc2(1.f / 12.f), mul2(d31, bc2(2.f / 3.f)));
   const float k = sq3 / 54.f;
@@ -75,7 +76,7 @@ HGKS_HD void tangential_linear_val_x2(float2 f0, float2 f1, float2 f2, float2 f3
   const float sq3 = 1.7320508075688772f;
   const float2 s13 = add2(f1, f3), s04 = add2(f0, f4);
   const float2 d04 = sub2(f0, f4), d31 = sub2(f3, f1);
-  const float2 E = fma2(f2, bc2(719.f / 720.f), fma2(s13, bc2(1.f / 1080.f), mul2(s04, bc2(-1.f / 4320.f))));
+  const float2 E = add2(f2, fma2(f2, bc2(-1.f / 720.f), fma2(s13, bc2(1.f / 1080.f), mul2(s04, bc2(-1.f / 4320.f)))));
   const float2 O = fma2(d04, bc2(sq3 * 7.f / 432.f), mul2(d31, bc2(sq3 * 25.f / 216.f)));
   v[0] = sub2(E, O);
   v[1] = add2(E, O);
@@ -90,11 +91,10 @@ struct PointStateX2 {
 
 // Smooth BGK flux at two points (physics.cuh, flux_smooth, through the
 // primitive derivatives and their time derivatives): F - E(Q_ref) (WANT_F)
-// and dF are accumulated into Fs[0..4] and Fs[5..9] summed over the halves:
-// Fs[i] += F_i(.x) + F_i(.y), Fs[5+i] += dF_i(.x) + dF_i(.y).  The time
-// derivatives are formed with the opposite sign (they enter dF linearly).
+// and dF are added to Fs[0..4] and Fs[5..9].  The time derivatives are formed
+// with the opposite sign (they enter dF linearly).
 template <bool WANT_F>
-__device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas<float>& g, float Fs[10]) {
+__device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas<float>& g, float2 Fs[10]) {
   // Primitive state (prim_of).
   const float2 rho = add2(bc2(g.rho_r), st.q[0]);
   const float2 inv = rcp2(rho);
@@ -138,7 +138,7 @@ __device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas
   dF[3] = fma2(mt, U[2], mul2(m, ut[2]));
   dF[4] = fma2(ut[0], H, mul2(U[0], Ht));
 #pragma unroll
-  for (int i = 0; i < 5; ++i) Fs[5 + i] -= dF[i].x + dF[i].y;
+  for (int i = 0; i < 5; ++i) Fs[5 + i] = sub2(Fs[5 + i], dF[i]);
   if constexpr (WANT_F) {
     // Viscosity mu(T) of the gas law at T = p/rho.
     const float2 theta = mul2(p, inv);
@@ -162,7 +162,7 @@ __device__ __forceinline__ void flux_smooth_x2(const PointStateX2& st, const Gas
     const float2 work = fma2(s00, U[0], fma2(s01, U[1], mul2(s02, U[2])));
     F[4] = fma2(mul2(mu, bc2(hc)), dT0, sub2(mul2(U[0], H), work));
 #pragma unroll
-    for (int i = 0; i < 5; ++i) Fs[i] += F[i].x + F[i].y;
+    for (int i = 0; i < 5; ++i) Fs[i] = add2(Fs[i], F[i]);
   }
 }
 

@@ -29,7 +29,7 @@ namespace hgks {
 
 template <class T>
 struct SweepArgs {
-  const T* __restrict__ q;     // padded state (deviation)
+  const T* q;                  // padded state (deviation)
   T* __restrict__ fd;          // face fluxes [10][fbox]: F then dF, global frame
   const T* __restrict__ wn;    // widths along d (offset kGhost)
   const T* __restrict__ wt1;   // widths along t1
@@ -38,9 +38,59 @@ struct SweepArgs {
   GridDev g;
   int d;
   int chunk;
-  int xt;  // d = x and q is the copy with x slowest ([5][x][z][y], k_transpose_x)
+  int xt;  // d = x and q is the copy with x slowest ([5][x][z][y], k_pad)
   Gas<T> gas;
 };
+
+// The three sweeps of a stage in one launch: block b belongs to direction d
+// with start[d] <= b < start[d + 1].  The sweeps are independent of each
+// other, so one grid fills the chip on grids where one direction cannot
+// (32^3: 24 tiles a direction) and has one tail instead of three.
+template <class T>
+struct SweepArgs3 {
+  const T* q;          // padded state
+  const T* qx;         // its copy with x slowest (or null: the x sweep reads q)
+  T* fd[3];
+  const T* w[3];
+  const double* scal;
+  GridDev g;
+  int gx[3], gy[3], chunk[3], start[4];
+  int share;           // k_march: rows per block (start counts rows)
+  int layers[3];       // face layers to compute: n + 1, or n where face n is face 0 (k_march)
+  Gas<T> gas;
+};
+
+// Arguments of direction d.
+template <class T>
+__device__ __forceinline__ SweepArgs<T> sweep_of(const SweepArgs3<T>& s, int d) {
+  auto pick = [&](auto x0, auto x1, auto x2) { return d == 0 ? x0 : (d == 1 ? x1 : x2); };
+  SweepArgs<T> a;
+  a.d = d;
+  a.xt = d == 0 && s.qx != nullptr;
+  a.q = a.xt ? s.qx : s.q;
+  a.fd = pick(s.fd[0], s.fd[1], s.fd[2]);
+  a.wn = pick(s.w[0], s.w[1], s.w[2]);
+  a.wt1 = pick(s.w[1], s.w[2], s.w[0]);
+  a.wt2 = pick(s.w[2], s.w[0], s.w[1]);
+  a.scal = s.scal;
+  a.g = s.g;
+  a.chunk = pick(s.chunk[0], s.chunk[1], s.chunk[2]);
+  a.gas = s.gas;
+  return a;
+}
+
+// Direction and block coordinates of block b, and its direction's arguments.
+template <class T>
+__device__ __forceinline__ SweepArgs<T> sweep_of_block(const SweepArgs3<T>& s, int b, int& bx, int& by, int& bz) {
+  const int d = b >= s.start[2] ? 2 : (b >= s.start[1] ? 1 : 0);
+  auto pick = [&](int x0, int x1, int x2) { return d == 0 ? x0 : (d == 1 ? x1 : x2); };
+  const int gx = pick(s.gx[0], s.gx[1], s.gx[2]), gy = pick(s.gy[0], s.gy[1], s.gy[2]);
+  const int r = b - pick(0, s.start[1], s.start[2]);
+  bx = r % gx;
+  by = (r / gx) % gy;
+  bz = r / (gx * gy);
+  return sweep_of(s, d);
+}
 
 template <int FLUX, int MODE = 0>
 struct SweepLayout {
@@ -491,35 +541,6 @@ __device__ __forceinline__ void t1_pass_group_wx2(const float* ff, float* tb, in
   }
 }
 
-// t1_pass_group with the packed layout of the last phase (FP32, linear
-// weights): the outputs at the two t1 abscissae are stored side by side as a
-// float2 -- state field k: pair plane 2k (values), 2k+1 (t1-derivatives);
-// normal slope of state field j: pair plane 2 NV + j (values).
-template <int MODE, int NV, int NH>
-__device__ __forceinline__ void t1_pass_group_x2(const float* ff, float* tb, int at, int st1, int grp) {
-  float2* tb2 = reinterpret_cast<float2*>(tb);
-  if (grp < NV / 5) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      const int k = 5 * grp + i;
-      const float* src = ff + k * NH + at;
-      float v[2], dd[2];
-      tangential<MODE>(src[-2 * st1], src[-st1], src[0], src[st1], src[2 * st1], v, dd);
-      tb2[(2 * k) * NH + at] = make_float2(v[0], v[1]);
-      tb2[(2 * k + 1) * NH + at] = make_float2(dd[0], dd[1]);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      const int j = 5 * (grp - NV / 5) + i;
-      const float* src = ff + (NV + j) * NH + at;
-      float v[2];
-      tangential_val<MODE>(src[-2 * st1], src[-st1], src[0], src[st1], src[2 * st1], v);
-      tb2[(2 * NV + j) * NH + at] = make_float2(v[0], v[1]);
-    }
-  }
-}
-
 // Resident CTAs per SM the register budget is sized for: the smooth FP32
 // sweep fits three (shared memory allows three as well), the others one or two
 // (two at most for the characteristic modes, which need more registers).
@@ -538,20 +559,12 @@ __host__ __device__ constexpr int sweep_min_blocks() {
                                                                       : SweepOccupancy<T, FLUX>::value;
 }
 
-// PK (FP32, linear weights, smooth flux, one thread per face): the last
-// phase evaluates the two t1 abscissae of a face as the halves of packed FP32
-// pairs (packed.cuh); shared memory allows two CTAs per SM for this tile, so
-// the register budget is sized for two.
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL, bool PK = false>
-__global__ void __launch_bounds__(sweep_threads(TP, TS), (PK ? 2 : sweep_min_blocks<T, MODE, FLUX, TP, TS>()))
-    k_sweep(SweepArgs<T> a) {
-#define HGKS_SW_BX blockIdx.x
-#define HGKS_SW_BY blockIdx.y
-#define HGKS_SW_BZ blockIdx.z
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
+__global__ void __launch_bounds__(sweep_threads(TP, TS), (sweep_min_blocks<T, MODE, FLUX, TP, TS>()))
+    k_sweep(const __grid_constant__ SweepArgs3<T> sweeps) {
+#define HGKS_SW_B blockIdx.x
 #include "sweep_body.inc"
-#undef HGKS_SW_BX
-#undef HGKS_SW_BY
-#undef HGKS_SW_BZ
+#undef HGKS_SW_B
 }
 
 }  // namespace hgks
