@@ -11,7 +11,7 @@
 
 #include "kernels.cuh"
 #include "march.cuh"
-#include "sweep.cuh"
+#include "sweep_full.cuh"
 
 namespace hgks {
 
@@ -62,10 +62,10 @@ struct PadJob {
   __device__ __forceinline__ void run(int b) const { pad_block(a, b % gx, (b / gx) % gy, b / (gx * gy)); }
 };
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
+template <class T, int MODE, int STAGE, int TP, int TS, int NL>
 struct SweepJob {
   static constexpr int kThreads = sweep_threads(TP, TS);
-  static constexpr int kMinBlocks = sweep_min_blocks<T, MODE, FLUX, TP, TS>();
+  static constexpr int kMinBlocks = sweep_min_blocks<T, MODE>();
   SweepArgs3<T> a;
   __device__ __forceinline__ void run(int b) const {
     const SweepArgs3<T>& sweeps = a;
@@ -73,6 +73,14 @@ struct SweepJob {
 #include "sweep_body.inc"
 #undef HGKS_SW_B
   }
+};
+
+template <class T, int MODE, int STAGE, int TP, int TS>
+struct SweepFullJob {
+  static constexpr int kThreads = FullSweep<T, MODE, TP, TS>::THREADS;
+  static constexpr int kMinBlocks = FullSweep<T, MODE, TP, TS>::MIN_BLOCKS;
+  SweepArgs3<T> a;
+  __device__ __forceinline__ void run(int b) const { sweep_full_block<T, MODE, STAGE, TP, TS>(a, b); }
 };
 
 template <int STAGE>

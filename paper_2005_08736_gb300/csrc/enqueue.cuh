@@ -6,6 +6,7 @@
 #include "kernels.cuh"
 #include "sweep.cuh"
 #include "march.cuh"
+#include "sweep_full.cuh"
 #include "adjoint.cuh"
 #include "turbulence.cuh"
 #include "batch.cuh"
@@ -71,14 +72,11 @@ cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe)
   return cudaGetLastError();
 }
 
-// Tile of the sweep kernel per precision and flux: TP x TS faces, sized so
-// that the shared-memory staging fits and every tile gives 1, 2 or 4 threads
-// per face.
-// NL face layers share one face-field pass (phase 1).
-template <class T, int FLUX> struct SweepTile { static constexpr int TP = 16, TS = 8, NL = 4; };
-template <> struct SweepTile<float, FLUX_FULL> { static constexpr int TP = 16, TS = 8, NL = 2; };
-template <> struct SweepTile<double, FLUX_SMOOTH> { static constexpr int TP = 16, TS = 8, NL = 2; };
-template <> struct SweepTile<double, FLUX_FULL> { static constexpr int TP = 8, TS = 8, NL = 2; };
+// Tiles of the sweep kernels: TP x TS faces, sized so that the shared-memory
+// staging fits; NL face layers share one face-field pass (phase 1) of the
+// smooth flux.
+template <class T> struct SweepTile { static constexpr int TP = 16, TS = 8, NL = sizeof(T) == 4 ? 4 : 2; };
+template <class T> struct FullTile { static constexpr int TP = 16, TS = 8; };
 
 // What the three sweeps of a stage on the padded state q share.
 template <class T>
@@ -90,7 +88,8 @@ SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
   for (int d = 0; d < 3; ++d) {
     a.fd[d] = static_cast<T*>(e.fd[d]);
     a.w[d] = static_cast<const T*>(e.w[d]);
-    a.layers[d] = e.n[d] + 1;
+    // Face n of a periodic direction is face 0.
+    a.layers[d] = e.n[d] + (d == 1 && e.cfg.bc_y != HGKS_BC_PERIODIC ? 1 : 0);
   }
   a.scal = e.scal;
   a.g = grid_of(e);
@@ -126,11 +125,11 @@ SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   return a;
 }
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
+template <class T, int MODE, int STAGE, int TP, int TS, int NL>
 cudaError_t launch_sweep_tile(const Engine& e, const T* q) {
   const SweepArgs3<T> a = sweep_args<T, TP, TS, NL>(e, q);
-  constexpr size_t smem = sweep_smem_bytes<T, MODE, FLUX, TP, TS, NL>();
-  auto kern = k_sweep<T, MODE, FLUX, STAGE, TP, TS, NL>;
+  constexpr size_t smem = sweep_smem_bytes<T, MODE, TP, TS, NL>();
+  auto kern = k_sweep<T, MODE, STAGE, TP, TS, NL>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   kern<<<a.start[3], sweep_threads(TP, TS), smem, e.stream>>>(a);
@@ -144,8 +143,6 @@ cudaError_t launch_sweep_tile(const Engine& e, const T* q) {
 inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks) {
   SweepArgs3<float> a = sweep_common(e, q);
   for (int d = 0; d < 3; ++d) {
-    // Face n of a periodic direction is face 0.
-    if (d != 1 || e.cfg.bc_y == HGKS_BC_PERIODIC) a.layers[d] = e.n[d];
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
     a.gx[d] = (e.n[P] + March::TP - 1) / March::TP;
     a.gy[d] = (a.layers[d] + March::LAYERS - 1) / March::LAYERS;
@@ -158,6 +155,17 @@ inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks
   return a;
 }
 
+template <class T, int MODE, int STAGE, int TP, int TS>
+cudaError_t launch_sweep_full(const Engine& e, const T* q) {
+  using L = FullSweep<T, MODE, TP, TS>;
+  const SweepArgs3<T> a = sweep_args<T, TP, TS, 1>(e, q);
+  auto kern = k_sweep_full<T, MODE, STAGE, TP, TS>;
+  const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM);
+  if (err != cudaSuccess) return err;
+  kern<<<a.start[3], L::THREADS, L::SMEM, e.stream>>>(a);
+  return cudaGetLastError();
+}
+
 template <class T, int MODE, int FLUX, int STAGE>
 cudaError_t launch_sweep(const Engine& e, const T* q) {
   if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
@@ -168,9 +176,10 @@ cudaError_t launch_sweep(const Engine& e, const T* q) {
     if (err != cudaSuccess) return err;
     k_march<STAGE><<<blocks, March::THREADS, March::SMEM, e.stream>>>(a);
     return cudaGetLastError();
+  } else if constexpr (FLUX == FLUX_FULL) {
+    return launch_sweep_full<T, MODE, STAGE, FullTile<T>::TP, FullTile<T>::TS>(e, q);
   } else {
-    return launch_sweep_tile<T, MODE, FLUX, STAGE, SweepTile<T, FLUX>::TP, SweepTile<T, FLUX>::TS,
-                             SweepTile<T, FLUX>::NL>(e, q);
+    return launch_sweep_tile<T, MODE, STAGE, SweepTile<T>::TP, SweepTile<T>::TS, SweepTile<T>::NL>(e, q);
   }
 }
 
@@ -491,14 +500,22 @@ cudaError_t batched_sweeps(const std::vector<Engine*>& ms, int stage, cudaStream
       blocks.push_back(nb);
     }
     return launch_batched(jobs, blocks, March::SMEM, s);
+  } else if constexpr (FLUX == FLUX_FULL) {
+    constexpr int TP = FullTile<T>::TP, TS = FullTile<T>::TS;
+    std::vector<SweepFullJob<T, MODE, STAGE, TP, TS>> jobs;
+    for (Engine* e : ms) {
+      jobs.push_back({sweep_args<T, TP, TS, 1>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
+      blocks.push_back(jobs.back().a.start[3]);
+    }
+    return launch_batched(jobs, blocks, FullSweep<T, MODE, TP, TS>::SMEM, s);
   } else {
-    constexpr int TP = SweepTile<T, FLUX>::TP, TS = SweepTile<T, FLUX>::TS, NL = SweepTile<T, FLUX>::NL;
-    std::vector<SweepJob<T, MODE, FLUX, STAGE, TP, TS, NL>> jobs;
+    constexpr int TP = SweepTile<T>::TP, TS = SweepTile<T>::TS, NL = SweepTile<T>::NL;
+    std::vector<SweepJob<T, MODE, STAGE, TP, TS, NL>> jobs;
     for (Engine* e : ms) {
       jobs.push_back({sweep_args<T, TP, TS, NL>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
       blocks.push_back(jobs.back().a.start[3]);
     }
-    return launch_batched(jobs, blocks, sweep_smem_bytes<T, MODE, FLUX, TP, TS, NL>(), s);
+    return launch_batched(jobs, blocks, sweep_smem_bytes<T, MODE, TP, TS, NL>(), s);
   }
 }
 

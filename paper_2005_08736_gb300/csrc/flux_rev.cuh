@@ -338,7 +338,7 @@ HGKS_HD void euler_jvp_rev_dq(const Prim<T>& s, T H, const Gas<T>& g, const T ob
 // Cotangents of the values q and slopes dq of the state of flux_full_side
 // (side 0: u > 0, side 1: u < 0) as it enters the full flux through the
 // fit weights w_k = Fq[k] (F) and dFq[k] (dF) of its three moment vectors V_k
-// (flux_full_combine), given the flux cotangents gF, gdF; added to cot.  The
+// (flux_full_close), given the flux cotangents gF, gdF; added to cot.  The
 // weights are dual numbers carrying d/dtau; returns the part's share of
 // gF . dF/dtau + gdF . d(dF)/dtau.  The cotangent of its pressure (through
 // tau) is applied by pressure_viscosity_rev.  The four moment matrices are
@@ -680,7 +680,7 @@ HGKS_HD void flux_smooth_rev(const PointState<T>& st0, const Gas<T>& g, bool wan
 }
 
 // Cotangents of the values q and slopes dq of the equilibrium state of
-// flux_full_eq as it enters the full flux (flux_full_combine): its three
+// flux_full_eq as it enters the full flux (flux_full_close): its three
 // moment vectors V_k with the fit weights Fq[k] (F) and dFq[k] (dF), dual
 // numbers carrying d/dtau, and the Prandtl fix -wpr tau p0 dT0 of F[4]
 // (wpr = gF[4] pr_fix c_p), given the flux cotangents gF, gdF and the

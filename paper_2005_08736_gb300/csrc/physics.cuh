@@ -603,9 +603,15 @@ HGKS_HD void flux_full_side(const PointState<T>& st, const Gas<T>& g, int side,
   o.p = s.p;
 }
 
+// |p_l - p_r| / (p_l + p_r)
+template <class T>
+HGKS_HD T pressure_jump(T pl, T pr) {
+  return tabs((pl - pr) / (pl + pr));
+}
+
 template <class T>
 HGKS_HD T collision_time_full(T mu0, T p0, T pl, T pr, const Gas<T>& g, T dt) {
-  return mu0 / p0 + g.tau_num_C * tabs((pl - pr) / (pl + pr)) * dt;
+  return mu0 / p0 + g.tau_num_C * pressure_jump(pl, pr) * dt;
 }
 
 // The parts of the full flux gathered for one Gauss point: the equilibrium
@@ -631,21 +637,11 @@ HGKS_HD void flux_full_add_side(const PointState<T>& st, const Gas<T>& g, int si
   if (side == 0) a.pl = h.p; else a.pr = h.p;
 }
 
-// The full flux from its parts: tau, the fit of Eq. (7), the Prandtl fix.
+// The full flux from its equilibrium part, the sums Vs of the half-space
+// parts and the pressure jump: tau, the fit of Eq. (7), the Prandtl fix.
 template <class T>
-HGKS_HD void flux_full_combine(const FullParts<T>& a, const Gas<T>& g, T dt, T F[5], T dF[5]) {
-  const FullEq<T>& e = a.e;
-  T V[6][5];
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      V[k][i] = e.V[k][i];
-      V[3 + k][i] = a.Vs[k][i];
-    }
-  const T pl = a.pl, pr = a.pr;
-  V[3][1] -= g.p_r;  // the half-space sum minus the reference Euler flux
-  const T tau = collision_time_full(e.mu, e.p, pl, pr, g, dt);
+HGKS_HD void flux_full_close(const FullEq<T>& e, const T Vs[3][5], T jump, const Gas<T>& g, T dt, T F[5], T dF[5]) {
+  const T tau = e.mu / e.p + g.tau_num_C * jump * dt;
   T Fq[6], dFq[6];
   fit_coefficients(tau, dt, Fq, dFq);
 #pragma unroll
@@ -653,8 +649,10 @@ HGKS_HD void flux_full_combine(const FullParts<T>& a, const Gas<T>& g, T dt, T F
     T f = T(0), df = T(0);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      f += Fq[k] * V[k][i];
-      df += dFq[k] * V[k][i];
+      // the half-space sum minus the reference Euler flux
+      const T v = k < 3 ? e.V[k][i] : (k == 3 && i == 1 ? Vs[0][1] - g.p_r : Vs[k - 3][i]);
+      f += Fq[k] * v;
+      df += dFq[k] * v;
     }
     F[i] = f;
     dF[i] = df;
@@ -675,7 +673,7 @@ HGKS_HD void flux_full(const PointState<T>& stl, const PointState<T>& str,
   flux_full_eq(st0, g, a.e);
 #pragma unroll 1  // one copy of the half-space code for both sides
   for (int side = 0; side < 2; ++side) flux_full_add_side(side == 0 ? stl : str, g, side, a);
-  flux_full_combine(a, g, dt, F, dF);
+  flux_full_close(a.e, a.Vs, pressure_jump(a.pl, a.pr), g, dt, F, dF);
 }
 
 // Equilibrium state of the compatibility condition, Q0 = int_{u>0} psi g_l +

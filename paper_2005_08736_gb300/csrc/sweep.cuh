@@ -1,6 +1,8 @@
-// Fused sweep kernel: for one direction d and one S2O4 stage, the face
-// fields, the tangential reconstruction to the 2x2 Gauss points and the BGK
-// flux there, for a 2D tile of faces marching along the normal.
+// Fused sweep kernel of the smooth flux: for one direction d and one S2O4
+// stage, the face fields, the tangential reconstruction to the 2x2 Gauss
+// points and the BGK flux there, for a 2D tile of faces marching along the
+// normal.  (FP32 with linear weights: march.cuh; the full flux:
+// sweep_full.cuh, with the pieces it shares here.)
 //
 // Tile: TP x TS faces in the transverse plane, P = the faster-varying
 // transverse axis in memory, S = the slower one; the CTA marches through a
@@ -38,6 +40,7 @@ struct SweepArgs {
   GridDev g;
   int d;
   int chunk;
+  int layers;
   int xt;  // d = x and q is the copy with x slowest ([5][x][z][y], k_pad)
   Gas<T> gas;
 };
@@ -56,7 +59,7 @@ struct SweepArgs3 {
   GridDev g;
   int gx[3], gy[3], chunk[3], start[4];
   int share;           // k_march: rows per block (start counts rows)
-  int layers[3];       // face layers to compute: n + 1, or n where face n is face 0 (k_march)
+  int layers[3];       // face layers to compute: n + 1, or n where face n is face 0
   Gas<T> gas;
 };
 
@@ -75,6 +78,7 @@ __device__ __forceinline__ SweepArgs<T> sweep_of(const SweepArgs3<T>& s, int d) 
   a.scal = s.scal;
   a.g = s.g;
   a.chunk = pick(s.chunk[0], s.chunk[1], s.chunk[2]);
+  a.layers = pick(s.layers[0], s.layers[1], s.layers[2]);
   a.gas = s.gas;
   return a;
 }
@@ -103,19 +107,13 @@ struct SweepLayout {
 // Threads of a sweep CTA: 256, or one per face for tiles of more faces.
 __host__ __device__ constexpr int sweep_threads(int tp, int ts) { return tp * ts > 256 ? tp * ts : 256; }
 
-// Per-thread slots of the full-flux phase 3 with two threads per face: the
-// three point states (20 values each) of the second t2 abscissa.
-template <int FLUX, int TPF>
-constexpr int sweep_scratch_elems() {
-  return FLUX == FLUX_FULL && TPF == 2 ? 60 * 256 : 0;
-}
-
-template <class T, int MODE, int FLUX, int TP, int TS, int NL>
+template <class T, int MODE, int TP, int TS, int NL>
 constexpr size_t sweep_smem_bytes() {
+  constexpr int FLUX = FLUX_SMOOTH;
   constexpr int NH = (TP + 4) * (TS + 4);
   constexpr int TPF = sweep_threads(TP, TS) / (TP * TS);
   return sizeof(T) * ((NL * SweepLayout<FLUX, MODE>::NFF + SweepLayout<FLUX, MODE>::NT1) * NH +
-                      (TPF - 1) * 10 * TP * TS + sweep_scratch_elems<FLUX, TPF>());
+                      (TPF - 1) * 10 * TP * TS);
 }
 
 // Tangential reconstruction of a 5-vector field (components at src + i*sc,
@@ -541,26 +539,15 @@ __device__ __forceinline__ void t1_pass_group_wx2(const float* ff, float* tb, in
   }
 }
 
-// Resident CTAs per SM the register budget is sized for: the smooth FP32
-// sweep fits three (shared memory allows three as well), the others one or two
-// (two at most for the characteristic modes, which need more registers).
-template <class T, int FLUX> struct SweepOccupancy { static constexpr int value = 1; };
-template <> struct SweepOccupancy<float, FLUX_SMOOTH> { static constexpr int value = 3; };
-template <> struct SweepOccupancy<double, FLUX_SMOOTH> { static constexpr int value = 2; };
-
-// Resident CTAs per SM for the register budget: SweepOccupancy for 256
-// threads (two at most in the characteristic modes); tiles of 384 threads
-// two, of 512 one.
-template <class T, int MODE, int FLUX, int TP, int TS>
+// Resident CTAs per SM the register budget is sized for: three in FP32 (two
+// in the characteristic modes, which need more registers), two in FP64.
+template <class T, int MODE>
 __host__ __device__ constexpr int sweep_min_blocks() {
-  return sweep_threads(TP, TS) == 512   ? 1
-         : sweep_threads(TP, TS) == 384 ? 2
-         : is_char_mode<MODE>() && SweepOccupancy<T, FLUX>::value > 2 ? 2
-                                                                      : SweepOccupancy<T, FLUX>::value;
+  return sizeof(T) == 4 && !is_char_mode<MODE>() ? 3 : 2;
 }
 
-template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, int NL>
-__global__ void __launch_bounds__(sweep_threads(TP, TS), (sweep_min_blocks<T, MODE, FLUX, TP, TS>()))
+template <class T, int MODE, int STAGE, int TP, int TS, int NL>
+__global__ void __launch_bounds__(sweep_threads(TP, TS), (sweep_min_blocks<T, MODE>()))
     k_sweep(const __grid_constant__ SweepArgs3<T> sweeps) {
 #define HGKS_SW_B blockIdx.x
 #include "sweep_body.inc"
