@@ -100,8 +100,8 @@ SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
 
 // k_sweep with a TP x TS tile and NL layers per face-field pass.  The march
 // along the normal carries nothing from one pass to the next, so its length
-// only sets the number of CTAs: four per SM, down to one pass each on small
-// grids.
+// only sets the number of CTAs: 24 per SM for the three directions, down to
+// one pass each on small grids.
 template <class T, int TP, int TS, int NL>
 SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   SweepArgs3<T> a = sweep_common(e, q);
@@ -115,7 +115,7 @@ SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   for (int d = 0; d < 3; ++d) {
     int chunk = e.sweep_chunk;
     if (chunk <= 0) {
-      const int want_chunks = (12 * e.sms + tiles - 1) / tiles;
+      const int want_chunks = (24 * e.sms + tiles - 1) / tiles;
       chunk = (a.layers[d] + want_chunks - 1) / want_chunks;
     }
     chunk = (chunk + NL - 1) / NL * NL;

@@ -20,9 +20,10 @@
 // overlap.  In FP64 the tile grows from 8 x 8 to 16 x 8 (face fields at 1.9
 // points per face instead of 2.25), and every reconstruction of the pass along
 // t2 serves both abscissae (four threads per face made each of them twice).
-// Measured (GB300, one step): FP32 WENO-Z 256^3 73.4 -> 59.9 ms; in
-// characteristic variables 90x75x67 2.59 -> 2.25 ms; eight boxes of 32^3 to 96^3
-// 11.4 -> 9.28 ms; FP64 WENO-Z 64^3 71.1 -> 48.1 ms.
+// Measured (GB300, one step): FP32 WENO-Z 256^3 73.4 -> 59.9 ms (56.3 with the
+// strides as constants and shorter chunks); in characteristic variables
+// 90x75x67 2.59 -> 2.24 ms; eight boxes of 32^3 to 96^3 11.4 -> 8.92 ms; FP64
+// WENO-Z 64^3 71.1 -> 46.0 ms.
 // Bound by the FMA pipe and the reciprocal unit (FP32), the FP64 pipe (FP64).
 #pragma once
 
@@ -172,9 +173,10 @@ __device__ __forceinline__ void t2_pass_full(const T* tb, int m1, int at, int st
   }
 }
 
-// Body of one block: `sweeps` the arguments, b the block.
-template <class T, int MODE, int STAGE, int TP, int TS>
-__device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, int b) {
+// One tile's chunk.  t1 runs along P (the x and z sweeps) or along S, as a
+// compile-time choice: the strides of both passes are then constants.
+template <class T, int MODE, int STAGE, int TP, int TS, bool T1P>
+__device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, int by, int bz) {
   using L = FullSweep<T, MODE, TP, TS>;
   constexpr int HP = L::HP, HS = L::HS, NH = L::NH, NV = L::NV, NT = L::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -182,12 +184,9 @@ __device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, in
   T* tb = ff + L::NFF * NH;                // [NT1][NH]
   T* slot = tb + L::NT1 * NH + threadIdx.x;  // [SLOTS][NT], this thread's column
 
-  int bx, by, bz;
-  const SweepArgs<T> a = sweep_of_block(sweeps, b, bx, by, bz);
   const int d = a.d;
   const SweepAxes ax = sweep_axes(d, a.g, a.xt != 0);
   const int P = ax.P, S = ax.S;
-  const bool t1P = ax.t1P;
   const int nP = a.g.n[P], nS = a.g.n[S], nd = a.g.n[d];
   const int p0 = bx * TP, s0 = by * TS;
   const int f0 = bz * a.chunk, f1 = min(f0 + a.chunk, a.layers);
@@ -200,9 +199,9 @@ __device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, in
   const bool live = s0 + is < nS;  // the warp's row exists
   const bool face = live && p0 + ip < nP;
   const int cP = min(p0 + ip, nP - 1), cS = min(s0 + is, nS - 1);
-  const T rh1 = T(1) / a.wt1[(t1P ? cP : cS) + kGhost], rh2 = T(1) / a.wt2[(t1P ? cS : cP) + kGhost];
+  const T rh1 = T(1) / a.wt1[(T1P ? cP : cS) + kGhost], rh2 = T(1) / a.wt2[(T1P ? cS : cP) + kGhost];
   const int at3 = (is + 2) * HP + (ip + 2);
-  const int st1 = t1P ? 1 : HP, st2 = t1P ? HP : 1;
+  constexpr int st1 = T1P ? 1 : HP, st2 = T1P ? HP : 1;
   const T dt = T(a.scal[0]);
   const long long FS = (long long)(a.g.n[0] + (d == 0)) * (a.g.n[1] + (d == 1)) * (a.g.n[2] + (d == 2));
   // Face-flux layout: x fastest for the y and z faces; y fastest ([z][x][y])
@@ -238,12 +237,12 @@ __device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, in
     for (int s = 0; s < 3; ++s) {
       // ---------------- phase 2: pass along t1 of group s ----------------
       // Points of the tile with a halo of 2 along t2.
-      const int items = t1P ? TP * HS : HP * TS;
+      constexpr int items = T1P ? TP * HS : HP * TS;
       constexpr int UNITS = is_char_mode<MODE>() ? 2 : 5;
 #pragma unroll 1
       for (int it = tid; it < UNITS * items; it += NT) {
         const int u = it / items, pt = it - u * items;
-        const int at = t1P ? (pt / TP) * HP + 2 + pt % TP : 2 * HP + pt;
+        const int at = T1P ? (pt / TP) * HP + 2 + pt % TP : 2 * HP + pt;
         if constexpr (is_char_mode<MODE>()) t1_pass_char<T, MODE, NV, NH>(ff, tb, s, u == 1, at, st1, a.gas);
         else t1_pass_unit<T, MODE, NV, NH>(ff, tb, s, at, st1, u);
       }
@@ -321,6 +320,15 @@ __device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, in
       if (s < 2 || is_char_mode<MODE>()) __syncthreads();
     }
   }
+}
+
+// Body of one block: `sweeps` the arguments, b the block.
+template <class T, int MODE, int STAGE, int TP, int TS>
+__device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, int b) {
+  int bx, by, bz;
+  const SweepArgs<T> a = sweep_of_block(sweeps, b, bx, by, bz);
+  if (a.d == 1) sweep_full_tile<T, MODE, STAGE, TP, TS, false>(a, bx, by, bz);
+  else sweep_full_tile<T, MODE, STAGE, TP, TS, true>(a, bx, by, bz);
 }
 
 template <class T, int MODE, int STAGE, int TP, int TS>
