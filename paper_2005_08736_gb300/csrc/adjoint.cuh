@@ -30,203 +30,198 @@
 
 namespace hgks {
 
+// cot[j] += hL drL/dq_j + hR drR/dq_j for the nonlinear WENO5 deviations of
+// weno5_dev (recon.cuh), in reverse mode through the same differences: rR =
+// nR/SR, so the cotangent of a candidate p_k is h a_k/S and that of its weight
+// a_k is h (p_k - rR)/S; the weight factors f_k depend on the smoothness
+// indicators (WENO-JS: f = B^-2; WENO-Z: f = 1 + tau5/B, tau5 = |b0 - b2|,
+// d|x|/dx = sign(x) with sign(0) = 0), each a sum of two squares of linear
+// forms in the differences, and the differences' cotangents telescope onto q.
+// FP64: one reciprocal of B0 B1 B2 and one of SR SL replace eight divisions
+// (in range for |q| up to 1e25, as in weno5_dev).  About 120 operations and
+// two divisions, against 230 and eight from the candidates' coefficients in
+// the averages (whose zero products FP64 has to carry out): the adjoint
+// evaluates this some 50 times per face.
+template <int MODE, class T>
+HGKS_HD void weno5_dev_vjp(const T q[5], T hL, T hR, T cot[5]) {
+  static_assert(MODE == RECON_WENO_JS || MODE == RECON_WENO_Z, "nonlinear weights");
+  const T D1 = q[1] - q[0], D2 = q[2] - q[1], D3 = q[3] - q[2], D4 = q[4] - q[3];
+  const T s0 = D2 - D1, s1 = D3 - D2, s2 = D4 - D3;
+  const T t0 = T(2) * D2 + s0, t1 = D2 + D3, t2 = T(2) * D3 - s2;
+  const T w = t0 + D2, z = t2 + D3;
+  const T c0 = w + s0, c1 = t1 + D3, e0 = z - s2, e1 = t1 + D2;
+  const T k = T(3) / T(13);
+  const T b0 = k * t0 * t0 + s0 * s0, b1 = k * t1 * t1 + s1 * s1, b2 = k * t2 * t2 + s2 * s2;
+  const T e = MODE == RECON_WENO_JS ? T(12e-6 / 13) : T(12e-20 / 13);
+  const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+  T r0, r1, r2;  // 1/B
+  if constexpr (std::is_same<T, float>::value) {
+    r0 = T(1) / B0;
+    r1 = T(1) / B1;
+    r2 = T(1) / B2;
+  } else {
+    const T p12 = B1 * B2, p = T(1) / (B0 * p12), u = p * B0;
+    r0 = p * p12;
+    r1 = u * B2;
+    r2 = u * B1;
+  }
+  T f0, f1, f2, tau5 = T(0);
+  if (MODE == RECON_WENO_JS) {
+    f0 = r0 * r0;
+    f1 = r1 * r1;
+    f2 = r2 * r2;
+  } else {
+    tau5 = tabs(b0 - b2);
+    f0 = T(1) + tau5 * r0;
+    f1 = T(1) + tau5 * r1;
+    f2 = T(1) + tau5 * r2;
+  }
+  const T g0 = T(3) * f0, g1 = T(6) * f1, g2 = T(3) * f2;
+  const T SR = f0 + g1 + g2, SL = f2 + g1 + g0;
+  T iR, iL;
+  if constexpr (std::is_same<T, float>::value) {
+    iR = T(1) / SR;
+    iL = T(1) / SL;
+  } else {
+    const T inv = T(1) / (SR * SL);
+    iR = SL * inv;
+    iL = SR * inv;
+  }
+  const T rR = (f0 * c0 + g1 * c1 + g2 * z) * iR, rl = (f2 * e0 + g1 * e1 + g0 * w) * iL;  // rl = -rL
+  const T aR = hR * iR, aL = -(hL * iL);
+  // weight factors, then the indicators
+  const T F0 = aR * (c0 - rR) + T(3) * (aL * (w - rl));
+  const T F1 = T(6) * (aR * (c1 - rR) + aL * (e1 - rl));
+  const T F2 = T(3) * (aR * (z - rR)) + aL * (e0 - rl);
+  T G0, G1, G2;
+  if (MODE == RECON_WENO_JS) {
+    G0 = T(-2) * F0 * f0 * r0;
+    G1 = T(-2) * F1 * f1 * r1;
+    G2 = T(-2) * F2 * f2 * r2;
+  } else {
+    // (F tau5 r) r in this order: r^2 alone overflows FP32 where b vanishes
+    // (r = 1e20), and tau5 = 0 there.
+    const T d02 = b0 - b2, sg = d02 > T(0) ? T(1) : (d02 < T(0) ? T(-1) : T(0));
+    const T gt = sg * (F0 * r0 + F1 * r1 + F2 * r2);
+    G0 = gt - F0 * tau5 * r0 * r0;
+    G1 = -(F1 * tau5 * r1 * r1);
+    G2 = -(gt + F2 * tau5 * r2 * r2);
+  }
+  // candidates and indicators onto the differences
+  const T C0 = aR * f0, C1 = aR * g1, E0 = aL * f2, E1 = aL * g1;
+  const T Z = aR * g2 + E0, W = aL * g0 + C0;
+  const T k2 = T(2) * k;
+  const T T0 = k2 * (t0 * G0) + W, T1 = k2 * (t1 * G1) + (C1 + E1), T2 = k2 * (t2 * G2) + Z;
+  const T S0 = T(2) * (s0 * G0) + C0 + T0, S1 = T(2) * (s1 * G1), S2 = T(2) * (s2 * G2) - E0 - T2;
+  const T d2 = T(2) * T0 + T1 + E1 + W + S0 - S1, d3 = T(2) * T2 + T1 + C1 + Z + S1 - S2;
+  // D1: -S0, D4: S2
+  cot[0] += S0;
+  cot[1] -= S0 + d2;
+  cot[2] += d2 - d3;
+  cot[3] += d3 - S2;
+  cot[4] += S2;
+}
+
 // cot[j] += gL dqL/dq_j + gR dqR/dq_j for the WENO5 end values of the centre
-// cell (weno5_pair), in reverse mode: q_end = sum_k a_k p_k / sum_k a_k, so
-// the cotangent of p_k is g a_k/S and that of a_k is g (p_k - q_end)/S; the
-// weights' factors f_k depend on the smoothness indicators beta_k (WENO-JS:
-// f = (eps + beta)^-2; WENO-Z: f = 1 + tau5/(beta + eps), tau5 = |beta0 -
-// beta2|, d|x|/dx = sign(x) with sign(0) = 0), each a quadratic form of q.
+// cell (weno5_pair).
 template <int MODE_, class T>
 HGKS_HD void weno5_pair_vjp(const T q[5], T gL, T gR, T cot[5]) {
   constexpr int MODE = recon_of<MODE_>();
-  const T c6 = T(1) / T(6);
-  // Candidate polynomials: d pR_k / dq and d pL_k / dq (times 6).
-  const T dR[3][5] = {{2, -7, 11, 0, 0}, {0, -1, 5, 2, 0}, {0, 0, 2, 5, -1}};
-  const T dL[3][5] = {{0, 0, 11, -7, 2}, {0, 2, 5, -1, 0}, {-1, 5, 2, 0, 0}};
   if constexpr (MODE == RECON_LINEAR) {
-    const T w[3] = {T(0.1), T(0.6), T(0.3)};
-#pragma unroll
-    for (int j = 0; j < 5; ++j)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) cot[j] += (gR * w[k] * dR[k][j] + gL * w[k] * dL[k][j]) * c6;
+    const T r = gR * (T(1) / T(60)), l = gL * (T(1) / T(60));
+    cot[0] += T(2) * r - T(3) * l;
+    cot[1] += T(27) * l - T(13) * r;
+    cot[2] += T(47) * (r + l);
+    cot[3] += T(27) * r - T(13) * l;
+    cot[4] += T(2) * l - T(3) * r;
   } else {
-    T pR[3], pL[3];
-  #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      pR[k] = T(0);
-      pL[k] = T(0);
-  #pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        pR[k] += dR[k][j] * q[j];
-        pL[k] += dL[k][j] * q[j];
-      }
-      pR[k] *= c6;
-      pL[k] *= c6;
-    }
-    const T sv[3] = {q[0] - T(2) * q[1] + q[2], q[1] - T(2) * q[2] + q[3], q[2] - T(2) * q[3] + q[4]};
-    const T tv[3] = {q[0] - T(4) * q[1] + T(3) * q[2], q[1] - q[3], T(3) * q[2] - T(4) * q[3] + q[4]};
-    const T c13 = T(13) / T(12);
-    T bt[3], f[3];
-  #pragma unroll
-    for (int k = 0; k < 3; ++k) bt[k] = c13 * sv[k] * sv[k] + T(0.25) * tv[k] * tv[k];
-    T tau5 = T(0), sg = T(0);
-    if (MODE == RECON_WENO_JS) {
-  #pragma unroll
-      for (int k = 0; k < 3; ++k) f[k] = T(1) / ((T(1e-6) + bt[k]) * (T(1e-6) + bt[k]));
-    } else {
-      const T d02 = bt[0] - bt[2];
-      tau5 = tabs(d02);
-      sg = d02 > T(0) ? T(1) : (d02 < T(0) ? T(-1) : T(0));
-  #pragma unroll
-      for (int k = 0; k < 3; ++k) f[k] = T(1) + tau5 / (bt[k] + T(1e-20));
-    }
-    const T aR[3] = {T(0.1) * f[0], T(0.6) * f[1], T(0.3) * f[2]};
-    const T aL[3] = {T(0.1) * f[2], T(0.6) * f[1], T(0.3) * f[0]};
-    const T iSR = T(1) / (aR[0] + aR[1] + aR[2]), iSL = T(1) / (aL[0] + aL[1] + aL[2]);
-    const T qR = (aR[0] * pR[0] + aR[1] * pR[1] + aR[2] * pR[2]) * iSR;
-    const T qL = (aL[0] * pL[0] + aL[1] * pL[1] + aL[2] * pL[2]) * iSL;
-    T gaR[3], gaL[3];
-  #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      gaR[k] = gR * (pR[k] - qR) * iSR;
-      gaL[k] = gL * (pL[k] - qL) * iSL;
-    }
-    const T gf[3] = {T(0.1) * gaR[0] + T(0.3) * gaL[2], T(0.6) * (gaR[1] + gaL[1]),
-                     T(0.3) * gaR[2] + T(0.1) * gaL[0]};
-    T gb[3];
-    if (MODE == RECON_WENO_JS) {
-  #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const T e = T(1e-6) + bt[k];
-        gb[k] = gf[k] * T(-2) / (e * e * e);
-      }
-    } else {
-      T gtau = T(0);
-  #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const T ie = T(1) / (bt[k] + T(1e-20));
-        gb[k] = -gf[k] * tau5 * ie * ie;
-        gtau += gf[k] * ie;
-      }
-      gb[0] += gtau * sg;
-      gb[2] -= gtau * sg;
-    }
-    // beta_k = 13/12 s_k^2 + t_k^2 / 4, s_k and t_k linear in q.
-    const T ds[3][5] = {{1, -2, 1, 0, 0}, {0, 1, -2, 1, 0}, {0, 0, 1, -2, 1}};
-    const T dt[3][5] = {{1, -4, 3, 0, 0}, {0, 1, 0, -1, 0}, {0, 0, 3, -4, 1}};
-  #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const T gs = gb[k] * T(2) * c13 * sv[k], gt = gb[k] * T(0.5) * tv[k];
-      const T gpR = gR * aR[k] * iSR * c6, gpL = gL * aL[k] * iSL * c6;
-  #pragma unroll
-      for (int j = 0; j < 5; ++j) cot[j] += gs * ds[k][j] + gt * dt[k][j] + gpR * dR[k][j] + gpL * dL[k][j];
-    }
+    const T c6 = T(1) / T(6);
+    cot[2] += gL + gR;
+    weno5_dev_vjp<MODE>(q, gL * c6, gR * c6, cot);
   }
 }
 
-// weno5_pair_vjp (nonlinear weights) for two stencils at once, in the
-// halves of packed FP32 pairs: the forward quantities and the reverse pass
-// of the scalar function, pairwise; |beta0 - beta2|, its sign and the
-// reciprocals per half.
+// weno5_dev_vjp for two stencils at once, in the halves of packed FP32 pairs;
+// |b0 - b2|, its sign and the reciprocals per half.
+template <int MODE>
+HGKS_HD void weno5_dev_vjp_x2(const float2 q[5], float2 hL, float2 hR, float2 cot[5]) {
+  const float2 two = bc2(2.f), three = bc2(3.f), six = bc2(6.f), neg = bc2(-1.f);
+  const float2 D1 = sub2(q[1], q[0]), D2 = sub2(q[2], q[1]), D3 = sub2(q[3], q[2]), D4 = sub2(q[4], q[3]);
+  const float2 s0 = sub2(D2, D1), s1 = sub2(D3, D2), s2 = sub2(D4, D3);
+  const float2 t0 = fma2(two, D2, s0), t1 = add2(D2, D3), t2 = sub2(add2(D3, D3), s2);
+  const float2 w = add2(t0, D2), z = add2(t2, D3);
+  const float2 c0 = add2(w, s0), c1 = add2(t1, D3), e0 = sub2(z, s2), e1 = add2(t1, D2);
+  const float2 k = bc2(3.f / 13.f);
+  const float2 b0 = fma2(mul2(k, t0), t0, mul2(s0, s0));
+  const float2 b1 = fma2(mul2(k, t1), t1, mul2(s1, s1));
+  const float2 b2 = fma2(mul2(k, t2), t2, mul2(s2, s2));
+  const float2 e = bc2(MODE == RECON_WENO_JS ? 12e-6f / 13.f : 12e-20f / 13.f);
+  const float2 r0 = rcp2(add2(b0, e)), r1 = rcp2(add2(b1, e)), r2 = rcp2(add2(b2, e));
+  float2 f0, f1, f2, tau5 = bc2(0.f), sg = bc2(0.f);
+  if constexpr (MODE == RECON_WENO_JS) {
+    f0 = mul2(r0, r0);
+    f1 = mul2(r1, r1);
+    f2 = mul2(r2, r2);
+  } else {
+    const float2 d = sub2(b0, b2);
+    tau5 = make_float2(fabsf(d.x), fabsf(d.y));
+    sg = make_float2(d.x > 0.f ? 1.f : (d.x < 0.f ? -1.f : 0.f), d.y > 0.f ? 1.f : (d.y < 0.f ? -1.f : 0.f));
+    f0 = fma2(tau5, r0, bc2(1.f));
+    f1 = fma2(tau5, r1, bc2(1.f));
+    f2 = fma2(tau5, r2, bc2(1.f));
+  }
+  const float2 g0 = mul2(three, f0), g1 = mul2(six, f1), g2 = mul2(three, f2);
+  const float2 iR = rcp2(add2(add2(f0, g1), g2)), iL = rcp2(add2(add2(f2, g1), g0));
+  const float2 rR = mul2(fma2(f0, c0, fma2(g1, c1, mul2(g2, z))), iR);
+  const float2 rl = mul2(fma2(f2, e0, fma2(g1, e1, mul2(g0, w))), iL);
+  const float2 aR = mul2(hR, iR), aL = mul2(mul2(hL, neg), iL);
+  const float2 F0 = fma2(aR, sub2(c0, rR), mul2(three, mul2(aL, sub2(w, rl))));
+  const float2 F1 = mul2(six, fma2(aR, sub2(c1, rR), mul2(aL, sub2(e1, rl))));
+  const float2 F2 = fma2(three, mul2(aR, sub2(z, rR)), mul2(aL, sub2(e0, rl)));
+  float2 G0, G1, G2;
+  if constexpr (MODE == RECON_WENO_JS) {
+    G0 = mul2(mul2(mul2(bc2(-2.f), F0), f0), r0);
+    G1 = mul2(mul2(mul2(bc2(-2.f), F1), f1), r1);
+    G2 = mul2(mul2(mul2(bc2(-2.f), F2), f2), r2);
+  } else {
+    const float2 gt = mul2(sg, fma2(F0, r0, fma2(F1, r1, mul2(F2, r2))));
+    const float2 nt = mul2(tau5, neg);
+    G0 = fma2(mul2(mul2(F0, nt), r0), r0, gt);
+    G1 = mul2(mul2(mul2(F1, nt), r1), r1);
+    G2 = fma2(mul2(mul2(F2, nt), r2), r2, mul2(gt, neg));
+  }
+  const float2 C0 = mul2(aR, f0), C1 = mul2(aR, g1), E0 = mul2(aL, f2), E1 = mul2(aL, g1);
+  const float2 Z = fma2(aR, g2, E0), W = fma2(aL, g0, C0);
+  const float2 k2 = bc2(6.f / 13.f);
+  const float2 T0 = fma2(mul2(k2, t0), G0, W), T1 = fma2(mul2(k2, t1), G1, add2(C1, E1)), T2 = fma2(mul2(k2, t2), G2, Z);
+  const float2 S0 = fma2(mul2(two, s0), G0, add2(C0, T0)), S1 = mul2(mul2(two, s1), G1);
+  const float2 S2 = sub2(mul2(mul2(two, s2), G2), add2(E0, T2));
+  const float2 d2 = add2(fma2(two, T0, add2(T1, E1)), add2(W, sub2(S0, S1)));
+  const float2 d3 = add2(fma2(two, T2, add2(T1, C1)), add2(Z, sub2(S1, S2)));
+  cot[0] = add2(cot[0], S0);
+  cot[1] = sub2(cot[1], add2(S0, d2));
+  cot[2] = add2(cot[2], sub2(d2, d3));
+  cot[3] = add2(cot[3], sub2(d3, S2));
+  cot[4] = add2(cot[4], S2);
+}
+
+// weno5_pair_vjp (nonlinear weights) for two stencils at once.
 template <int MODE>
 HGKS_HD void weno5_pair_vjp_x2(const float2 q[5], float2 gL, float2 gR, float2 cot[5]) {
-  const float c6 = 1.f / 6.f;
-  const float dR[3][5] = {{2, -7, 11, 0, 0}, {0, -1, 5, 2, 0}, {0, 0, 2, 5, -1}};
-  const float dL[3][5] = {{0, 0, 11, -7, 2}, {0, 2, 5, -1, 0}, {-1, 5, 2, 0, 0}};
-  float2 pR[3], pL[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    pR[k] = bc2(0.f);
-    pL[k] = bc2(0.f);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      if (dR[k][j] != 0.f) pR[k] = fma2(bc2(dR[k][j]), q[j], pR[k]);
-      if (dL[k][j] != 0.f) pL[k] = fma2(bc2(dL[k][j]), q[j], pL[k]);
-    }
-    pR[k] = mul2(pR[k], bc2(c6));
-    pL[k] = mul2(pL[k], bc2(c6));
-  }
-  const float2 sv[3] = {fma2(bc2(-2.f), q[1], add2(q[0], q[2])), fma2(bc2(-2.f), q[2], add2(q[1], q[3])),
-                        fma2(bc2(-2.f), q[3], add2(q[2], q[4]))};
-  const float2 tv[3] = {fma2(bc2(-4.f), q[1], fma2(bc2(3.f), q[2], q[0])), sub2(q[1], q[3]),
-                        fma2(bc2(3.f), q[2], fma2(bc2(-4.f), q[3], q[4]))};
-  const float c13 = 13.f / 12.f;
-  float2 bt[3], f[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) bt[k] = fma2(mul2(bc2(c13), sv[k]), sv[k], mul2(mul2(bc2(0.25f), tv[k]), tv[k]));
-  float2 tau5 = bc2(0.f), sg = bc2(0.f);
-  if constexpr (MODE == RECON_WENO_JS) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float2 e = add2(bc2(1e-6f), bt[k]);
-      f[k] = rcp2(mul2(e, e));
-    }
-  } else {
-    const float2 d02 = sub2(bt[0], bt[2]);
-    tau5 = make_float2(fabsf(d02.x), fabsf(d02.y));
-    sg = make_float2(d02.x > 0.f ? 1.f : (d02.x < 0.f ? -1.f : 0.f), d02.y > 0.f ? 1.f : (d02.y < 0.f ? -1.f : 0.f));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) f[k] = fma2(tau5, rcp2(add2(bt[k], bc2(1e-20f))), bc2(1.f));
-  }
-  const float2 aR[3] = {mul2(bc2(0.1f), f[0]), mul2(bc2(0.6f), f[1]), mul2(bc2(0.3f), f[2])};
-  const float2 aL[3] = {mul2(bc2(0.1f), f[2]), mul2(bc2(0.6f), f[1]), mul2(bc2(0.3f), f[0])};
-  const float2 iSR = rcp2(add2(add2(aR[0], aR[1]), aR[2])), iSL = rcp2(add2(add2(aL[0], aL[1]), aL[2]));
-  const float2 qR = mul2(fma2(aR[0], pR[0], fma2(aR[1], pR[1], mul2(aR[2], pR[2]))), iSR);
-  const float2 qL = mul2(fma2(aL[0], pL[0], fma2(aL[1], pL[1], mul2(aL[2], pL[2]))), iSL);
-  float2 gaR[3], gaL[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    gaR[k] = mul2(mul2(gR, sub2(pR[k], qR)), iSR);
-    gaL[k] = mul2(mul2(gL, sub2(pL[k], qL)), iSL);
-  }
-  const float2 gf[3] = {fma2(bc2(0.1f), gaR[0], mul2(bc2(0.3f), gaL[2])), mul2(bc2(0.6f), add2(gaR[1], gaL[1])),
-                        fma2(bc2(0.3f), gaR[2], mul2(bc2(0.1f), gaL[0]))};
-  float2 gb[3];
-  if constexpr (MODE == RECON_WENO_JS) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float2 e = add2(bc2(1e-6f), bt[k]);
-      gb[k] = mul2(mul2(gf[k], bc2(-2.f)), rcp2(mul2(mul2(e, e), e)));
-    }
-  } else {
-    float2 gtau = bc2(0.f);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      // (-gf tau5 ie) ie, in the scalar order: ie^2 alone overflows FP32
-      // where beta vanishes (ie = 1e20), and tau5 = 0 there.
-      const float2 ie = rcp2(add2(bt[k], bc2(1e-20f)));
-      gb[k] = mul2(mul2(mul2(mul2(gf[k], bc2(-1.f)), tau5), ie), ie);
-      gtau = fma2(gf[k], ie, gtau);
-    }
-    gb[0] = fma2(gtau, sg, gb[0]);
-    gb[2] = fma2(mul2(gtau, bc2(-1.f)), sg, gb[2]);
-  }
-  // beta_k = 13/12 s_k^2 + t_k^2 / 4, s_k and t_k linear in q.
-  const float ds[3][5] = {{1, -2, 1, 0, 0}, {0, 1, -2, 1, 0}, {0, 0, 1, -2, 1}};
-  const float dt[3][5] = {{1, -4, 3, 0, 0}, {0, 1, 0, -1, 0}, {0, 0, 3, -4, 1}};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float2 gs = mul2(gb[k], mul2(bc2(2.f * c13), sv[k])), gt = mul2(gb[k], mul2(bc2(0.5f), tv[k]));
-    const float2 gpR = mul2(mul2(gR, aR[k]), mul2(iSR, bc2(c6))), gpL = mul2(mul2(gL, aL[k]), mul2(iSL, bc2(c6)));
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      if (ds[k][j] != 0.f) cot[j] = fma2(gs, bc2(ds[k][j]), cot[j]);
-      if (dt[k][j] != 0.f) cot[j] = fma2(gt, bc2(dt[k][j]), cot[j]);
-      if (dR[k][j] != 0.f) cot[j] = fma2(gpR, bc2(dR[k][j]), cot[j]);
-      if (dL[k][j] != 0.f) cot[j] = fma2(gpL, bc2(dL[k][j]), cot[j]);
-    }
-  }
+  const float2 c6 = bc2(1.f / 6.f);
+  cot[2] = add2(cot[2], add2(gL, gR));
+  weno5_dev_vjp_x2<MODE>(q, mul2(gL, c6), mul2(gR, c6), cot);
 }
 
 // tangential_vjp (nonlinear weights) of two five-point stencils at once.
 template <int MODE>
 HGKS_HD void tangential_vjp_x2(const float2 f[5], const float2 gv[2], const float2 gd[2],
                                                   float2 cot[5]) {
-  const float gs = 0.5f / 1.7320508075688772f;
-  const float2 gb = fma2(bc2(gs), sub2(gv[1], gv[0]), add2(gd[0], gd[1]));
-  const float2 gc = mul2(bc2(2.f * gs), sub2(gd[1], gd[0]));
-  cot[2] = add2(cot[2], fma2(bc2(-6.f), gc, add2(gv[0], gv[1])));
-  weno5_pair_vjp_x2<MODE>(f, fma2(bc2(3.f), gc, mul2(gb, bc2(-1.f))), fma2(bc2(3.f), gc, gb), cot);
+  const float gs = 0.5f / 1.7320508075688772f, c6 = 1.f / 6.f;
+  const float2 gb = fma2(bc2(gs * c6), sub2(gv[1], gv[0]), mul2(bc2(c6), add2(gd[0], gd[1])));
+  const float2 gr = mul2(bc2(gs), sub2(gd[1], gd[0]));
+  cot[2] = add2(cot[2], add2(gv[0], gv[1]));
+  weno5_dev_vjp_x2<MODE>(f, sub2(gr, gb), add2(gr, gb), cot);
 }
 
 // cot[j] += sum_m gv[m] dv[m]/df_j + gd[m] dd[m]/df_j for the tangential
@@ -236,7 +231,7 @@ HGKS_HD void tangential_vjp(const T f[5], const T gv[2], const T gd[2],
                                                T cot[5]) {
   constexpr int MODE = recon_of<MODE_>();
   const T sq3 = T(1.7320508075688772);
-  if (MODE == RECON_LINEAR) {
+  if constexpr (MODE == RECON_LINEAR) {
     // v = E -+ O, d = A -+ B (quartic through the five averages)
     const T gE = gv[0] + gv[1], gO = gv[1] - gv[0], gA = gd[0] + gd[1], gB = gd[1] - gd[0];
     const T e0 = T(1) / T(4320), e1 = T(1) / T(1080), e2 = T(719) / T(720);
@@ -248,14 +243,14 @@ HGKS_HD void tangential_vjp(const T f[5], const T gv[2], const T gd[2],
     cot[2] += gE * e2 - gB * b0 * T(24);
     cot[3] += gE * e1 + gO * o1 + gA * a1 + gB * b0 * T(13);
     cot[4] += -gE * e0 - gO * o0 - gA * a0 - gB * b0;
-    return;
+  } else {
+    // b = rR - rL, r = rL + rR: v = f2 -+ gs b/6, d = b/6 -+ gs r (tangential).
+    const T gs = T(0.5) / sq3, c6 = T(1) / T(6);
+    const T gb = (gs * c6) * (gv[1] - gv[0]) + c6 * (gd[0] + gd[1]);
+    const T gr = gs * (gd[1] - gd[0]);
+    cot[2] += gv[0] + gv[1];
+    weno5_dev_vjp<MODE>(f, gr - gb, gr + gb, cot);
   }
-  // p(+-g) = f2 +- b g, p'(+-g) = b +- 2 c g, b = qR - qL, c = 3(qL + qR) - 6 f2.
-  const T gs = T(0.5) / sq3;
-  const T gb = gs * (gv[1] - gv[0]) + gd[0] + gd[1];
-  const T gc = T(2) * gs * (gd[1] - gd[0]);
-  cot[2] += gv[0] + gv[1] - T(6) * gc;
-  weno5_pair_vjp<MODE>(f, -gb + T(3) * gc, gb + T(3) * gc, cot);
 }
 
 // (cl, cr) += J^T g0 for the compatibility state Q0(Q_l, Q_r) =
@@ -286,19 +281,20 @@ __device__ __forceinline__ void flux_vjp(const PointState<T>* st, const Gas<T>& 
   else flux_smooth_rev(st[0], gas, want_F, gF, gdF, cot[0]);
 }
 
+// The sweeps of the three directions in one launch: block b belongs to
+// direction d with start[d] <= b < start[d + 1] (they only add into acc).  One
+// direction of 64^3 or less fills the chip between four and five times, and its
+// last wave is nearly empty; the three together have one tail.
 template <class T>
 struct AdjArgs {
-  const T* __restrict__ q;      // padded state (deviation) with ghost cells filled
-  const T* __restrict__ wL;     // cotangent of L, [5][N] (null: zero)
-  const T* __restrict__ wdL;    // cotangent of dL/dt, [5][N]
-  T* __restrict__ acc;          // padded cotangent of the state, [5][P], accumulated
-  const T* __restrict__ wn;
-  const T* __restrict__ wt1;
-  const T* __restrict__ wt2;
-  const double* __restrict__ scal;
+  const T* q;      // padded state (deviation) with ghost cells filled
+  const T* wL;     // cotangent of L, [5][N] (null: zero)
+  const T* wdL;    // cotangent of dL/dt, [5][N]
+  T* acc;          // padded cotangent of the state, [5][P], accumulated
+  const T* w[3];   // widths (offset kGhost)
+  const double* scal;
   GridDev g;
-  int d;
-  int chunk;
+  int gx[3], gy[3], chunk[3], start[4];
   Gas<T> gas;
 };
 
@@ -343,7 +339,7 @@ __device__ __forceinline__ void t2_cot(const PointState<T>& p, int c, T rh1, T r
 }
 
 template <class T, int MODE, int FLUX, int TP, int TS, int NT>
-__global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
+__global__ void __launch_bounds__(NT) k_sweep_adj(const __grid_constant__ AdjArgs<T> a) {
   constexpr int HP = TP + 4, HS = TS + 4, NH = HP * HS;
   constexpr int NV = SweepLayout<FLUX>::NV;
   constexpr int NFF = SweepLayout<FLUX>::NFF;
@@ -352,6 +348,7 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
   constexpr int NFACE = TP * TS;
   constexpr int TPF = NT / NFACE;
   static_assert(TPF * NFACE == NT && (TPF == 2 || TPF == 4), "tile must give 2 or 4 threads per face");
+  static_assert(TP * TPF == 32, "a warp holds one row of the tile");
   constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ff = reinterpret_cast<T*>(smem_raw);  // [NFF][NH] face fields
@@ -359,14 +356,17 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
   T* tbc = tb + NT1 * NH;                  // [NT1][NH] cotangents of the t1 pass
   T* ffc = tbc + NT1 * NH;                 // [NFF][NH] cotangents of the face fields
 
-  const int d = a.d;
+  const int b = blockIdx.x;
+  const int d = b >= a.start[2] ? 2 : (b >= a.start[1] ? 1 : 0);
   const SweepAxes ax = sweep_axes(d, a.g);
   const int P = ax.P, S = ax.S;
   const bool t1P = ax.t1P;
   const int nP = a.g.n[P], nS = a.g.n[S], nd = a.g.n[d];
-  const int p0 = blockIdx.x * TP, s0 = blockIdx.y * TS;
-  const int f0 = blockIdx.z * a.chunk;
-  const int f1 = min(f0 + a.chunk, nd + 1);
+  const int rel = b - a.start[d], gx = a.gx[d], gy = a.gy[d];
+  const int p0 = (rel % gx) * TP, s0 = (rel / gx) % gy * TS;
+  const int f0 = rel / (gx * gy) * a.chunk[d];
+  const int f1 = min(f0 + a.chunk[d], nd);  // periodic: face n is face 0
+  const T *wn = a.w[d], *wt1 = a.w[(d + 1) % 3], *wt2 = a.w[(d + 2) % 3];
   const int tid = threadIdx.x;
   const T dt = T(a.scal[0]);
 
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
   const bool f_valid = (p0 + ip < nP) && (s0 + is < nS);
   const int cP = min(p0 + ip, nP - 1), cS = min(s0 + is, nS - 1);
   const int ct1 = t1P ? cP : cS, ct2 = t1P ? cS : cP;
-  const T rh1 = T(1) / a.wt1[ct1 + kGhost], rh2 = T(1) / a.wt2[ct2 + kGhost];
+  const T rh1 = T(1) / wt1[ct1 + kGhost], rh2 = T(1) / wt2[ct2 + kGhost];
   const int at3 = (is + 2) * HP + (ip + 2);
   const int st2 = t1P ? HP : 1;
   const int st1 = t1P ? 1 : HP;
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
       const int hp = h % HP, hs = h / HP;
       const int Pc = p0 - 2 + hp, Sc = s0 - 2 + hs;
       if (Pc <= nP + 1 && Sc <= nS + 1) {
-        face_fields_item<T, MODE, FLUX, NH>(a.q, a.g, ax, a.wn, a.gas, f, Pc, Sc, h, ff);
+        face_fields_item<T, MODE, FLUX, NH>(a.q, a.g, ax, wn, a.gas, f, Pc, Sc, h, ff);
       } else {
 #pragma unroll 1
         for (int k = 0; k < NFF; ++k) ff[k * NH + h] = T(0);
@@ -415,9 +415,10 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
     __syncthreads();
 
     // ---------------- R3: flux VJP and transposed t2 pass ----------------
-    // Every thread takes part (the pair shuffles); a face outside the grid
-    // computes on the tile's padding and adds nothing.
-    {
+    // A warp holds faces of one row, and every thread of a row that exists
+    // takes part (the pair shuffles); a face outside the grid computes on the
+    // tile's padding and adds nothing.
+    if (s0 + is < nS) {
       // Face-flux cotangents from L_c = -(F_{c+1/2} - F_{c-1/2}) / h_c: the face
       // f is the right face of cell f-1 and the left face of cell f.
       T gF[5], gdF[5];
@@ -428,12 +429,11 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
         c[S] = cS;
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
-          const int cell = f - 1 + side;
-          if (cell < 0 || cell >= nd) continue;
+          const int cell = f - 1 + side < 0 ? nd - 1 : f - 1 + side;
           c[d] = cell;
           const long long ci = ((long long)c[2] * a.g.n[1] + c[1]) * a.g.n[0] + c[0];
           const T sgn = side == 0 ? T(-1) : T(1);
-          const T r = sgn / a.wn[cell + kGhost];
+          const T r = sgn / wn[cell + kGhost];
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
             if (a.wL) cF[v] += r * a.wL[v * a.g.N + ci];
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(NT) k_sweep_adj(AdjArgs<T> a) {
     // R1b, per point and component: the normal slopes and the WENO5 pairs
     // transposed, scattered into the cells f-3 .. f+2.
     {
-      const T hl = a.wn[f - 1 + kGhost], hr = a.wn[f + kGhost];
+      const T hl = wn[f - 1 + kGhost], hr = wn[f + kGhost];
       const T rhl = T(1) / hl, rhr = T(1) / hr, r6 = T(1) / (T(6) * (hl + hr));
       for (int u = tid; u < 5 * NH; u += NT) {
         const int h = u % NH, i = u / NH;

@@ -378,31 +378,33 @@ cudaError_t launch_adjoint_sweeps(const Engine& e, const T* q, const T* wL, cons
   auto kern = k_sweep_adj<T, MODE, FLUX, TP, TS, NT>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
+  AdjArgs<T> a;
+  a.q = q;
+  a.wL = wL;
+  a.wdL = wdL;
+  a.acc = static_cast<T*>(e.adj_acc);
+  a.scal = e.scal;
+  a.g = g;
+  a.gas = gas_of<T>(e.cfg);
+  a.start[0] = 0;
+  int tiles = 0;
   for (int d = 0; d < 3; ++d) {
-    AdjArgs<T> a;
-    a.q = q;
-    a.wL = wL;
-    a.wdL = wdL;
-    a.acc = static_cast<T*>(e.adj_acc);
-    a.wn = static_cast<const T*>(e.w[d]);
-    a.wt1 = static_cast<const T*>(e.w[(d + 1) % 3]);
-    a.wt2 = static_cast<const T*>(e.w[(d + 2) % 3]);
-    a.scal = e.scal;
-    a.g = g;
-    a.d = d;
-    a.gas = gas_of<T>(e.cfg);
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
-    const int gx = (g.n[P] + TP - 1) / TP, gy = (g.n[S] + TS - 1) / TS;
-    const int layers = g.n[d] + 1;
-    const int want_chunks = (4 * e.sms + gx * gy - 1) / (gx * gy);
-    int chunk = (layers + want_chunks - 1) / want_chunks;
-    if (chunk < 1) chunk = 1;
-    a.chunk = chunk;
-    const int gz = (layers + chunk - 1) / chunk;
-    kern<<<dim3(gx, gy, gz), NT, smem, e.stream>>>(a);
-    err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
+    a.w[d] = static_cast<const T*>(e.w[d]);
+    a.gx[d] = (g.n[P] + TP - 1) / TP;
+    a.gy[d] = (g.n[S] + TS - 1) / TS;
+    tiles += a.gx[d] * a.gy[d];
   }
+  // A layer takes tens of microseconds and shares nothing with the next, so
+  // the chunks are short: 24 CTAs per SM keep the tail under a few per cent.
+  const int want_chunks = (24 * e.sms + tiles - 1) / tiles;
+  for (int d = 0; d < 3; ++d) {
+    a.chunk[d] = std::max(1, (g.n[d] + want_chunks - 1) / want_chunks);
+    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * ((g.n[d] + a.chunk[d] - 1) / a.chunk[d]);
+  }
+  kern<<<a.start[3], NT, smem, e.stream>>>(a);
+  err = cudaGetLastError();
+  if (err != cudaSuccess) return err;
   T* acc = static_cast<T*>(e.adj_acc);
   k_fold_ghosts_z<T><<<blocks_for(6LL * g.p[0] * g.p[1], 256), 256, 0, e.stream>>>(acc, g);
   k_fold_ghosts_y<T><<<blocks_for(6LL * g.p[0] * g.n[2], 256), 256, 0, e.stream>>>(acc, g);
