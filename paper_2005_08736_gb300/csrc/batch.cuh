@@ -11,7 +11,7 @@
 
 #include "kernels.cuh"
 #include "march.cuh"
-#include "sweep_full.cuh"
+#include "sweep_tile.cuh"
 
 namespace hgks {
 
@@ -62,25 +62,12 @@ struct PadJob {
   __device__ __forceinline__ void run(int b) const { pad_block(a, b % gx, (b / gx) % gy, b / (gx * gy)); }
 };
 
-template <class T, int MODE, int STAGE, int TP, int TS, int NL>
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS>
 struct SweepJob {
-  static constexpr int kThreads = sweep_threads(TP, TS);
-  static constexpr int kMinBlocks = sweep_min_blocks<T, MODE>();
+  static constexpr int kThreads = SweepShape<T, MODE, FLUX, TP, TS>::THREADS;
+  static constexpr int kMinBlocks = SweepShape<T, MODE, FLUX, TP, TS>::MIN_BLOCKS;
   SweepArgs3<T> a;
-  __device__ __forceinline__ void run(int b) const {
-    const SweepArgs3<T>& sweeps = a;
-#define HGKS_SW_B b
-#include "sweep_body.inc"
-#undef HGKS_SW_B
-  }
-};
-
-template <class T, int MODE, int STAGE, int TP, int TS>
-struct SweepFullJob {
-  static constexpr int kThreads = FullSweep<T, MODE, TP, TS>::THREADS;
-  static constexpr int kMinBlocks = FullSweep<T, MODE, TP, TS>::MIN_BLOCKS;
-  SweepArgs3<T> a;
-  __device__ __forceinline__ void run(int b) const { sweep_full_block<T, MODE, STAGE, TP, TS>(a, b); }
+  __device__ __forceinline__ void run(int b) const { sweep_block<T, MODE, FLUX, STAGE, TP, TS>(a, b); }
 };
 
 template <int STAGE>

@@ -6,7 +6,7 @@
 #include "kernels.cuh"
 #include "sweep.cuh"
 #include "march.cuh"
-#include "sweep_full.cuh"
+#include "sweep_tile.cuh"
 #include "adjoint.cuh"
 #include "turbulence.cuh"
 #include "batch.cuh"
@@ -72,11 +72,12 @@ cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe)
   return cudaGetLastError();
 }
 
-// Tiles of the sweep kernels: TP x TS faces, sized so that the shared-memory
-// staging fits; NL face layers share one face-field pass (phase 1) of the
-// smooth flux.
-template <class T> struct SweepTile { static constexpr int TP = 16, TS = 8, NL = sizeof(T) == 4 ? 4 : 2; };
-template <class T> struct FullTile { static constexpr int TP = 16, TS = 8; };
+// Tile of k_sweep, TP x TS faces.  FP64 is bound by its pipe, not by latency:
+// with the smooth flux one CTA of 512 threads has 1.56 points of face fields
+// per face where two of 16 x 8 faces have 1.88.
+template <class T, int FLUX> struct SweepTile {
+  static constexpr int TP = 16, TS = sizeof(T) == 8 && FLUX == FLUX_SMOOTH ? 16 : 8;
+};
 
 // What the three sweeps of a stage on the padded state q share.
 template <class T>
@@ -98,11 +99,10 @@ SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
   return a;
 }
 
-// k_sweep with a TP x TS tile and NL layers per face-field pass.  The march
-// along the normal carries nothing from one pass to the next, so its length
-// only sets the number of CTAs: 24 per SM for the three directions, down to
-// one pass each on small grids.
-template <class T, int TP, int TS, int NL>
+// k_sweep with a TP x TS tile.  The march along the normal carries nothing
+// from one layer to the next, so its length only sets the number of CTAs: 24
+// per SM for the three directions, down to one layer each on small grids.
+template <class T, int TP, int TS>
 SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   SweepArgs3<T> a = sweep_common(e, q);
   int tiles = 0;
@@ -118,22 +118,10 @@ SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
       const int want_chunks = (24 * e.sms + tiles - 1) / tiles;
       chunk = (a.layers[d] + want_chunks - 1) / want_chunks;
     }
-    chunk = (chunk + NL - 1) / NL * NL;
     a.chunk[d] = chunk;
     a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * ((a.layers[d] + chunk - 1) / chunk);
   }
   return a;
-}
-
-template <class T, int MODE, int STAGE, int TP, int TS, int NL>
-cudaError_t launch_sweep_tile(const Engine& e, const T* q) {
-  const SweepArgs3<T> a = sweep_args<T, TP, TS, NL>(e, q);
-  constexpr size_t smem = sweep_smem_bytes<T, MODE, TP, TS, NL>();
-  auto kern = k_sweep<T, MODE, STAGE, TP, TS, NL>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  kern<<<a.start[3], sweep_threads(TP, TS), smem, e.stream>>>(a);
-  return cudaGetLastError();
 }
 
 // k_march: every block takes the same number of rows of the sequence of all
@@ -155,17 +143,6 @@ inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks
   return a;
 }
 
-template <class T, int MODE, int STAGE, int TP, int TS>
-cudaError_t launch_sweep_full(const Engine& e, const T* q) {
-  using L = FullSweep<T, MODE, TP, TS>;
-  const SweepArgs3<T> a = sweep_args<T, TP, TS, 1>(e, q);
-  auto kern = k_sweep_full<T, MODE, STAGE, TP, TS>;
-  const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM);
-  if (err != cudaSuccess) return err;
-  kern<<<a.start[3], L::THREADS, L::SMEM, e.stream>>>(a);
-  return cudaGetLastError();
-}
-
 template <class T, int MODE, int FLUX, int STAGE>
 cudaError_t launch_sweep(const Engine& e, const T* q) {
   if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
@@ -176,10 +153,15 @@ cudaError_t launch_sweep(const Engine& e, const T* q) {
     if (err != cudaSuccess) return err;
     k_march<STAGE><<<blocks, March::THREADS, March::SMEM, e.stream>>>(a);
     return cudaGetLastError();
-  } else if constexpr (FLUX == FLUX_FULL) {
-    return launch_sweep_full<T, MODE, STAGE, FullTile<T>::TP, FullTile<T>::TS>(e, q);
   } else {
-    return launch_sweep_tile<T, MODE, STAGE, SweepTile<T>::TP, SweepTile<T>::TS, SweepTile<T>::NL>(e, q);
+    constexpr int TP = SweepTile<T, FLUX>::TP, TS = SweepTile<T, FLUX>::TS;
+    using L = SweepShape<T, MODE, FLUX, TP, TS>;
+    const SweepArgs3<T> a = sweep_args<T, TP, TS>(e, q);
+    auto kern = k_sweep<T, MODE, FLUX, STAGE, TP, TS>;
+    const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM);
+    if (err != cudaSuccess) return err;
+    kern<<<a.start[3], L::THREADS, L::SMEM, e.stream>>>(a);
+    return cudaGetLastError();
   }
 }
 
@@ -502,22 +484,14 @@ cudaError_t batched_sweeps(const std::vector<Engine*>& ms, int stage, cudaStream
       blocks.push_back(nb);
     }
     return launch_batched(jobs, blocks, March::SMEM, s);
-  } else if constexpr (FLUX == FLUX_FULL) {
-    constexpr int TP = FullTile<T>::TP, TS = FullTile<T>::TS;
-    std::vector<SweepFullJob<T, MODE, STAGE, TP, TS>> jobs;
-    for (Engine* e : ms) {
-      jobs.push_back({sweep_args<T, TP, TS, 1>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
-      blocks.push_back(jobs.back().a.start[3]);
-    }
-    return launch_batched(jobs, blocks, FullSweep<T, MODE, TP, TS>::SMEM, s);
   } else {
-    constexpr int TP = SweepTile<T>::TP, TS = SweepTile<T>::TS, NL = SweepTile<T>::NL;
-    std::vector<SweepJob<T, MODE, STAGE, TP, TS, NL>> jobs;
+    constexpr int TP = SweepTile<T, FLUX>::TP, TS = SweepTile<T, FLUX>::TS;
+    std::vector<SweepJob<T, MODE, FLUX, STAGE, TP, TS>> jobs;
     for (Engine* e : ms) {
-      jobs.push_back({sweep_args<T, TP, TS, NL>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
+      jobs.push_back({sweep_args<T, TP, TS>(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
       blocks.push_back(jobs.back().a.start[3]);
     }
-    return launch_batched(jobs, blocks, sweep_smem_bytes<T, MODE, TP, TS, NL>(), s);
+    return launch_batched(jobs, blocks, SweepShape<T, MODE, FLUX, TP, TS>::SMEM, s);
   }
 }
 

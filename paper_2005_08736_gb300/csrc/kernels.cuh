@@ -56,7 +56,7 @@ __host__ __device__ __forceinline__ FaceBox face_box(const GridDev& g, int d, in
 // The ghost fill and the CFL reduction are bodies over explicit block
 // coordinates (device functions) with thin __global__ wrappers; the update
 // and the sweep keep their bodies in the kernels, as included texts
-// (update_body.inc, sweep_body.inc).  The ensemble's batched launches
+// (update_body.inc).  The ensemble's batched launches
 // (batch.cuh) run the same bodies for many instances in one grid.
 
 // Ghost cells of the padded state q and, if qx is not null, the copy of the

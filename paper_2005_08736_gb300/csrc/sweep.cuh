@@ -1,23 +1,5 @@
-// Fused sweep kernel of the smooth flux: for one direction d and one S2O4
-// stage, the face fields, the tangential reconstruction to the 2x2 Gauss
-// points and the BGK flux there, for a 2D tile of faces marching along the
-// normal.  (FP32 with linear weights: march.cuh; the full flux:
-// sweep_full.cuh, with the pieces it shares here.)
-//
-// Tile: TP x TS faces in the transverse plane, P = the faster-varying
-// transverse axis in memory, S = the slower one; the CTA marches through a
-// chunk of faces f0..f1-1 along d (face f lies between cells f-1 and f).
-// Per face layer:
-//   phase 1  one thread per transverse point of the tile plus a halo of 2:
-//            the six cells f-3..f+2 along d (L1-cached loads), WENO5 end
-//            values of cells f-1 and f, the normal slopes, the compatibility
-//            state Q0 and its normal slope -> face fields in shared memory;
-//   phase 2  the tangential pass along t1 = d+1 for every point of the tile
-//            (halo 2 along t2): values at the two t1 Gauss abscissae, and
-//            t1-derivatives of the state fields -> shared memory;
-//   phase 3  the tangential pass along t2 = d+2 and the flux at each Gauss
-//            point; TPF threads per face, each with 4/TPF Gauss points,
-//            summed with weights 1/4 into the face flux, written to HBM.
+// Pieces of the fused sweep kernels (sweep_tile.cuh, march.cuh, adjoint.cuh):
+// launch arguments, tile geometry, face fields and the tangential passes.
 #pragma once
 
 #include "charvars.cuh"
@@ -104,16 +86,25 @@ struct SweepLayout {
   static constexpr int NT1 = 4 * NV + 2 * NV;            // t1 pass outputs
 };
 
-// Threads of a sweep CTA: 256, or one per face for tiles of more faces.
-__host__ __device__ constexpr int sweep_threads(int tp, int ts) { return tp * ts > 256 ? tp * ts : 256; }
-
-template <class T, int MODE, int TP, int TS, int NL>
-constexpr size_t sweep_smem_bytes() {
-  constexpr int FLUX = FLUX_SMOOTH;
-  constexpr int NH = (TP + 4) * (TS + 4);
-  constexpr int TPF = sweep_threads(TP, TS) / (TP * TS);
-  return sizeof(T) * ((NL * SweepLayout<FLUX, MODE>::NFF + SweepLayout<FLUX, MODE>::NT1) * NH +
-                      (TPF - 1) * 10 * TP * TS);
+// tangential() with the sums and differences of the linear weights shared and
+// their constants folded: 18 operations against 22 (11 against 12 for values
+// only), which FP64 pays for one by one.
+template <int MODE, class T>
+__device__ __forceinline__ void tangential_fast(T f0, T f1, T f2, T f3, T f4, T v[2], T d[2]) {
+  if constexpr (recon_of<MODE>() == RECON_LINEAR) {
+    const T sq3 = T(1.7320508075688772);
+    const T s13 = f1 + f3, s04 = f0 + f4, d04 = f0 - f4, d31 = f3 - f1;
+    const T E = T(719) / T(720) * f2 + (s13 * (T(1) / T(1080)) - s04 * (T(1) / T(4320)));
+    const T O = d04 * (sq3 * T(7) / T(432)) + d31 * (sq3 * T(25) / T(216));
+    const T A = d04 * (T(1) / T(12)) + d31 * (T(2) / T(3));
+    const T B = s13 * (sq3 * T(13) / T(54)) - (f2 * (sq3 * T(24) / T(54)) + s04 * (sq3 / T(54)));
+    v[0] = E - O;
+    v[1] = E + O;
+    d[0] = A - B;
+    d[1] = A + B;
+  } else {
+    tangential<MODE>(f0, f1, f2, f3, f4, v, d);
+  }
 }
 
 // Tangential reconstruction of a 5-vector field (components at src + i*sc,
@@ -170,10 +161,10 @@ __device__ __forceinline__ void t2_group(const T* tb, int s, int m1, int at3, in
       const T* a = sv + 4 * i * NH;
       const T* c = sdv + 4 * i * NH;
       const T* e = ss + 2 * i * NH;
-      T v[2], dd[2], vd[2], vs[2];
-      tangential<MODE>(a[-2 * st2], a[-st2], a[0], a[st2], a[2 * st2], v, dd);
-      tangential_val<MODE>(c[-2 * st2], c[-st2], c[0], c[st2], c[2 * st2], vd);
-      tangential_val<MODE>(e[-2 * st2], e[-st2], e[0], e[st2], e[2 * st2], vs);
+      T v[2], dd[2], vd[2], vs[2], unused[2];
+      tangential_fast<MODE>(a[-2 * st2], a[-st2], a[0], a[st2], a[2 * st2], v, dd);
+      tangential_fast<MODE>(c[-2 * st2], c[-st2], c[0], c[st2], c[2 * st2], vd, unused);
+      tangential_fast<MODE>(e[-2 * st2], e[-st2], e[0], e[st2], e[2 * st2], vs, unused);
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         val[m][i] = v[m];
@@ -272,53 +263,6 @@ HGKS_HD void face_fields_cells(const T qa[5][6], T hl, T hr, const Gas<T>& gas,
   }
 }
 
-// Face fields of the x sweep (conservative variables) for the layers
-// fb .. fb+nl-1 at transverse point (Pc, Sc): one thread reads the nl+5 cells
-// fb-3 .. fb+nl+1 along x of each variable, contiguous in memory, as pairs
-// (two-element vector loads; the caller guarantees an even padded row length,
-// so that with fb even every pair is aligned), and forms the fields of each
-// layer l into ffb + l * NFF * NH.
-template <class T, int MODE, int FLUX, int NH, int NL, int NFF>
-__device__ __forceinline__ void face_fields_x_item(const T* __restrict__ q, const GridDev& g,
-                                                   const SweepAxes& ax, const T* __restrict__ wn,
-                                                   const Gas<T>& gas, int fb, int nl, int Pc, int Sc,
-                                                   int h, T* ffb) {
-  using V2 = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
-  constexpr int NC = NL + 5;  // cells of NL layers
-  const long long cb = pad_index(g, fb - 3, ax.P == 1 ? Pc : Sc, ax.P == 1 ? Sc : Pc);
-  T cells[5][NC + 1];
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const T* qv = q + ax.gv[i] * g.P + cb;
-#pragma unroll
-    for (int j = 0; j < (NC + 1) / 2; ++j) {
-      if (2 * j + 1 < nl + 5) {
-        const V2 v = __ldg(reinterpret_cast<const V2*>(qv + 2 * j));
-        cells[i][2 * j] = v.x;
-        cells[i][2 * j + 1] = v.y;
-      } else if (2 * j < nl + 5) {
-        cells[i][2 * j] = __ldg(qv + 2 * j);
-        cells[i][2 * j + 1] = T(0);
-      } else {
-        cells[i][2 * j] = cells[i][2 * j + 1] = T(0);
-      }
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    if (l < nl) {
-      T qa[5][6];
-#pragma unroll
-      for (int i = 0; i < 5; ++i)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) qa[i][k] = cells[i][l + k];
-      const int f = fb + l;
-      face_fields_cells<T, MODE, FLUX, NH>(qa, wn[f - 1 + kGhost], wn[f + kGhost], gas, h,
-                                           ffb + l * NFF * NH);
-    }
-  }
-}
-
 // Face fields of face layer f at transverse point (Pc, Sc) into ff[k * NH + h]:
 // WENO5 end values of cells f-1 and f, their normal slopes, the compatibility
 // state Q0 and its normal slope (local frame).  Smooth flux: fields Q0, dQ0/dn;
@@ -397,63 +341,6 @@ __device__ __forceinline__ void face_fields_item(const T* __restrict__ q, const 
         ff[(25 + i) * NH + h] = D0[i];
       }
     }
-  }
-}
-
-// Tangential pass along t1 for one point `at` of the tile (stride st1 in the
-// shared-memory plane): values at both t1 Gauss abscissae of every field and
-// t1-derivatives of the state fields, into tb.
-template <class T, int MODE, int FLUX, int NH>
-__device__ __forceinline__ void t1_pass_item(const T* ff, T* tb, int at, int st1, const Gas<T>& gas) {
-  constexpr int NV = SweepLayout<FLUX>::NV;
-  if constexpr (is_char_mode<MODE>()) {
-    // Characteristic variables of Qm at the centre point.
-    T qm[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) qm[i] = ff[(SweepLayout<FLUX, MODE>::QM + i) * NH + at];
-    const CharBasis<T> b = char_basis(qm, gas);
-#pragma unroll 1
-    for (int grp = 0; grp < 2 * NV / 5; ++grp) {
-      // groups 0 .. NV/5-1: state fields (values and t1-derivatives);
-      // then their normal slopes (values only)
-      const bool state = grp < NV / 5;
-      const int k0 = 5 * grp;  // first field of the group in ff
-      T v[2][5], d[2][5];
-      tangential_char<MODE>(ff + k0 * NH + at, NH, st1, b, v, d);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        if (state) {
-          const int k = k0 + i;
-          tb[(4 * k + 0) * NH + at] = v[0][i];
-          tb[(4 * k + 1) * NH + at] = v[1][i];
-          tb[(4 * k + 2) * NH + at] = d[0][i];
-          tb[(4 * k + 3) * NH + at] = d[1][i];
-        } else {
-          const int k = k0 - NV + i;
-          tb[(4 * NV + 2 * k + 0) * NH + at] = v[0][i];
-          tb[(4 * NV + 2 * k + 1) * NH + at] = v[1][i];
-        }
-      }
-    }
-  } else {
-#pragma unroll(FLUX == FLUX_SMOOTH ? 5 : 1)
-  for (int k = 0; k < NV; ++k) {
-    const T* src = ff + k * NH + at;
-    T v[2], dd[2];
-    tangential<MODE>(src[-2 * st1], src[-st1], src[0], src[st1], src[2 * st1], v, dd);
-    tb[(4 * k + 0) * NH + at] = v[0];
-    tb[(4 * k + 1) * NH + at] = v[1];
-    tb[(4 * k + 2) * NH + at] = dd[0];
-    tb[(4 * k + 3) * NH + at] = dd[1];
-  }
-#pragma unroll(FLUX == FLUX_SMOOTH ? 5 : 1)
-  for (int k = 0; k < NV; ++k) {
-    const T* src = ff + (NV + k) * NH + at;
-    T v[2];
-    tangential_val<MODE>(src[-2 * st1], src[-st1], src[0], src[st1], src[2 * st1], v);
-    tb[(4 * NV + 2 * k + 0) * NH + at] = v[0];
-    tb[(4 * NV + 2 * k + 1) * NH + at] = v[1];
-  }
   }
 }
 
@@ -537,21 +424,6 @@ __device__ __forceinline__ void t1_pass_group_wx2(const float* ff, float* tb, in
       tb[(4 * NV + 2 * j + 1) * NH + at] = v[1];
     }
   }
-}
-
-// Resident CTAs per SM the register budget is sized for: three in FP32 (two
-// in the characteristic modes, which need more registers), two in FP64.
-template <class T, int MODE>
-__host__ __device__ constexpr int sweep_min_blocks() {
-  return sizeof(T) == 4 && !is_char_mode<MODE>() ? 3 : 2;
-}
-
-template <class T, int MODE, int STAGE, int TP, int TS, int NL>
-__global__ void __launch_bounds__(sweep_threads(TP, TS), (sweep_min_blocks<T, MODE>()))
-    k_sweep(const __grid_constant__ SweepArgs3<T> sweeps) {
-#define HGKS_SW_B blockIdx.x
-#include "sweep_body.inc"
-#undef HGKS_SW_B
 }
 
 }  // namespace hgks

@@ -1,46 +1,51 @@
-// Fused sweep for the full flux (Eq. (5)): face fields, tangential passes and
-// flux of a TP x TS tile of faces marching through a chunk of face layers,
-// like sweep.cuh, with the tangential passes and the flux taken one STATE
-// GROUP (Q_l, Q_r, Q_0, five fields and five slopes each) at a time.
+// Fused sweep kernel: for one S2O4 stage, the face fields, the tangential
+// reconstruction to the 2x2 Gauss points and the BGK flux there, for a TP x TS
+// tile of faces (P the faster-varying transverse axis in memory, S the slower
+// one) marching through a chunk of face layers along the normal (face f lies
+// between cells f-1 and f).  (FP32 with linear weights and the smooth flux:
+// march.cuh.)
 //
 // Per face layer:
-//   phase 1  the 30 face fields at the tile's points plus a halo of 2;
-//   then for s = l, r, 0:
-//   phase 2  the pass along t1 of group s (30 values per point);
+//   phase 1  one thread per point of the tile plus a halo of 2: the six cells
+//            f-3..f+2 along d, WENO5 end values of cells f-1 and f, the normal
+//            slopes, the compatibility state Q0 and its normal slope;
+//   then for each STATE GROUP s of five fields and five slopes (smooth flux:
+//   Q_0; full flux: Q_l, Q_r, Q_0 one after the other):
+//   phase 2  the pass along t1 = d+1 (30 values per point, halo 2 along t2);
 //   phase 3  two threads per face, thread m1 for the t1 abscissa m1: the pass
-//            along t2 gives both t2 abscissae; s = l, r add their half-space
-//            moments to the Gauss points' sums, s = 0 closes the flux.
+//            along t2 = d+2 gives both t2 abscissae; Q_l, Q_r add their
+//            half-space moments to the Gauss points' sums, Q_0 closes the flux.
 // A group's values of the second t2 abscissa and the half-space sums wait in
 // the thread's own slots of shared memory.
 //
-// Why by groups: all three at once need 90 planes of t1-pass values and three
-// point states in registers (FP32: 210 KB and 246 registers, 8 warps per SM,
-// FMA pipe 54 % active).  One group needs 30 planes and one point state: 111 KB
-// and 128 registers without spills, 16 warps per SM in two CTAs whose phases
-// overlap.  In FP64 the tile grows from 8 x 8 to 16 x 8 (face fields at 1.9
-// points per face instead of 2.25), and every reconstruction of the pass along
-// t2 serves both abscissae (four threads per face made each of them twice).
-// Measured (GB300, one step): FP32 WENO-Z 256^3 73.4 -> 59.9 ms (56.3 with the
-// strides as constants and shorter chunks); in characteristic variables
-// 90x75x67 2.59 -> 2.24 ms; eight boxes of 32^3 to 96^3 11.4 -> 8.92 ms; FP64
-// WENO-Z 64^3 71.1 -> 46.0 ms.
-// Bound by the FMA pipe and the reciprocal unit (FP32), the FP64 pipe (FP64).
+// Why by groups: the full flux's three at once need 90 planes of t1-pass values
+// and three point states in registers (FP32: 210 KB and 246 registers, 8 warps
+// per SM, FMA pipe 54 % active).  One group needs 30 planes and one point
+// state: 111 KB and 128 registers without spills, 16 warps per SM in two CTAs
+// whose phases overlap.  In FP64 the tile grows from 8 x 8 to 16 x 8 (face
+// fields at 1.9 points per face instead of 2.25), and every reconstruction of
+// the pass along t2 serves both abscissae.
+// Measured (GB300, one step): FP32 WENO-Z + full flux 256^3 73.4 -> 59.9 ms
+// (56.3 with the strides as constants and shorter chunks); in characteristic
+// variables 90x75x67 2.59 -> 2.24 ms; eight boxes of 32^3 to 96^3 11.4 -> 8.92
+// ms; FP64 WENO-Z + full flux 64^3 71.1 -> 46.0 ms.
+// Bound by the FMA pipe and instruction issue (FP32), the FP64 pipe (FP64).
 #pragma once
 
 #include "sweep.cuh"
 
 namespace hgks {
 
-template <class T, int MODE, int TP, int TS>
-struct FullSweep {
+template <class T, int MODE, int FLUX, int TP, int TS>
+struct SweepShape {
   static constexpr int HP = TP + 4, HS = TS + 4, NH = HP * HS;
-  static constexpr int NV = 15, NFF = SweepLayout<FLUX_FULL, MODE>::NFF, NT1 = 30;
+  static constexpr int NV = FLUX == FLUX_FULL ? 15 : 5, NFF = SweepLayout<FLUX, MODE>::NFF, NT1 = 30;
   static constexpr int THREADS = 2 * TP * TS;
-  // Slots per thread: the point state of the second t2 abscissa, then per t2
-  // abscissa the half-space sums (15) and the pressure term of tau.
-  static constexpr int ST = 20, SUMS = 16, SLOTS = ST + 2 * SUMS;
+  // Slots per thread: the point state of the second t2 abscissa, then (full
+  // flux) per t2 abscissa the half-space sums (15) and the pressure term of tau.
+  static constexpr int ST = 20, SUMS = FLUX == FLUX_FULL ? 16 : 0, SLOTS = ST + 2 * SUMS;
   static constexpr size_t SMEM = sizeof(T) * ((NFF + NT1) * NH + SLOTS * THREADS);
-  static constexpr int MIN_BLOCKS = sizeof(T) == 4 ? 2 : 1;
+  static constexpr int MIN_BLOCKS = sizeof(T) == 8 ? 1 : (FLUX == FLUX_FULL || is_char_mode<MODE>() ? 2 : 3);
   static_assert(TP == 16, "a warp holds one row of 16 faces and both t1 abscissae");
 };
 
@@ -69,8 +74,8 @@ __device__ __forceinline__ void t1_pass_unit(const T* ff, T* tb, int s, int at, 
       db[m] = d[m].y;
     }
   } else {
-    tangential<MODE>(sa[-2 * st1], sa[-st1], sa[0], sa[st1], sa[2 * st1], va, da);
-    tangential<MODE>(sb[-2 * st1], sb[-st1], sb[0], sb[st1], sb[2 * st1], vb, db);
+    tangential_fast<MODE>(sa[-2 * st1], sa[-st1], sa[0], sa[st1], sa[2 * st1], va, da);
+    tangential_fast<MODE>(sb[-2 * st1], sb[-st1], sb[0], sb[st1], sb[2 * st1], vb, db);
   }
   oa[0] = va[0];
   oa[NH] = va[1];
@@ -113,7 +118,7 @@ __device__ __forceinline__ void t1_pass_char(const T* ff, T* tb, int s, bool slo
 // first t2 abscissa in g0, that of the second in the slots (component c of
 // value, n, t1, t2 derivative: slot 5 c + i).
 template <class T, int MODE, int NH, int NT>
-__device__ __forceinline__ void t2_pass_full(const T* tb, int m1, int at, int st2, const CharBasis<T>& cbs, T rh1,
+__device__ __forceinline__ void t2_pass(const T* tb, int m1, int at, int st2, const CharBasis<T>& cbs, T rh1,
                                              T rh2, PointState<T>& g0, T* slot) {
   if constexpr (std::is_same<T, float>::value && recon_of<MODE>() != RECON_LINEAR && !is_char_mode<MODE>()) {
     // Two reconstructions per packed evaluation: each component's
@@ -175,9 +180,9 @@ __device__ __forceinline__ void t2_pass_full(const T* tb, int m1, int at, int st
 
 // One tile's chunk.  t1 runs along P (the x and z sweeps) or along S, as a
 // compile-time choice: the strides of both passes are then constants.
-template <class T, int MODE, int STAGE, int TP, int TS, bool T1P>
-__device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, int by, int bz) {
-  using L = FullSweep<T, MODE, TP, TS>;
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS, bool T1P>
+__device__ __forceinline__ void sweep_tile(const SweepArgs<T>& a, int bx, int by, int bz) {
+  using L = SweepShape<T, MODE, FLUX, TP, TS>;
   constexpr int HP = L::HP, HS = L::HS, NH = L::NH, NV = L::NV, NT = L::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ff = reinterpret_cast<T*>(smem_raw);  // [NFF][NH]
@@ -225,7 +230,7 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
     for (int h = tid; h < NH; h += NT) {
       const int Pc = p0 - 2 + h % HP, Sc = s0 - 2 + h / HP;
       if (Pc <= nP + 1 && Sc <= nS + 1) {
-        face_fields_item<T, MODE, FLUX_FULL, NH>(a.q, a.g, ax, a.wn, a.gas, f, Pc, Sc, h, ff);
+        face_fields_item<T, MODE, FLUX, NH>(a.q, a.g, ax, a.wn, a.gas, f, Pc, Sc, h, ff);
       } else {
 #pragma unroll 1
         for (int k = 0; k < L::NFF; ++k) ff[k * NH + h] = T(0);
@@ -234,7 +239,7 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
     __syncthreads();
 
 #pragma unroll 1
-    for (int s = 0; s < 3; ++s) {
+    for (int s = 0; s < NV / 5; ++s) {
       // ---------------- phase 2: pass along t1 of group s ----------------
       // Points of the tile with a halo of 2 along t2.
       constexpr int items = T1P ? TP * HS : HP * TS;
@@ -258,7 +263,7 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
           cbs = char_basis(qm, a.gas);
         }
         PointState<T> st;
-        t2_pass_full<T, MODE, NH, NT>(tb, m1, at3, st2, cbs, rh1, rh2, st, slot);
+        t2_pass<T, MODE, NH, NT>(tb, m1, at3, st2, cbs, rh1, rh2, st, slot);
         T Fs[10];
 #pragma unroll
         for (int i = 0; i < 10; ++i) Fs[i] = T(0);
@@ -274,7 +279,15 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
             }
           }
           T* sum = slot + (L::ST + m2 * L::SUMS) * NT;
-          if (s < 2) {
+          if constexpr (FLUX == FLUX_SMOOTH) {
+            T F[5], dF[5];
+            flux_smooth(st, a.gas, STAGE == 1, F, dF);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+              if (STAGE == 1) Fs[i] += F[i];
+              Fs[5 + i] += dF[i];
+            }
+          } else if (s < 2) {
             FullSide<T> h;
             flux_full_side(st, a.gas, s, h);
             if (s == 0) {
@@ -300,7 +313,7 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
             }
           }
         }
-        if (s == 2) {
+        if (s == NV / 5 - 1) {
           const long long o = fout + (long long)f * fstep;
 #pragma unroll
           for (int i = 0; i < 5; ++i) {
@@ -317,24 +330,24 @@ __device__ __forceinline__ void sweep_full_tile(const SweepArgs<T>& a, int bx, i
       }
       // The next group's t1 pass overwrites tb; the next layer's face fields
       // overwrite ff, whose Qm planes phase 3 reads in the characteristic modes.
-      if (s < 2 || is_char_mode<MODE>()) __syncthreads();
+      if (s < NV / 5 - 1 || is_char_mode<MODE>()) __syncthreads();
     }
   }
 }
 
 // Body of one block: `sweeps` the arguments, b the block.
-template <class T, int MODE, int STAGE, int TP, int TS>
-__device__ __forceinline__ void sweep_full_block(const SweepArgs3<T>& sweeps, int b) {
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS>
+__device__ __forceinline__ void sweep_block(const SweepArgs3<T>& sweeps, int b) {
   int bx, by, bz;
   const SweepArgs<T> a = sweep_of_block(sweeps, b, bx, by, bz);
-  if (a.d == 1) sweep_full_tile<T, MODE, STAGE, TP, TS, false>(a, bx, by, bz);
-  else sweep_full_tile<T, MODE, STAGE, TP, TS, true>(a, bx, by, bz);
+  if (a.d == 1) sweep_tile<T, MODE, FLUX, STAGE, TP, TS, false>(a, bx, by, bz);
+  else sweep_tile<T, MODE, FLUX, STAGE, TP, TS, true>(a, bx, by, bz);
 }
 
-template <class T, int MODE, int STAGE, int TP, int TS>
-__global__ void __launch_bounds__(FullSweep<T, MODE, TP, TS>::THREADS, (FullSweep<T, MODE, TP, TS>::MIN_BLOCKS))
-    k_sweep_full(const __grid_constant__ SweepArgs3<T> sweeps) {
-  sweep_full_block<T, MODE, STAGE, TP, TS>(sweeps, blockIdx.x);
+template <class T, int MODE, int FLUX, int STAGE, int TP, int TS>
+__global__ void __launch_bounds__(SweepShape<T, MODE, FLUX, TP, TS>::THREADS, (SweepShape<T, MODE, FLUX, TP, TS>::MIN_BLOCKS))
+    k_sweep(const __grid_constant__ SweepArgs3<T> sweeps) {
+  sweep_block<T, MODE, FLUX, STAGE, TP, TS>(sweeps, blockIdx.x);
 }
 
 }  // namespace hgks

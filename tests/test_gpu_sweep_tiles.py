@@ -1,6 +1,6 @@
 """Sweep kernels at the edges of their tiles against the FP64 oracle.
 
-Grids one face past a tile (16 x 8 faces of k_sweep and k_sweep_full, 32 faces
+Grids one face past a tile (16 x 8 faces of k_sweep, 16 x 16 in FP64 with the smooth flux; 32 faces
 by 10 layers of k_march), exactly one tile, the smallest grid the library
 takes, and a walled direction, whose face n is a face of its own (in periodic
 directions it is a copy of face 0).  Bounds as elsewhere: 1e-12 in FP64; 2e-5
