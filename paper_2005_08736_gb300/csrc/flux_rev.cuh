@@ -57,59 +57,6 @@ HGKS_HD void prim_of_rev(const T q[5], const Prim<T>& s, const Gas<T>& g, PrimBa
   qb[0] += b.rho;
 }
 
-// slope_solve transposed: a = slope_solve(s, b); given ab (cotangent of a)
-// adds to sb (the state's fields) and bb (cotangent of b).
-template <class T>
-HGKS_HD void slope_solve_rev(const Prim<T>& s, const Gas<T>& g, const T b[5], const T ab[5],
-                             PrimBar<T>& sb, T bb[5]) {
-  const T U = s.U, V = s.V, W = s.W;
-  const T q2 = U * U + V * V + W * W;
-  const T k3t = (g.K + T(3)) * s.theta;
-  const T l2 = T(2) * s.lam;
-  const T c4 = l2 * l2 / (g.K + T(3));
-  const T t = T(2) * (b[4] - U * b[1] - V * b[2] - W * b[3]) + (q2 - k3t) * b[0];
-  const T a4 = c4 * t;
-  const T a3 = l2 * (b[3] - W * b[0]) - W * a4;
-  const T a2 = l2 * (b[2] - V * b[0]) - V * a4;
-  const T a1 = l2 * (b[1] - U * b[0]) - U * a4;
-  // a0 = b0 - U a1 - V a2 - W a3 - a4 (q2 + k3t)/2
-  T a1b = ab[1] - ab[0] * U, a2b = ab[2] - ab[0] * V, a3b = ab[3] - ab[0] * W;
-  T a4b = ab[4] - T(0.5) * ab[0] * (q2 + k3t);
-  T Ub = -ab[0] * a1, Vb = -ab[0] * a2, Wb = -ab[0] * a3;
-  T q2b = -T(0.5) * ab[0] * a4, k3tb = -T(0.5) * ab[0] * a4;
-  bb[0] += ab[0];
-  // a_i = l2 (b_i - U_i b0) - U_i a4, i = 1, 2, 3
-  T l2b = a1b * (b[1] - U * b[0]) + a2b * (b[2] - V * b[0]) + a3b * (b[3] - W * b[0]);
-  bb[1] += a1b * l2;
-  bb[2] += a2b * l2;
-  bb[3] += a3b * l2;
-  bb[0] += -l2 * (a1b * U + a2b * V + a3b * W);
-  Ub += -a1b * (l2 * b[0] + a4);
-  Vb += -a2b * (l2 * b[0] + a4);
-  Wb += -a3b * (l2 * b[0] + a4);
-  a4b += -(a1b * U + a2b * V + a3b * W);
-  // a4 = c4 t
-  const T c4b = a4b * t, tb = a4b * c4;
-  // t = 2 (b4 - U b1 - V b2 - W b3) + (q2 - k3t) b0
-  bb[4] += T(2) * tb;
-  bb[1] += -T(2) * tb * U;
-  bb[2] += -T(2) * tb * V;
-  bb[3] += -T(2) * tb * W;
-  bb[0] += tb * (q2 - k3t);
-  Ub += -T(2) * tb * b[1];
-  Vb += -T(2) * tb * b[2];
-  Wb += -T(2) * tb * b[3];
-  q2b += tb * b[0];
-  k3tb += -tb * b[0];
-  // c4 = l2^2/(K+3), l2 = 2 lam, k3t = (K+3) theta, q2 = |U|^2
-  l2b += c4b * T(2) * l2 / (g.K + T(3));
-  sb.lam += T(2) * l2b;
-  sb.theta += (g.K + T(3)) * k3tb;
-  sb.U += Ub + T(2) * U * q2b;
-  sb.V += Vb + T(2) * V * q2b;
-  sb.W += Wb + T(2) * W * q2b;
-}
-
 // euler_jvp<J> transposed in the state (dQ held fixed): out = J_J(Q) dQ;
 // given ob adds to sb and Hb.
 template <int J, class T>
@@ -155,110 +102,6 @@ HGKS_HD void euler_jvp_rev_state(const Prim<T>& s, T H, const T dQ[5], const Gas
   sb.W += Ub[2];
 }
 
-// Cotangents of the normalised moments of Mom.
-template <class T>
-struct MomBar {
-  T u[7], v[7], w[7];
-  T xi1, xi2;
-};
-
-template <int A, int B, int C, class T>
-HGKS_HD void mm_rev(const Mom<T>& m, T bar, MomBar<T>& mb) {
-  mb.u[A] += bar * m.v[B] * m.w[C];
-  mb.v[B] += bar * m.u[A] * m.w[C];
-  mb.w[C] += bar * m.u[A] * m.v[B];
-}
-
-// mom_psipsi<A,B,C> transposed: Mb (cotangents of the 15 entries) into mb.
-template <int A, int B, int C, class T>
-HGKS_HD void mom_psipsi_rev(const Mom<T>& m, const T Mb[15], MomBar<T>& mb) {
-  const T x1 = m.xi1, x2 = m.xi2;
-  const T m0 = mm<A, B, C>(m);
-  const T mu1 = mm<A + 1, B, C>(m), mv1 = mm<A, B + 1, C>(m), mw1 = mm<A, B, C + 1>(m);
-  const T mu2 = mm<A + 2, B, C>(m), mv2 = mm<A, B + 2, C>(m), mw2 = mm<A, B, C + 2>(m);
-  T m0b = Mb[0], mu1b = Mb[1], mv1b = Mb[2], mw1b = Mb[3];
-  T mu2b = Mb[5], mv2b = Mb[9], mw2b = Mb[12];
-  T x1b = T(0), x2b = T(0);
-  // M[4] = (mu2 + mv2 + mw2 + m0 x1)/2
-  {
-    const T h = T(0.5) * Mb[4];
-    mu2b += h;
-    mv2b += h;
-    mw2b += h;
-    m0b += h * x1;
-    x1b += h * m0;
-  }
-  mm_rev<A + 1, B + 1, C>(m, Mb[6], mb);
-  mm_rev<A + 1, B, C + 1>(m, Mb[7], mb);
-  // M[8] = (u^3 + u v^2 + u w^2 + mu1 x1)/2
-  {
-    const T h = T(0.5) * Mb[8];
-    mm_rev<A + 3, B, C>(m, h, mb);
-    mm_rev<A + 1, B + 2, C>(m, h, mb);
-    mm_rev<A + 1, B, C + 2>(m, h, mb);
-    mu1b += h * x1;
-    x1b += h * mu1;
-  }
-  mm_rev<A, B + 1, C + 1>(m, Mb[10], mb);
-  {
-    const T h = T(0.5) * Mb[11];
-    mm_rev<A + 2, B + 1, C>(m, h, mb);
-    mm_rev<A, B + 3, C>(m, h, mb);
-    mm_rev<A, B + 1, C + 2>(m, h, mb);
-    mv1b += h * x1;
-    x1b += h * mv1;
-  }
-  {
-    const T h = T(0.5) * Mb[13];
-    mm_rev<A + 2, B, C + 1>(m, h, mb);
-    mm_rev<A, B + 2, C + 1>(m, h, mb);
-    mm_rev<A, B, C + 3>(m, h, mb);
-    mw1b += h * x1;
-    x1b += h * mw1;
-  }
-  // M[14] = (u4 + v4 + w4 + 2(u2v2 + u2w2 + v2w2) + 2 x1 (mu2 + mv2 + mw2) + x2 m0)/4
-  {
-    const T h = T(0.25) * Mb[14];
-    mm_rev<A + 4, B, C>(m, h, mb);
-    mm_rev<A, B + 4, C>(m, h, mb);
-    mm_rev<A, B, C + 4>(m, h, mb);
-    mm_rev<A + 2, B + 2, C>(m, T(2) * h, mb);
-    mm_rev<A + 2, B, C + 2>(m, T(2) * h, mb);
-    mm_rev<A, B + 2, C + 2>(m, T(2) * h, mb);
-    x1b += T(2) * h * (mu2 + mv2 + mw2);
-    mu2b += T(2) * h * x1;
-    mv2b += T(2) * h * x1;
-    mw2b += T(2) * h * x1;
-    x2b += h * m0;
-    m0b += h * x2;
-  }
-  mm_rev<A, B, C>(m, m0b, mb);
-  mm_rev<A + 1, B, C>(m, mu1b, mb);
-  mm_rev<A, B + 1, C>(m, mv1b, mb);
-  mm_rev<A, B, C + 1>(m, mw1b, mb);
-  mm_rev<A + 2, B, C>(m, mu2b, mb);
-  mm_rev<A, B + 2, C>(m, mv2b, mb);
-  mm_rev<A, B, C + 2>(m, mw2b, mb);
-  mb.xi1 += x1b;
-  mb.xi2 += x2b;
-}
-
-// out = M a (sym5_matvec_add) transposed: adds the cotangents of the 15
-// stored entries of the symmetric M and of a, given ob.
-template <class T>
-HGKS_HD void sym5_matvec_rev(const T M[15], const T a[5], const T ob[5], T Mb[15], T ab[5]) {
-  // index of the stored entry (i <= j)
-  constexpr int idx[5][5] = {{0, 1, 2, 3, 4}, {1, 5, 6, 7, 8}, {2, 6, 9, 10, 11}, {3, 7, 10, 12, 13},
-                             {4, 8, 11, 13, 14}};
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      Mb[idx[i][j]] += ob[i] * a[j];
-      ab[j] += ob[i] * M[idx[i][j]];
-    }
-}
-
 // gauss_recursion transposed (m[n+2] = U m[n+1] + (n+1) theta m[n]).
 template <class T>
 HGKS_HD void gauss_recursion_rev(const T* m, T U, T theta, T* mb, T& Ub, T& thb) {
@@ -270,37 +113,6 @@ HGKS_HD void gauss_recursion_rev(const T* m, T U, T theta, T* mb, T& Ub, T& thb)
     thb += b * T(n + 1) * m[n];
     mb[n] += b * T(n + 1) * theta;
   }
-}
-
-// moments(s, half = +-1) transposed into sb.
-template <class T>
-HGKS_HD void moments_rev(const Prim<T>& s, const Gas<T>& g, int half, const Mom<T>& m, MomBar<T> mb,
-                         PrimBar<T>& sb) {
-  sb.theta += mb.xi1 * g.K + mb.xi2 * g.K * (g.K + T(2)) * T(2) * s.theta;
-  T Ub = T(0), Vb = T(0), Wb = T(0), thb = T(0);
-  gauss_recursion_rev(m.w, s.W, s.theta, mb.w, Wb, thb);
-  Wb += mb.w[1];
-  gauss_recursion_rev(m.v, s.V, s.theta, mb.v, Vb, thb);
-  Vb += mb.v[1];
-  gauss_recursion_rev(m.u, s.U, s.theta, mb.u, Ub, thb);
-  // half line: u0 = (1 + sg erf(x))/2, u1 = U u0 + sg e,
-  // x = sqrt(lam) U, e = exp(-x^2) / (2 sqrt(pi) sqrt(lam))
-  const T sl = tsqrt(s.lam);
-  const T x = sl * s.U;
-  const T ex = texp(-x * x);
-  const T e = ex * T(0.28209479177387814) / sl;
-  const T sg = T(half);
-  Ub += mb.u[1] * m.u[0];
-  T u0b = mb.u[0] + mb.u[1] * s.U;
-  const T eb = mb.u[1] * sg;
-  T xb = eb * e * (-T(2) * x) + u0b * T(0.5) * sg * T(1.1283791670955126) * ex;
-  T slb = -eb * e / sl + xb * s.U;
-  Ub += xb * sl;
-  sb.lam += slb * T(0.5) / sl;
-  sb.U += Ub;
-  sb.V += Vb;
-  sb.W += Wb;
-  sb.theta += thb;
 }
 
 // euler_jvp<J> transposed in dQ (the state held fixed): adds J_J(Q)^T ob to dQb.
@@ -341,142 +153,242 @@ HGKS_HD void euler_jvp_rev_dq(const Prim<T>& s, T H, const Gas<T>& g, const T ob
 // (flux_full_close), given the flux cotangents gF, gdF; added to cot.  The
 // weights are dual numbers carrying d/dtau; returns the part's share of
 // gF . dF/dtau + gdF . d(dF)/dtau.  The cotangent of its pressure (through
-// tau) is applied by pressure_viscosity_rev.  The four moment matrices are
-// formed one at a time, forward and again backward, to keep few values live.
+// tau) is applied by pressure_viscosity_rev.
+//
+// The transpose of flux_full_side line by line: in the frame of the
+// tangential velocity, with the slopes as primitive derivatives and the seven
+// distinct entries of each moment matrix (a prefix g marks a cotangent).  About
+// 700 operations; forming the four full moment matrices forward and again
+// backward took some 2800, in straight-line code that the instruction cache
+// did not hold (0.9 fetch stalls per issue).  FP32 64^3 WENO-JS, one adjoint
+// step: 7.89 -> 6.30 ms.
 template <class T>
 HGKS_HD T flux_full_side_rev(const PointState<T>& st, const Gas<T>& g, int side, const T gF[5],
                              const T gdF[5], const Dual<T> Fq[3], const Dual<T> dFq[3], PointState<T>& cot) {
+  // ---- forward (flux_full_side) ----
   const Prim<T> s = prim_of(st.q, g);
-  const T inv = s.inv_rho;
-  // forward: slopes a_d = slope_solve(s, dq_d inv), Q_t, A = slope_solve(s, Q_t inv)
-  T a[3][5];
+  const T inv = s.inv_rho, th = s.theta, U = s.U, V = s.V, W = s.W;
+  const T il = T(1) / th, il2 = il * il;
+  const T hk3 = T(0.5) * (g.K + T(3));
+  const T hv2 = T(0.5) * (V * V + W * W), hu2 = T(0.5) * U * U;
+  T r[3], du[3][3], pi[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    T bd[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) bd[i] = st.dq[d][i] * inv;
-    slope_solve(s, g, bd, a[d]);
+    r[d] = st.dq[d][0] * inv;
+    du[d][0] = st.dq[d][1] * inv - U * r[d];
+    du[d][1] = st.dq[d][2] * inv - V * r[d];
+    du[d][2] = st.dq[d][3] * inv - W * r[d];
+    pi[d] = g.gm1 * (st.dq[d][4] * inv - V * du[d][1] - W * du[d][2] - U * du[d][0] - (hv2 + hu2) * r[d]);
   }
-  const T H = g.h_r + st.q[4] + s.dp;
-  T Qt[5];
-  state_time_derivative(s, H, st.dq, g, Qt);
-  T bA[5], A[5];
+  auto slope = [&](const T dr, const T* dv, const T dpi, T* c) {
+    const T dth = dpi - th * dr;
+    const T c1 = dv[0] * il;
+    c[4] = dth * il2;
+    c[3] = dv[2] * il;
+    c[2] = dv[1] * il;
+    c[1] = c1 - U * c[4];
+    c[0] = dr - hk3 * (dth * il) - U * c1 + hu2 * c[4];
+  };
+  T a[3][5], A[5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) bA[i] = Qt[i] * inv;
-  slope_solve(s, g, bA, A);
-  const int half = side == 0 ? +1 : -1;
-  Mom<T> mh;
-  moments(s, g, half, mh);
-  // V0 = rho <u psi> (the first column of M1), V1 = rho ua, V2 = rho uA with
-  // M1 = <u psi psi^T>, uA = M1 A, ua = sum_d <u u_d psi psi^T> a_d.
-  T m1[5], ua[5] = {0, 0, 0, 0, 0}, uA[5] = {0, 0, 0, 0, 0};
+  for (int d = 0; d < 3; ++d) slope(r[d], du[d], pi[d], a[d]);
+  const T div = du[0][0] + du[1][1] + du[2][2];
+  const T rt = -(U * r[0] + V * r[1] + W * r[2] + div);
+  T ut[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) ut[i] = -(U * du[0][i] + V * du[1][i] + W * du[2][i] + pi[i]);
+  const T pt = -(U * pi[0] + V * pi[1] + W * pi[2] + g.gamma * th * div);
+  slope(rt, ut, pt, A);
+  const T R = tsqrt(th + th), iR = T(1) / R, x = U * iR;
+  const T e = texp(-x * x) * T(0.28209479177387814) * R;  // exp(-x^2) / (2 sqrt(pi lam))
+  const T sg = T(side == 0 ? 1 : -1);
+  const T half = T(0.5) * (T(1) + sg * terf(x));
+  T m[7];
+  m[0] = s.rho * half;
+  m[1] = U * m[0] + sg * (s.rho * e);
+  gauss_recursion(m, U, th);
+  const T c1 = (g.K + T(2)) * th, c2 = c1 * (c1 + T(2) * th);
+  const T P1 = T(0.5) * (m[3] + c1 * m[1]), P2 = T(0.5) * (m[4] + c1 * m[2]), P3 = T(0.5) * (m[5] + c1 * m[3]);
+  const T R1 = T(0.25) * (m[5] + T(2) * c1 * m[3] + c2 * m[1]);
+  const T R2 = T(0.25) * (m[6] + T(2) * c1 * m[4] + c2 * m[2]);
+  const T t1 = th * m[1], t2 = th * m[2];
+  const T B1 = T(0.5) * (th * m[3] + (c1 + T(2) * th) * t1);
+  T uA[5], ua[5], h[5];
+  uA[0] = m[1] * A[0] + m[2] * A[1] + P1 * A[4];
+  uA[1] = m[2] * A[0] + m[3] * A[1] + P2 * A[4];
+  uA[2] = t1 * A[2];
+  uA[3] = t1 * A[3];
+  uA[4] = P1 * A[0] + P2 * A[1] + R1 * A[4];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) h[i] = V * a[1][i] + W * a[2][i];
+  const T cross = a[1][2] + a[2][3], ah = a[0][0] + h[1];
+  ua[0] = m[2] * ah + m[3] * a[0][1] + P2 * a[0][4] + m[1] * h[0] + P1 * h[4] + t1 * cross;
+  ua[1] = m[3] * ah + m[4] * a[0][1] + P3 * a[0][4] + m[2] * h[0] + P2 * h[4] + t2 * cross;
+  ua[2] = t2 * (a[0][2] + a[1][1]) + t1 * (h[2] + a[1][0]) + B1 * a[1][4];
+  ua[3] = t2 * (a[0][3] + a[2][1]) + t1 * (h[3] + a[2][0]) + B1 * a[2][4];
+  ua[4] = P2 * ah + P3 * a[0][1] + R2 * a[0][4] + P1 * h[0] + R1 * h[4] + B1 * cross;
+
+  // ---- backward ----
+  // Back to the frame of the face: y = (x0, x1, x2 + V x0, x3 + W x0, x4 + V x2
+  // + W x3 + hv2 x0) for V0 (x = (m1, m2, 0, 0, P1)), V1 (ua) and V2 (uA).
+  T gU = T(0), gV, gW, ghv2, gth = T(0), phi;
+  T w0[5], z[5], y[5];  // cotangents of the three x
   {
-    T M[15];
-    mom_psipsi<1, 0, 0>(mh, M);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) m1[i] = M[i];
-    sym5_matvec_add(M, A, uA);
-  }
-  {
-    T M[15];
-    mom_psipsi<2, 0, 0>(mh, M);
-    sym5_matvec_add(M, a[0], ua);
-  }
-  {
-    T M[15];
-    mom_psipsi<1, 1, 0>(mh, M);
-    sym5_matvec_add(M, a[1], ua);
-  }
-  {
-    T M[15];
-    mom_psipsi<1, 0, 1>(mh, M);
-    sym5_matvec_add(M, a[2], ua);
-  }
-  // backward: the cotangents of V_k are gV_k = gF w_k + gdF dw_k
-  PrimBar<T> sb;
-  prim_bar_zero(sb);
-  T phi = T(0), uab[5], uAb[5], m1b[5];
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const T gv0 = gF[i] * Fq[0].v + gdF[i] * dFq[0].v, gt0 = gF[i] * Fq[0].d + gdF[i] * dFq[0].d;
-    const T gv1 = gF[i] * Fq[1].v + gdF[i] * dFq[1].v, gt1 = gF[i] * Fq[1].d + gdF[i] * dFq[1].d;
-    const T gv2 = gF[i] * Fq[2].v + gdF[i] * dFq[2].v, gt2 = gF[i] * Fq[2].d + gdF[i] * dFq[2].d;
-    phi += s.rho * (gt0 * m1[i] + gt1 * ua[i] + gt2 * uA[i]);
-    sb.rho += gv0 * m1[i] + gv1 * ua[i] + gv2 * uA[i];
-    m1b[i] = s.rho * gv0;
-    uab[i] = s.rho * gv1;
-    uAb[i] = s.rho * gv2;
-  }
-  MomBar<T> mb;
-#pragma unroll
-  for (int n = 0; n < 7; ++n) mb.u[n] = mb.v[n] = mb.w[n] = T(0);
-  mb.xi1 = mb.xi2 = T(0);
-  T Ab[5] = {0, 0, 0, 0, 0}, ab[3][5] = {{0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}};
-  {
-    T M[15], Mb[15];
-    mom_psipsi<1, 0, 0>(mh, M);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) Mb[k] = k < 5 ? m1b[k] : T(0);
-    sym5_matvec_rev(M, A, uAb, Mb, Ab);
-    mom_psipsi_rev<1, 0, 0>(mh, Mb, mb);
-  }
-  {
-    T M[15], Mb[15];
-    mom_psipsi<2, 0, 0>(mh, M);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) Mb[k] = T(0);
-    sym5_matvec_rev(M, a[0], uab, Mb, ab[0]);
-    mom_psipsi_rev<2, 0, 0>(mh, Mb, mb);
-  }
-  {
-    T M[15], Mb[15];
-    mom_psipsi<1, 1, 0>(mh, M);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) Mb[k] = T(0);
-    sym5_matvec_rev(M, a[1], uab, Mb, ab[1]);
-    mom_psipsi_rev<1, 1, 0>(mh, Mb, mb);
-  }
-  {
-    T M[15], Mb[15];
-    mom_psipsi<1, 0, 1>(mh, M);
-#pragma unroll
-    for (int k = 0; k < 15; ++k) Mb[k] = T(0);
-    sym5_matvec_rev(M, a[2], uab, Mb, ab[2]);
-    mom_psipsi_rev<1, 0, 1>(mh, Mb, mb);
-  }
-  moments_rev(s, g, half, mh, mb, sb);
-  // A = slope_solve(s, Q_t inv), Q_t = -sum_d J_d(Q) dq_d
-  T bAb[5] = {0, 0, 0, 0, 0};
-  slope_solve_rev(s, g, bA, Ab, sb, bAb);
-  T nQtb[5], Hb = T(0);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    nQtb[i] = -bAb[i] * inv;
-    sb.inv += bAb[i] * Qt[i];
-  }
-  // Q_t = -(J_0 dq_0 + J_1 dq_1 + J_2 dq_2): both the state and the slopes
-  euler_jvp_rev_state<0>(s, H, st.dq[0], g, nQtb, sb, Hb);
-  euler_jvp_rev_state<1>(s, H, st.dq[1], g, nQtb, sb, Hb);
-  euler_jvp_rev_state<2>(s, H, st.dq[2], g, nQtb, sb, Hb);
-  euler_jvp_rev_dq<0>(s, H, g, nQtb, cot.dq[0]);
-  euler_jvp_rev_dq<1>(s, H, g, nQtb, cot.dq[1]);
-  euler_jvp_rev_dq<2>(s, H, g, nQtb, cot.dq[2]);
-  // H = h_r + q4 + dp
-  cot.q[4] += Hb;
-  sb.dp += Hb;
-  // a_d = slope_solve(s, dq_d inv)
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    T bd[5], bdb[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) bd[i] = st.dq[d][i] * inv;
-    slope_solve_rev(s, g, bd, ab[d], sb, bdb);
+    const T GF[5] = {gF[0] + V * gF[2] + W * gF[3] + hv2 * gF[4], gF[1], gF[2] + V * gF[4], gF[3] + W * gF[4], gF[4]};
+    const T GD[5] = {gdF[0] + V * gdF[2] + W * gdF[3] + hv2 * gdF[4], gdF[1], gdF[2] + V * gdF[4],
+                     gdF[3] + W * gdF[4], gdF[4]};
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-      sb.inv += bdb[i] * st.dq[d][i];
-      cot.dq[d][i] += bdb[i] * inv;
+      w0[i] = GF[i] * Fq[0].v + GD[i] * dFq[0].v;
+      z[i] = GF[i] * Fq[1].v + GD[i] * dFq[1].v;
+      y[i] = GF[i] * Fq[2].v + GD[i] * dFq[2].v;
     }
+    auto dot = [](const T* p, const T* q) {
+      return p[0] * q[0] + p[1] * q[1] + p[2] * q[2] + p[3] * q[3] + p[4] * q[4];
+    };
+    phi = Fq[0].d * (GF[0] * m[1] + GF[1] * m[2] + GF[4] * P1) + dFq[0].d * (GD[0] * m[1] + GD[1] * m[2] + GD[4] * P1) +
+          Fq[1].d * dot(GF, ua) + dFq[1].d * dot(GD, ua) + Fq[2].d * dot(GF, uA) + dFq[2].d * dot(GD, uA);
+    const T S0 = Fq[0].v * m[1] + Fq[1].v * ua[0] + Fq[2].v * uA[0];
+    const T D0 = dFq[0].v * m[1] + dFq[1].v * ua[0] + dFq[2].v * uA[0];
+    const T S2 = Fq[1].v * ua[2] + Fq[2].v * uA[2], D2 = dFq[1].v * ua[2] + dFq[2].v * uA[2];
+    const T S3 = Fq[1].v * ua[3] + Fq[2].v * uA[3], D3 = dFq[1].v * ua[3] + dFq[2].v * uA[3];
+    gV = gF[2] * S0 + gF[4] * S2 + gdF[2] * D0 + gdF[4] * D2;
+    gW = gF[3] * S0 + gF[4] * S3 + gdF[3] * D0 + gdF[4] * D3;
+    ghv2 = gF[4] * S0 + gdF[4] * D0;
   }
+  // <u A psi'> and <u (a.u) psi'>
+  T gA[5], ga[3][5];
+  gA[0] = m[1] * y[0] + m[2] * y[1] + P1 * y[4];
+  gA[1] = m[2] * y[0] + m[3] * y[1] + P2 * y[4];
+  gA[2] = t1 * y[2];
+  gA[3] = t1 * y[3];
+  gA[4] = P1 * y[0] + P2 * y[1] + R1 * y[4];
+  const T gh0 = m[1] * z[0] + m[2] * z[1] + P1 * z[4], gh1 = m[2] * z[0] + m[3] * z[1] + P2 * z[4];
+  const T gh2 = t1 * z[2], gh3 = t1 * z[3], gh4 = P1 * z[0] + P2 * z[1] + R1 * z[4];
+  const T gcross = t1 * z[0] + t2 * z[1] + B1 * z[4];
+  ga[0][0] = gh1;
+  ga[0][1] = m[3] * z[0] + m[4] * z[1] + P3 * z[4];
+  ga[0][2] = t2 * z[2];
+  ga[0][3] = t2 * z[3];
+  ga[0][4] = P2 * z[0] + P3 * z[1] + R2 * z[4];
+  ga[1][0] = V * gh0 + gh2;
+  ga[1][1] = V * gh1 + t2 * z[2];
+  ga[1][2] = V * gh2 + gcross;
+  ga[1][3] = V * gh3;
+  ga[1][4] = V * gh4 + B1 * z[2];
+  ga[2][0] = W * gh0 + gh3;
+  ga[2][1] = W * gh1 + t2 * z[3];
+  ga[2][2] = W * gh2;
+  ga[2][3] = W * gh3 + gcross;
+  ga[2][4] = W * gh4 + B1 * z[3];
+  gV += a[1][0] * gh0 + a[1][1] * gh1 + a[1][2] * gh2 + a[1][3] * gh3 + a[1][4] * gh4;
+  gW += a[2][0] * gh0 + a[2][1] * gh1 + a[2][2] * gh2 + a[2][3] * gh3 + a[2][4] * gh4;
+  T gm[7];
+  gm[0] = T(0);
+  gm[1] = w0[0] + y[0] * A[0] + z[0] * h[0];
+  gm[2] = w0[1] + y[0] * A[1] + y[1] * A[0] + z[0] * ah + z[1] * h[0];
+  gm[3] = y[1] * A[1] + z[0] * a[0][1] + z[1] * ah;
+  gm[4] = z[1] * a[0][1];
+  const T gP1 = w0[4] + y[0] * A[4] + y[4] * A[0] + z[0] * h[4] + z[4] * h[0];
+  const T gP2 = y[1] * A[4] + y[4] * A[1] + z[0] * a[0][4] + z[1] * h[4] + z[4] * ah;
+  const T gP3 = z[1] * a[0][4] + z[4] * a[0][1];
+  const T gR1 = y[4] * A[4] + z[4] * h[4], gR2 = z[4] * a[0][4];
+  const T gB1 = z[2] * a[1][4] + z[3] * a[2][4] + z[4] * cross;
+  const T gt1 = y[2] * A[2] + y[3] * A[3] + z[0] * cross + z[2] * (h[2] + a[1][0]) + z[3] * (h[3] + a[2][0]) +
+                T(0.5) * gB1 * (c1 + T(2) * th);
+  const T gt2 = z[1] * cross + z[2] * (a[0][2] + a[1][1]) + z[3] * (a[0][3] + a[2][1]);
+  // the moments, from the combinations down the recursion
+  T gc1 = T(0.5) * (gB1 * t1 + gP1 * m[1] + gP2 * m[2] + gP3 * m[3] + gR1 * m[3] + gR2 * m[4]);
+  const T gc2 = T(0.25) * (gR1 * m[1] + gR2 * m[2]);
+  gm[1] += gt1 * th + T(0.5) * c1 * gP1 + T(0.25) * c2 * gR1;
+  gm[2] += gt2 * th + T(0.5) * c1 * gP2 + T(0.25) * c2 * gR2;
+  gm[3] += T(0.5) * (gB1 * th + gP1 + c1 * (gP3 + gR1));
+  gm[4] += T(0.5) * (gP2 + c1 * gR2);
+  gm[5] = T(0.5) * gP3 + T(0.25) * gR1;
+  gm[6] = T(0.25) * gR2;
+  gc1 += gc2 * T(2) * (c1 + th);
+  gth += T(0.5) * gB1 * (m[3] + T(2) * t1) + gt1 * m[1] + gt2 * m[2] + T(2) * c1 * gc2 + (g.K + T(2)) * gc1;
+  gauss_recursion_rev(m, U, th, gm, gU, gth);
+  PrimBar<T> sb;
+  prim_bar_zero(sb);
+  {
+    gU += gm[1] * m[0];
+    gm[0] += gm[1] * U;
+    sb.rho = sg * gm[1] * e + gm[0] * half;
+    const T ge = sg * gm[1] * s.rho, eR = e * iR;          // d erf/dx / 4 = e / R
+    const T gx = T(2) * (sg * gm[0] * s.rho * eR - ge * e * x);
+    gU += gx * iR;
+    gth += (ge * eR - gx * x * iR) * iR;
+  }
+  // the slopes
+  T gr[3] = {T(0), T(0), T(0)}, gdu[3][3], gpi[3], gil = T(0), gil2 = T(0), ghu2 = T(0);
+  auto slope_rev = [&](const T dr, const T* dv, const T dpi, const T* gc, T& gdr, T* gdv, T& gdpi) {
+    const T dth = dpi - th * dr, c4 = dth * il2;
+    const T gl = gc[1] - U * gc[0], g4 = gc[4] - U * gc[1] + hu2 * gc[0];
+    gU -= gc[1] * c4 + gc[0] * (dv[0] * il);
+    ghu2 += gc[0] * c4;
+    const T gdth = g4 * il2 - gc[0] * (hk3 * il);
+    gil += gl * dv[0] + gc[2] * dv[1] + gc[3] * dv[2] - gc[0] * (hk3 * dth);
+    gil2 += g4 * dth;
+    gdv[0] = gl * il;
+    gdv[1] = gc[2] * il;
+    gdv[2] = gc[3] * il;
+    gdpi = gdth;
+    gth -= gdth * dr;
+    gdr = gc[0] - gdth * th;
+  };
+#pragma unroll
+  for (int d = 0; d < 3; ++d) slope_rev(r[d], du[d], pi[d], ga[d], gr[d], gdu[d], gpi[d]);
+  {
+    T nr, nu[3], np;
+    slope_rev(rt, ut, pt, gA, nr, nu, np);
+    nr = -nr;
+    np = -np;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      nu[i] = -nu[i];
+      gpi[i] += nu[i];
+      gdu[0][i] += nu[i] * U;
+      gdu[1][i] += nu[i] * V;
+      gdu[2][i] += nu[i] * W;
+    }
+    gU += nr * r[0] + nu[0] * du[0][0] + nu[1] * du[0][1] + nu[2] * du[0][2] + np * pi[0];
+    gV += nr * r[1] + nu[0] * du[1][0] + nu[1] * du[1][1] + nu[2] * du[1][2] + np * pi[1];
+    gW += nr * r[2] + nu[0] * du[2][0] + nu[1] * du[2][1] + nu[2] * du[2][2] + np * pi[2];
+    gr[0] += nr * U;
+    gr[1] += nr * V;
+    gr[2] += nr * W;
+    gpi[0] += np * U;
+    gpi[1] += np * V;
+    gpi[2] += np * W;
+    const T gdiv = nr + np * (g.gamma * th);
+    gth += np * (g.gamma * div);
+    gdu[0][0] += gdiv;
+    gdu[1][1] += gdiv;
+    gdu[2][2] += gdiv;
+  }
+  // the primitive derivatives
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const T ge = g.gm1 * gpi[d];
+    const T g0 = gdu[d][0] - U * ge, g1 = gdu[d][1] - V * ge, g2 = gdu[d][2] - W * ge;
+    const T gr0 = gr[d] - (hv2 + hu2) * ge - U * g0 - V * g1 - W * g2;
+    gU -= ge * du[d][0] + g0 * r[d];
+    gV -= ge * du[d][1] + g1 * r[d];
+    gW -= ge * du[d][2] + g2 * r[d];
+    ghv2 -= ge * r[d];
+    ghu2 -= ge * r[d];
+    sb.inv += ge * st.dq[d][4] + g0 * st.dq[d][1] + g1 * st.dq[d][2] + g2 * st.dq[d][3] + gr0 * st.dq[d][0];
+    cot.dq[d][0] += gr0 * inv;
+    cot.dq[d][1] += g0 * inv;
+    cot.dq[d][2] += g1 * inv;
+    cot.dq[d][3] += g2 * inv;
+    cot.dq[d][4] += ge * inv;
+  }
+  sb.U = gU + U * ghu2;
+  sb.V = gV + V * ghv2;
+  sb.W = gW + W * ghv2;
+  sb.theta = gth - il2 * (gil + T(2) * il * gil2);
   prim_of_rev(st.q, s, g, sb, cot.q);
   return phi;
 }

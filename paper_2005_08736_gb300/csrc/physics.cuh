@@ -77,152 +77,11 @@ HGKS_HD Prim<T> prim_of(const T dq[5], const Gas<T>& g) {
   return s;
 }
 
-// Normalised moments <.> = (1/rho) int g (.) dXi of a Maxwellian.  u may be
-// taken over the whole line or over a half line; v, w over the whole line.
-template <class T>
-struct Mom {
-  T u[7], v[7], w[7];
-  T xi1, xi2;  // <xi^2> = K theta, <xi^4> = K (K+2) theta^2
-};
-
 template <class T>
 HGKS_HD void gauss_recursion(T* m, T U, T theta) {
   // <c^(n+2)> = U <c^(n+1)> + (n+1) theta <c^n>, on the line and on half lines.
 #pragma unroll
   for (int n = 0; n < 5; ++n) m[n + 2] = U * m[n + 1] + T(n + 1) * theta * m[n];
-}
-
-// half: 0 whole line, +1 u > 0, -1 u < 0.
-template <class T>
-HGKS_HD void moments(const Prim<T>& s, const Gas<T>& g, int half, Mom<T>& m) {
-  if (half == 0) {
-    m.u[0] = T(1);
-    m.u[1] = s.U;
-  } else {
-    // <u^0>_{u>0} = erfc(-sqrt(lam) U)/2, <u^1>_{u>0} = U <u^0> + exp(-lam U^2)/(2 sqrt(pi lam)).
-    const T x = tsqrt(s.lam) * s.U;
-    const T e = texp(-x * x) * T(0.28209479177387814) / tsqrt(s.lam);  // 1/(2 sqrt(pi))
-    const T sg = T(half);
-    m.u[0] = T(0.5) * (T(1) + sg * terf(x));
-    m.u[1] = s.U * m.u[0] + sg * e;
-  }
-  gauss_recursion(m.u, s.U, s.theta);
-  m.v[0] = T(1);
-  m.v[1] = s.V;
-  gauss_recursion(m.v, s.V, s.theta);
-  m.w[0] = T(1);
-  m.w[1] = s.W;
-  gauss_recursion(m.w, s.W, s.theta);
-  m.xi1 = g.K * s.theta;
-  m.xi2 = g.K * (g.K + T(2)) * s.theta * s.theta;
-}
-
-// <u^a v^b w^c>
-template <int A, int B, int C, class T>
-HGKS_HD T mm(const Mom<T>& m) {
-  return m.u[A] * m.v[B] * m.w[C];
-}
-
-// <u^a v^b w^c psi>, psi = (1, u, v, w, (u^2+v^2+w^2+xi^2)/2)
-template <int A, int B, int C, class T>
-HGKS_HD void mom_psi(const Mom<T>& m, T out[5]) {
-  const T m0 = mm<A, B, C>(m);
-  out[0] = m0;
-  out[1] = mm<A + 1, B, C>(m);
-  out[2] = mm<A, B + 1, C>(m);
-  out[3] = mm<A, B, C + 1>(m);
-  out[4] = T(0.5) * (mm<A + 2, B, C>(m) + mm<A, B + 2, C>(m) + mm<A, B, C + 2>(m) + m0 * m.xi1);
-}
-
-// <(a.psi) u^a v^b w^c psi>, a.psi = a0 + a1 u + a2 v + a3 w + a4 (u^2+v^2+w^2+xi^2)/2.
-template <int A, int B, int C, class T>
-HGKS_HD void mom_apsi(const Mom<T>& m, const T a[5], T out[5]) {
-  T t0[5], t1[5], t2[5], t3[5], tu[5], tv[5], tw[5];
-  mom_psi<A, B, C>(m, t0);
-  mom_psi<A + 1, B, C>(m, t1);
-  mom_psi<A, B + 1, C>(m, t2);
-  mom_psi<A, B, C + 1>(m, t3);
-  mom_psi<A + 2, B, C>(m, tu);
-  mom_psi<A, B + 2, C>(m, tv);
-  mom_psi<A, B, C + 2>(m, tw);
-  // <xi^2 u^a v^b w^c psi>: xi^2 multiplies every component, and psi_4 adds xi^4/2.
-  const T m0 = mm<A, B, C>(m);
-  T tx[5];
-  tx[0] = m.xi1 * m0;
-  tx[1] = m.xi1 * mm<A + 1, B, C>(m);
-  tx[2] = m.xi1 * mm<A, B + 1, C>(m);
-  tx[3] = m.xi1 * mm<A, B, C + 1>(m);
-  tx[4] = T(0.5) * (m.xi1 * (mm<A + 2, B, C>(m) + mm<A, B + 2, C>(m) + mm<A, B, C + 2>(m)) +
-                    m.xi2 * m0);
-  const T h = T(0.5) * a[4];
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-    out[i] = a[0] * t0[i] + a[1] * t1[i] + a[2] * t2[i] + a[3] * t3[i] +
-             h * (tu[i] + tv[i] + tw[i] + tx[i]);
-}
-
-// Symmetric matrix <u^a v^b w^c psi_i psi_j> (upper triangle, 15 entries in
-// the order 00 01 02 03 04 11 12 13 14 22 23 24 33 34 44).
-template <int A, int B, int C, class T>
-HGKS_HD void mom_psipsi(const Mom<T>& m, T M[15]) {
-  const T x1 = m.xi1, x2 = m.xi2;
-  const T m0 = mm<A, B, C>(m);
-  const T mu1 = mm<A + 1, B, C>(m), mv1 = mm<A, B + 1, C>(m), mw1 = mm<A, B, C + 1>(m);
-  const T mu2 = mm<A + 2, B, C>(m), mv2 = mm<A, B + 2, C>(m), mw2 = mm<A, B, C + 2>(m);
-  M[0] = m0;
-  M[1] = mu1;
-  M[2] = mv1;
-  M[3] = mw1;
-  M[4] = T(0.5) * (mu2 + mv2 + mw2 + m0 * x1);
-  M[5] = mu2;
-  M[6] = mm<A + 1, B + 1, C>(m);
-  M[7] = mm<A + 1, B, C + 1>(m);
-  M[8] = T(0.5) * (mm<A + 3, B, C>(m) + mm<A + 1, B + 2, C>(m) + mm<A + 1, B, C + 2>(m) + mu1 * x1);
-  M[9] = mv2;
-  M[10] = mm<A, B + 1, C + 1>(m);
-  M[11] = T(0.5) * (mm<A + 2, B + 1, C>(m) + mm<A, B + 3, C>(m) + mm<A, B + 1, C + 2>(m) + mv1 * x1);
-  M[12] = mw2;
-  M[13] = T(0.5) * (mm<A + 2, B, C + 1>(m) + mm<A, B + 2, C + 1>(m) + mm<A, B, C + 3>(m) + mw1 * x1);
-  M[14] = T(0.25) * (mm<A + 4, B, C>(m) + mm<A, B + 4, C>(m) + mm<A, B, C + 4>(m) +
-                     T(2) * (mm<A + 2, B + 2, C>(m) + mm<A + 2, B, C + 2>(m) + mm<A, B + 2, C + 2>(m)) +
-                     T(2) * x1 * (mu2 + mv2 + mw2) + x2 * m0);
-}
-
-// out += M a for the symmetric matrix M of mom_psipsi.
-template <class T>
-HGKS_HD void sym5_matvec_add(const T M[15], const T a[5], T out[5]) {
-  out[0] += M[0] * a[0] + M[1] * a[1] + M[2] * a[2] + M[3] * a[3] + M[4] * a[4];
-  out[1] += M[1] * a[0] + M[5] * a[1] + M[6] * a[2] + M[7] * a[3] + M[8] * a[4];
-  out[2] += M[2] * a[0] + M[6] * a[1] + M[9] * a[2] + M[10] * a[3] + M[11] * a[4];
-  out[3] += M[3] * a[0] + M[7] * a[1] + M[10] * a[2] + M[12] * a[3] + M[13] * a[4];
-  out[4] += M[4] * a[0] + M[8] * a[1] + M[11] * a[2] + M[13] * a[3] + M[14] * a[4];
-}
-
-// Solution a of <a.psi psi> = b (moment matrix of the Maxwellian, K internal
-// degrees of freedom), in closed form.
-template <class T>
-HGKS_HD void slope_solve(const Prim<T>& s, const Gas<T>& g, const T b[5],
-                                            T a[5]) {
-  const T q2 = s.U * s.U + s.V * s.V + s.W * s.W;
-  const T k3t = (g.K + T(3)) * s.theta;
-  const T l2 = T(2) * s.lam;
-  a[4] = (l2 * l2 / (g.K + T(3))) *
-         (T(2) * (b[4] - s.U * b[1] - s.V * b[2] - s.W * b[3]) + (q2 - k3t) * b[0]);
-  a[3] = l2 * (b[3] - s.W * b[0]) - s.W * a[4];
-  a[2] = l2 * (b[2] - s.V * b[0]) - s.V * a[4];
-  a[1] = l2 * (b[1] - s.U * b[0]) - s.U * a[4];
-  a[0] = b[0] - s.U * a[1] - s.V * a[2] - s.W * a[3] - T(0.5) * a[4] * (q2 + k3t);
-}
-
-// <u (a_n.psi u + a_t1.psi v + a_t2.psi w) psi>
-template <class T>
-HGKS_HD void mom_u_adotu(const Mom<T>& m, const T a[3][5], T out[5]) {
-  T r0[5], r1[5], r2[5];
-  mom_apsi<2, 0, 0>(m, a[0], r0);
-  mom_apsi<1, 1, 0>(m, a[1], r1);
-  mom_apsi<1, 0, 1>(m, a[2], r2);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) out[i] = r0[i] + r1[i] + r2[i];
 }
 
 // rho <u psi> - E(Q_ref): the Euler flux of the state minus that of the
@@ -278,27 +137,6 @@ HGKS_HD void state_time_derivative(const Prim<T>& s, T H, const T dq[3][5],
   euler_jvp<2>(s, H, dq[2], g, j2);
 #pragma unroll
   for (int i = 0; i < 5; ++i) Qt[i] = -(j0[i] + j1[i] + j2[i]);
-}
-
-// Spatial slopes a_n, a_t1, a_t2 from <a_d.psi psi> = (dQ/dx_d)/rho, and the
-// time coefficient A from <(a_n u + a_t1 v + a_t2 w + A) psi> = 0 (Sec. 2.1),
-// i.e. <A psi> = Q_t / rho.
-template <class T>
-HGKS_HD void slopes_and_A(const Prim<T>& s, const Gas<T>& g, const T q[5],
-                                             const T dq[3][5], T a[3][5], T A[5]) {
-  const T inv = s.inv_rho;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    T b[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) b[i] = dq[d][i] * inv;
-    slope_solve(s, g, b, a[d]);
-  }
-  T Qt[5];
-  state_time_derivative(s, g.h_r + q[4] + s.dp, dq, g, Qt);
-#pragma unroll
-  for (int i = 0; i < 5; ++i) Qt[i] *= inv;
-  slope_solve(s, g, Qt, A);
 }
 
 // Non-equilibrium flux of the smooth BGK solution, -tau rho (<u (a.u) psi> +
