@@ -83,7 +83,7 @@ struct UpdateJob {
   UpdateArgs<T> a;
   int gx, gy;
   __device__ __forceinline__ void run(int b) const {
-    __shared__ T sfx[STAGE == 1 ? 10 : 5][kUpdTX + 1][kUpdTY];
+    __shared__ T sfx[STAGE == 1 ? 10 : 5][kUpdTX + 1][kUpdTY + 1];
 #define HGKS_UPD_BX (b % gx)
 #define HGKS_UPD_BY ((b / gx) % gy)
 #define HGKS_UPD_BZ (b / (gx * gy))
