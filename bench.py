@@ -34,8 +34,8 @@ sys.path.insert(0, ROOT)
 N_GRID = 256
 PAPER_MCUPS_256 = 2.0 ** 24 / 9.09 / 1e6  # Sec. 3.2 table: 256^3, 64 cores, 9.09 s/step
 METRIC = "Mcell-updates/s per S2O4 step"
-# cfl, dt, 2 x (3 ghost fills + transposed copy + 3 sweeps + update), time
-LAUNCHES_PER_STEP = 19
+# cfl and dt, 2 x (ghost fill with the transposed copy, three sweeps, update)
+LAUNCHES_PER_STEP = 7
 # Algorithmic work of the sweep kernel per face comes from hgks_count_flops:
 # the kernel's closed forms run on the host with a counting number type, for
 # one face point's face fields, one point's t1 pass and one face's t2 pass and
@@ -47,17 +47,9 @@ LAUNCHES_PER_STEP = 19
 # writes Q* and the increment, stage 2 reads Q* and the increment and writes
 # Q^{n+1}: 6 x 5 x 4 B.
 ALG_BYTES_PER_CELL_STEP = 120.0
-# Per tile variant: EXECUTED FP32 flops per face (fadd + fmul + 2 ffma, mean
-# of the three directions, ncu at 128^3, halo recomputation and the
-# polynomial evaluation of erf/exp included; the packed variant performs the
-# operations of variant 1) and DRAM bytes (read + write) per face of the
-# stage-1 sweep from a one-pass ncu capture at 256^3 (None where not captured
-# for the current kernel; at 128^3 the L2 holds part of the writes, so
-# smaller grids undercount).  Reported beside the algorithmic count.
-SWEEP_COUNTS = {0: {"tile": "16x8, 4 layers", "flops": 2391.8, "dram": None},
-                1: {"tile": "32x8, 2 layers", "flops": 2313.7, "dram": None},
-                2: {"tile": "16x16, 2 layers", "flops": 2247.7, "dram": None},
-                3: {"tile": "32x8, 2 layers, packed FP32 pairs", "flops": 2313.7, "dram": 58.3}}
+# DRAM bytes (read + write) per face of the stage-1 sweeps (k_march, three
+# directions in one launch) from a one-pass ncu capture at 256^3.
+SWEEP_DRAM_PER_FACE = 102.4
 
 
 def alg_flops_per_face(cfg, stage: int = 1) -> dict:
@@ -720,18 +712,17 @@ def run_ours(args, rank: int, world: int):
     peaks = load_peaks()
     sm_clock = clocks.summary()
     faces_per_launch = (N_GRID + 1) * N_GRID * N_GRID
-    flux_ms = prof["flux_stage1"] / 3.0  # average launch duration of the dominant kernel
+    flux_ms = prof["flux_stage1"] / 3.0  # the dominant kernel, per direction (one launch does three)
     sms, lanes = torch.cuda.get_device_properties(local).multi_processor_count, 128
     clock_mhz = peaks.get("sm_max_mhz", 2070.0)
     nominal_tflops = sms * lanes * 2 * clock_mhz * 1e6 / 1e12
     fp_peaks = measure_fp_peaks()  # FMA throughput of this GPU, outside the timed region
     peak_tflops = fp_peaks["fp32"]
-    counts = SWEEP_COUNTS[tune["variant"]]
     alg1, alg2 = alg_flops_per_face(cfg, 1), alg_flops_per_face(cfg, 2)
     achieved = alg1["flops"] * faces_per_launch / (flux_ms * 1e-3) / 1e12
-    traffic = counts["dram"] * faces_per_launch if counts["dram"] else None
+    traffic = SWEEP_DRAM_PER_FACE * faces_per_launch
     roofline = {"bound": "alu",
-                "kernel": f"k_sweep stage 1 (FP32, linear WENO5, smooth flux, tile {counts['tile']})",
+                "kernel": "k_march stage 1 (FP32, linear WENO5, smooth flux), per direction",
                 "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved / peak_tflops,
                 "traffic": traffic,
@@ -740,17 +731,13 @@ def run_ours(args, rank: int, world: int):
                 "flops_note": "algorithmic (hgks_count_flops): the kernel's closed forms tallied on "
                               "the host per face, no halo recomputation, common subexpressions "
                               "once, dead results not counted, erf/exp/sqrt not counted",
-                "executed_flops_per_launch": counts["flops"] * faces_per_launch,
-                "executed_note": "ncu fadd + fmul + 2 ffma per face at 128^3 (halo recomputation and "
-                                 "the polynomial work of erf/exp included)",
                 "peak_source": "measured: FP32 FMA throughput of this GPU (hgks_measure_fp_peaks)",
                 "nominal_peak": nominal_tflops,
                 "nominal_source": f"{sms} SMs x 128 FP32 lanes x 2 flops x {clock_mhz:.0f} MHz",
                 "frac_of_nominal": achieved / nominal_tflops,
                 "measured_fma_tflops": fp_peaks,
                 "launch_ms": flux_ms, "kernel_ms_per_step": prof,
-                "hbm_frac": (traffic / (flux_ms * 1e-3) / (peaks.get("hbm_gbs", 6802.0) * 1e9)
-                             if traffic else None)}
+                "hbm_frac": traffic / (flux_ms * 1e-3) / (peaks.get("hbm_gbs", 6802.0) * 1e9)}
     # The whole step against its own roofline: the slower of its algorithmic
     # FP32 work at the measured FMA peak and its algorithmic HBM bytes at the
     # measured copy bandwidth.

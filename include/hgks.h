@@ -322,26 +322,26 @@ const char* hgks_ensemble_last_error(const hgks_ensemble* ens);
 hgks_status hgks_adjoint_step(hgks_ctx* ctx, double dt, const double* adj_in, double* adj_out);
 
 /* Tile autotuner (no counterpart in the paper): time the launch shapes of
- * the sweep kernel on the context's current state -- the tile variants
- * available for its configuration (four for linear weights + smooth flux in
- * FP32, one otherwise) times the number of face layers each CTA marches
+ * the sweep kernel on the context's current state -- the number of face
+ * layers (rows, for linear weights + smooth flux in FP32) each CTA marches
  * through -- with CUDA events on the context's stream, and keep the fastest
- * for later steps.  The state is unchanged (ghost layers and face-flux
+ * for later steps; the variant is always 0.  The state is unchanged (ghost layers and face-flux
  * buffers are scratch).  Writes the choice and the time of one stage's three
  * sweeps (ms) if the pointers are non-NULL.  Synchronises. */
 hgks_status hgks_autotune(hgks_ctx* ctx, int* variant_out, int* chunk_out, double* ms_out);
 
 /* Set the sweep launch shape directly (a cached autotuner result): variant
- * in [0, number of variants), chunk >= 0 face layers per CTA (0 automatic). */
+ * in [0, number of variants): linear weights + smooth flux in FP32 accept 0..3,
+ * all the same kernel, others 0; chunk >= 0 face layers (rows) per CTA (0
+ * automatic). */
 hgks_status hgks_set_sweep_shape(hgks_ctx* ctx, int variant, int chunk);
 
 /* Profiling aid (not on the hot path): advance ONE step without the graph,
  * with CUDA events around every kernel launch on the context's stream, and
  * write the summed device time in milliseconds of each kernel class to
  * ms_out[0..nclass-1] (nclass >= 6): 0 CFL reduction and dt, 1 ghost-cell
- * fills, 2 face fields (3 directions x 2 stages), 3 Gauss-point flux of
- * stage 1 (3 launches), 4 Gauss-point flux of stage 2 (3 launches),
- * 5 update (2 launches).  dt as in hgks_step.  Synchronises. */
+ * fills, 2 unused (0), 3 sweeps of stage 1 (face fields to flux, three
+ * directions in one launch), 4 sweeps of stage 2, 5 update (2 launches).  dt as in hgks_step.  Synchronises. */
 hgks_status hgks_profile_step(hgks_ctx* ctx, double dt, double* ms_out, int nclass);
 
 /* Advance nsteps S2O4 steps of the conservative state cons_inout (DEVICE
