@@ -74,7 +74,9 @@ cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe)
 
 // Tile of k_sweep, TP x TS faces.  FP64 is bound by its pipe, not by latency:
 // with the smooth flux one CTA of 512 threads has 1.56 points of face fields
-// per face where two of 16 x 8 faces have 1.88.
+// per face where two of 16 x 8 faces have 1.88 (128^3: 44.3 -> 40.5 ms a step
+// against one CTA of 16 x 8).  FP32 needs the second CTA's other phase: the full
+// flux on 16 x 16 tiles, one CTA, takes 58.1 ms at 256^3, on 16 x 8 56.3.
 template <class T, int FLUX> struct SweepTile {
   static constexpr int TP = 16, TS = sizeof(T) == 8 && FLUX == FLUX_SMOOTH ? 16 : 8;
 };
