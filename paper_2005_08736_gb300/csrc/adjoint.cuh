@@ -38,7 +38,8 @@ namespace hgks {
 // d|x|/dx = sign(x) with sign(0) = 0), each a sum of two squares of linear
 // forms in the differences, and the differences' cotangents telescope onto q.
 // FP64: one reciprocal of B0 B1 B2 and one of SR SL replace eight divisions
-// (in range for |q| up to 1e25, as in weno5_dev).  About 120 operations and
+// (in range through normalise_indicators, whose power of two the indicators'
+// cotangents take back).  About 120 operations and
 // two divisions, against 230 and eight from the candidates' coefficients in
 // the averages (whose zero products FP64 has to carry out): the adjoint
 // evaluates this some 50 times per face.
@@ -53,7 +54,11 @@ HGKS_HD void weno5_dev_vjp(const T q[5], T hL, T hR, T cot[5]) {
   const T k = T(3) / T(13);
   const T b0 = k * t0 * t0 + s0 * s0, b1 = k * t1 * t1 + s1 * s1, b2 = k * t2 * t2 + s2 * s2;
   const T e = MODE == RECON_WENO_JS ? T(12e-6 / 13) : T(12e-20 / 13);
-  const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+  T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e, d02 = b0 - b2, scale = T(1);
+  if constexpr (std::is_same<T, double>::value) {
+    scale = with_high_word(1.0, (1023 << 20) - normalise_indicators(B0, B1, B2));
+    d02 = B0 - B2;
+  }
   T r0, r1, r2;  // 1/B
   if constexpr (std::is_same<T, float>::value) {
     r0 = T(1) / B0;
@@ -71,7 +76,7 @@ HGKS_HD void weno5_dev_vjp(const T q[5], T hL, T hR, T cot[5]) {
     f1 = r1 * r1;
     f2 = r2 * r2;
   } else {
-    tau5 = tabs(b0 - b2);
+    tau5 = tabs(d02);
     f0 = T(1) + tau5 * r0;
     f1 = T(1) + tau5 * r1;
     f2 = T(1) + tau5 * r2;
@@ -95,17 +100,18 @@ HGKS_HD void weno5_dev_vjp(const T q[5], T hL, T hR, T cot[5]) {
   const T F2 = T(3) * (aR * (z - rR)) + aL * (e0 - rl);
   T G0, G1, G2;
   if (MODE == RECON_WENO_JS) {
-    G0 = T(-2) * F0 * f0 * r0;
-    G1 = T(-2) * F1 * f1 * r1;
-    G2 = T(-2) * F2 * f2 * r2;
+    const T m = T(-2) * scale;
+    G0 = m * F0 * f0 * r0;
+    G1 = m * F1 * f1 * r1;
+    G2 = m * F2 * f2 * r2;
   } else {
     // (F tau5 r) r in this order: r^2 alone overflows FP32 where b vanishes
     // (r = 1e20), and tau5 = 0 there.
-    const T d02 = b0 - b2, sg = d02 > T(0) ? T(1) : (d02 < T(0) ? T(-1) : T(0));
+    const T sg = d02 > T(0) ? scale : (d02 < T(0) ? -scale : T(0)), t = tau5 * scale;
     const T gt = sg * (F0 * r0 + F1 * r1 + F2 * r2);
-    G0 = gt - F0 * tau5 * r0 * r0;
-    G1 = -(F1 * tau5 * r1 * r1);
-    G2 = -(gt + F2 * tau5 * r2 * r2);
+    G0 = gt - F0 * t * r0 * r0;
+    G1 = -(F1 * t * r1 * r1);
+    G2 = -(gt + F2 * t * r2 * r2);
   }
   // candidates and indicators onto the differences
   const T C0 = aR * f0, C1 = aR * g1, E0 = aL * f2, E1 = aL * g1;

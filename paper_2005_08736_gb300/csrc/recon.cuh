@@ -12,6 +12,7 @@
 
 #include "physics.cuh"
 
+#include <cstring>
 #include <type_traits>
 
 namespace hgks {
@@ -24,6 +25,45 @@ enum FluxKind { FLUX_SMOOTH = 0, FLUX_FULL = 1 };
 // The scalar reconstructions below see the underlying Recon.
 template <int MODE> __host__ __device__ constexpr int recon_of() { return MODE >= 3 ? MODE - 2 : MODE; }
 template <int MODE> __host__ __device__ constexpr bool is_char_mode() { return MODE >= 3; }
+
+// The high word of a double, and the double with it replaced.
+HGKS_HD int high_word(double x) {
+#if defined(__CUDA_ARCH__)
+  return __double2hiint(x);
+#else
+  long long b;
+  std::memcpy(&b, &x, sizeof b);
+  return int(b >> 32);
+#endif
+}
+HGKS_HD double with_high_word(double x, int hi) {
+#if defined(__CUDA_ARCH__)
+  return __hiloint2double(hi, __double2loint(x));
+#else
+  long long b;
+  std::memcpy(&b, &x, sizeof b);
+  b = ((long long)hi << 32) | (b & 0xffffffffLL);
+  std::memcpy(&x, &b, sizeof x);
+  return x;
+#endif
+}
+
+// Divides the FP64 smoothness indicators, positive, by the power of two that
+// brings the largest to [1, 2); what would fall below 2^-240 stays there (its
+// candidate has all the weight as it is).  The weights depend on the ratios
+// alone, so their products then fit FP64 for any data whose squares do.  Ten
+// integer operations on the exponents, none on the FP64 pipe that bounds the
+// callers; a test with a branch instead cost 4 % of the whole step (FP64
+// WENO-Z + full flux 64^3).  Returns the exponent field of that power.
+HGKS_HD int normalise_indicators(double& B0, double& B1, double& B2) {
+  const int h0 = high_word(B0), h1 = high_word(B1), h2 = high_word(B2), one = 1023 << 20, least = (1023 - 240) << 20;
+  int e = h0 > h1 ? h0 : h1;
+  e = ((e > h2 ? e : h2) & 0x7ff00000) - one;
+  B0 = with_high_word(B0, h0 - e > least ? h0 - e : least);
+  B1 = with_high_word(B1, h1 - e > least ? h1 - e : least);
+  B2 = with_high_word(B2, h2 - e > least ? h2 - e : least);
+  return e;
+}
 
 // Nonlinear WENO5 end values of the centre cell, as six times their
 // deviation from its average: rL = 6 (q(x_{i-1/2}) - q2), rR = 6 (q(x_{i+1/2}) - q2).
@@ -45,8 +85,8 @@ template <int MODE> __host__ __device__ constexpr bool is_char_mode() { return M
 // FP64: a division costs as much as ten multiplications there, so the
 // weights are multiplied through by the product of the denominators (WENO-Z:
 // B0 B1 B2; WENO-JS: its square), which leaves one (WENO-Z) or two divisions
-// of the five; the products stay in range for |q| up to 1e25 (WENO-Z) and
-// 1e38 (WENO-JS).  FP32's range does not allow the products.
+// of the five; normalise_indicators keeps the products in range.  FP32's range
+// does not allow them.
 template <int MODE, class T>
 HGKS_HD void weno5_dev(T q0, T q1, T q2, T q3, T q4, T& rL, T& rR) {
   static_assert(MODE == RECON_WENO_JS || MODE == RECON_WENO_Z, "nonlinear weights");
@@ -63,8 +103,9 @@ HGKS_HD void weno5_dev(T q0, T q1, T q2, T q3, T q4, T& rL, T& rR) {
   T f0, f1, f2;  // weight factors of beta0, beta1, beta2 (up to a common factor)
   if (MODE == RECON_WENO_JS) {
     const T e = T(12e-6 / 13);
-    const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+    T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
     if constexpr (std::is_same<T, double>::value) {
+      normalise_indicators(B0, B1, B2);
       const T p12 = B1 * B2, p02 = B0 * B2, p01 = B0 * B1;
       f0 = p12 * p12;
       f1 = p02 * p02;
@@ -76,13 +117,15 @@ HGKS_HD void weno5_dev(T q0, T q1, T q2, T q3, T q4, T& rL, T& rR) {
     }
   } else {
     const T e = T(12e-20 / 13);
-    const T tau5 = tabs(b0 - b2);
-    const T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
+    T B0 = b0 + e, B1 = b1 + e, B2 = b2 + e;
     if constexpr (std::is_same<T, double>::value) {
+      normalise_indicators(B0, B1, B2);
+      const T tau5 = tabs(B0 - B2);
       f0 = (B0 + tau5) * (B1 * B2);
       f1 = (B1 + tau5) * (B0 * B2);
       f2 = (B2 + tau5) * (B0 * B1);
     } else {
+      const T tau5 = tabs(b0 - b2);
       f0 = tau5 * (T(1) / B0) + T(1);
       f1 = tau5 * (T(1) / B1) + T(1);
       f2 = tau5 * (T(1) / B2) + T(1);
@@ -93,8 +136,8 @@ HGKS_HD void weno5_dev(T q0, T q1, T q2, T q3, T q4, T& rL, T& rR) {
   const T nL = f2 * e0 + g1 * e1 + g0 * w, SL = f2 + g1 + g0;
   if constexpr (std::is_same<T, double>::value && MODE == RECON_WENO_Z) {
     const T inv = T(1) / (SR * SL);
-    rR = nR * SL * inv;
-    rL = -(nL * SR * inv);
+    rR = nR * (SL * inv);
+    rL = -(nL * (SR * inv));
   } else {
     rR = nR * (T(1) / SR);
     rL = -(nL * (T(1) / SL));
