@@ -123,8 +123,10 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
     }
     // Cells f0-3 .. f0+LAYERS+1 along n of the CTA's columns, one row ahead:
     // thread (variable v, column hp) copies its PLANES cells asynchronously.
-    // Planes past the ghost cells are left out: no layer that exists reads
-    // them.
+    // Planes past the ghost cells repeat the last one: only layers that do not
+    // exist read them, but such a layer shares its pair with face n (walls, an
+    // even number of cells), and the two choose their compatibility rule
+    // together.
     const int gvv = v == 0 ? 0 : (v == 1 ? 1 + d : (v == 2 ? 1 + P : (v == 3 ? 1 + S : 4)));
     const float* src = a.q + gvv * g.P + (long long)f0 * sn + (min(p0 - 2 + hp, nP + 1) + kGhost) * sp +
                        (long long)kGhost * ss;
@@ -133,11 +135,18 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
     auto stage = [&](int row) {
       const float* q = src + (long long)row * ss;
       const unsigned to = dst + (row & 1) * (March::CELLS * 4);
+      auto copy = [&](int j) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + j * (HP * 4)), "l"(q) : "memory");
+      };
+      if (planes == March::PLANES) {
 #pragma unroll
-      for (int j = 0; j < March::PLANES; ++j) {
-        if (j < planes)
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + j * (HP * 4)), "l"(q) : "memory");
-        q += sn;
+        for (int j = 0; j < March::PLANES; ++j, q += sn) copy(j);
+      } else if (planes > 0) {
+#pragma unroll 1
+        for (int j = 0; j < March::PLANES; ++j) {
+          copy(j);
+          if (j + 1 < planes) q += sn;
+        }
       }
     };
     stage(s0 - 2);
