@@ -816,7 +816,7 @@ def main():
     ap.add_argument("--char", action="store_true",
                     help="WENO in characteristic variables (profiling cases)")
     ap.add_argument("--shape", default="",
-                    help="V,C: sweep tile variant and march length (skips the autotuner)")
+                    help="V,C: a stored launch shape (variant and face layers per CTA; skips the autotuner)")
     ap.add_argument("--history", action="store_true",
                     help="Taylor-Green E_k / dissipation history, FP32 against FP64")
     ap.add_argument("--t-end", type=float, default=10.0)

@@ -286,14 +286,13 @@ hgks_status hgks_kinetic_energy(hgks_ctx* ctx, const double* cons, double* grad,
  * for the work already enqueued on the other members' streams; they wait for
  * the batch afterwards).  Two forms of the graph:
  *   - batched (the default when the members share precision, reconstruction
- *     and its variables, flux and sweep tile variant, and have no mass-flux
- *     force and no statistics history): ONE kernel launch per phase of the
- *     step (CFL reduction, dt, the ghost fills, the transposed copy, the three
- *     sweeps and the update of each stage, time) for all members, driven by
- *     an instance table of up to 32 members per launch (kernel parameter):
- *     each block finds its instance and its local block and runs that
- *     instance's part of the phase; ragged grids are fine, no block waits on
- *     another;
+ *     and its variables and flux, and have no mass-flux force and no
+ *     statistics history): ONE kernel launch per phase of the step (CFL
+ *     reduction with dt; ghost fill with the transposed copy, the three sweeps
+ *     and the update of each stage) for all members, driven by an instance
+ *     table of up to 32 members per launch (kernel parameter): each block
+ *     finds its instance and its local block and runs that instance's part of
+ *     the phase; ragged grids are fine, no block waits on another;
  *   - graph branches (any members): every member's own launches as a parallel
  *     branch forked from and joined into the first member's stream.
  * dt > 0 fixes every member's step; dt <= 0 takes each member's own CFL step.
@@ -323,17 +322,18 @@ hgks_status hgks_adjoint_step(hgks_ctx* ctx, double dt, const double* adj_in, do
 
 /* Tile autotuner (no counterpart in the paper): time the launch shapes of
  * the sweep kernel on the context's current state -- the number of face
- * layers (rows, for linear weights + smooth flux in FP32) each CTA marches
- * through -- with CUDA events on the context's stream, and keep the fastest
- * for later steps; the variant is always 0.  The state is unchanged (ghost layers and face-flux
- * buffers are scratch).  Writes the choice and the time of one stage's three
- * sweeps (ms) if the pointers are non-NULL.  Synchronises. */
+ * layers each CTA marches through (linear weights + smooth flux in FP32 have
+ * one shape, 0) -- with CUDA events on the context's stream, and keep the
+ * fastest for later steps; the variant is always 0.  The state is unchanged
+ * (ghost layers and face-flux buffers are scratch).  Writes the choice and the
+ * time of one stage's three sweeps (ms) if the pointers are non-NULL.
+ * Synchronises. */
 hgks_status hgks_autotune(hgks_ctx* ctx, int* variant_out, int* chunk_out, double* ms_out);
 
 /* Set the sweep launch shape directly (a cached autotuner result): variant
- * in [0, number of variants): linear weights + smooth flux in FP32 accept 0..3,
- * all the same kernel, others 0; chunk >= 0 face layers (rows) per CTA (0
- * automatic). */
+ * in [0, number of variants) and chunk >= 0 face layers per CTA (0 automatic).
+ * Linear weights + smooth flux in FP32 accept variants 0..3 and any chunk, all
+ * of which run their one launch shape; others variant 0. */
 hgks_status hgks_set_sweep_shape(hgks_ctx* ctx, int variant, int chunk);
 
 /* Profiling aid (not on the hot path): advance ONE step without the graph,

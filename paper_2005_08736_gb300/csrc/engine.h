@@ -59,10 +59,8 @@ struct Engine {
   int diag_blocks = 0;
   int cfl_blocks = 0;
   int sms = 152;  // multiprocessors of the device
-  // Sweep launch choices (set by hgks_autotune): the variant of a stored
-  // choice (it no longer selects a kernel) and the length of each CTA's march,
-  // in rows (k_march) or face layers (k_sweep); 0: automatic.
-  int sweep_variant = 0;
+  // Face layers each CTA of k_sweep marches through (set by hgks_autotune or
+  // hgks_set_sweep_shape); 0: automatic.
   int sweep_chunk = 0;
 };
 
@@ -141,16 +139,15 @@ template <class T> cudaError_t enqueue_sweep_only(const Engine& e);
 template <class T> cudaError_t enqueue_diag(const Engine& e);
 template <class T> cudaError_t enqueue_from_fp64(const Engine& e, const double* src, int conservative);
 template <class T> cudaError_t enqueue_to_fp64(const Engine& e, double* dst);
+// Whether the sweeps run in k_march (march.cuh), else in k_sweep (sweep_tile.cuh).
+bool sweeps_march(const hgks_config& c);
 // Adjoint of one S2O4 step at the state e.q with the step dt already in
 // e.scal[0]: adj_out = (dQ^{n+1}/dQ^n)^T adj_in (FP64 device arrays, [5][N]).
-// Number of tile variants of the sweep kernel for the context's configuration.
-int sweep_variant_count(const Engine& e);
 template <class T> cudaError_t enqueue_adjoint_step(const Engine& e, const double* adj_in,
                                                     double* adj_out);
 // One S2O4 step of every member with one batched launch per phase (the
-// members share precision, reconstruction, flux and tile variant and have
-// no mass-flux force and no statistics history); Q^{n+1} of each ends in its
-// qs.  On stream s.
+// members share precision, reconstruction and flux and have no mass-flux force
+// and no statistics history); Q^{n+1} of each ends in its qs.  On stream s.
 template <class T> cudaError_t enqueue_batched_step(const std::vector<Engine*>& members, double dt_fixed,
                                                     cudaStream_t s);
 cudaError_t enqueue_reset_scalars(const Engine& e);

@@ -928,15 +928,14 @@ struct hgks_ensemble {
 };
 
 // Whether the members can share batched launches: same precision,
-// reconstruction (and variables), flux and sweep tile variant, no mass-flux
-// force and no statistics history.
+// reconstruction (and variables) and flux, no mass-flux force and no
+// statistics history.
 static bool ensemble_batchable(const hgks_ensemble* en) {
   const hgks::Engine& a = en->members[0]->e;
   for (hgks_ctx* c : en->members) {
     const hgks::Engine& e = c->e;
     if (e.cfg.prec != a.cfg.prec || e.cfg.recon != a.cfg.recon || e.cfg.flux != a.cfg.flux ||
-        e.cfg.recon_vars != a.cfg.recon_vars || e.sweep_variant != a.sweep_variant ||
-        e.cfg.force_mode != HGKS_FORCE_CONSTANT || e.hist_every != 0)
+        e.cfg.recon_vars != a.cfg.recon_vars || e.cfg.force_mode != HGKS_FORCE_CONSTANT || e.hist_every != 0)
       return false;
   }
   return true;
@@ -973,8 +972,8 @@ hgks_status hgks_ensemble_create(hgks_ctx** ctxs, int n, hgks_ensemble** out) {
 hgks_status hgks_ensemble_set_batched(hgks_ensemble* en, int batched) {
   if (!en) return HGKS_E_INVAL;
   if (batched && !ensemble_batchable(en)) {
-    en->err = "batched launches need members of one precision, scheme and tile variant, without the "
-              "mass-flux force or a statistics history";
+    en->err = "batched launches need members of one precision and scheme, without the mass-flux force or a "
+              "statistics history";
     return HGKS_E_UNSUPPORTED;
   }
   if (en->batched != (batched != 0)) {
@@ -1121,12 +1120,12 @@ hgks_status hgks_autotune(hgks_ctx* c, int* variant_out, int* chunk_out, double*
   HGKS_CHECK(c, cudaEventCreate(&t1));
   const int nmax = std::max(e.n[0], std::max(e.n[1], e.n[2])) + 1;
   const int chunks[] = {0, 8, 16, 32, 64, 128};
+  const int candidates = hgks::sweeps_march(e.cfg) ? 1 : 6;  // k_march has one shape
   float best = 1e30f;
   int best_c = 0;
   cudaError_t err = cudaSuccess;
-  for (int ci = 0; ci < 6 && err == cudaSuccess; ++ci) {
+  for (int ci = 0; ci < candidates && err == cudaSuccess; ++ci) {
     if (chunks[ci] > 2 * nmax) continue;
-    e.sweep_variant = 0;
     e.sweep_chunk = chunks[ci];
     float ms = 0.f;
     for (int rep = 0; rep < 3 && err == cudaSuccess; ++rep) {  // rep 0 warms up
@@ -1144,7 +1143,6 @@ hgks_status hgks_autotune(hgks_ctx* c, int* variant_out, int* chunk_out, double*
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
   HGKS_CHECK(c, err);
-  e.sweep_variant = 0;
   e.sweep_chunk = best_c;
   drop_graphs(c);  // the captured steps hold the old launch shapes
   if (variant_out) *variant_out = 0;
@@ -1155,9 +1153,10 @@ hgks_status hgks_autotune(hgks_ctx* c, int* variant_out, int* chunk_out, double*
 
 hgks_status hgks_set_sweep_shape(hgks_ctx* c, int variant, int chunk) {
   if (!c) return fail(c, HGKS_E_INVAL, "null context");
-  if (variant < 0 || variant >= hgks::sweep_variant_count(c->e) || chunk < 0)
+  // Linear weights + smooth flux in FP32 had four tile variants once, which
+  // stored choices may name.
+  if (variant < 0 || variant >= (hgks::sweeps_march(c->e.cfg) ? 4 : 1) || chunk < 0)
     return fail(c, HGKS_E_INVAL, "no such sweep variant");
-  c->e.sweep_variant = variant;
   c->e.sweep_chunk = chunk;
   drop_graphs(c);
   return HGKS_OK;
@@ -1200,11 +1199,8 @@ const char* hgks_last_error(const hgks_ctx* c) {
 
 namespace hgks {
 
-// Variants a stored launch shape may name: linear weights + smooth flux in
-// FP32 had four tiles once, all of which run k_march now.
-int sweep_variant_count(const Engine& e) {
-  return (e.cfg.prec == HGKS_FP32 && e.cfg.recon == HGKS_RECON_LINEAR &&
-          e.cfg.flux == HGKS_FLUX_SMOOTH) ? 4 : 1;
+bool sweeps_march(const hgks_config& c) {
+  return c.prec == HGKS_FP32 && c.recon == HGKS_RECON_LINEAR && c.flux == HGKS_FLUX_SMOOTH;
 }
 
 long long face_flux_elems(const Engine& e, int d) {

@@ -217,8 +217,8 @@ class Simulation:
         torch.cuda.current_stream(self.device).wait_stream(self.stream)
 
     def autotune(self, cache: str | None = None) -> dict:
-        """Pick the sweep's launch shape for this configuration (tile variant and
-        face layers per CTA) by timing the candidates on the current state; with
+        """Pick the sweep's launch shape for this configuration (face layers per
+        CTA; the variant is 0) by timing the candidates on the current state; with
         `cache` (a JSON file) a known configuration reuses its stored choice."""
         import json
         import os

@@ -1,0 +1,37 @@
+"""Launch shapes of the sweeps: what earlier builds stored is accepted and does
+not slow the step down, and members that differ in it share batched launches."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from paper_2005_08736_gb300 import inputs  # noqa: E402
+from paper_2005_08736_gb300.solver import Ensemble, Simulation, taylor_green_config  # noqa: E402
+
+
+def simulation(n, shape=(0, 0)):
+    sim = Simulation(taylor_green_config(n, "fp32"))
+    sim._call(sim.lib.hgks_set_sweep_shape(sim.h, *shape))
+    sim.init_primitive(inputs.taylor_green(n))
+    return sim
+
+
+def sweep_ms(sim):
+    sim.profile_step()
+    return min(sim.profile_step()["flux_stage1"] for _ in range(5))
+
+
+@pytest.mark.parametrize("shape", [(3, 16), (0, 64), (1, 8), (0, 2 ** 31 - 1)])
+def test_stored_shapes_cost_no_more_than_the_automatic_one(shape):
+    # 64^3: 64 rows a block made the sweeps 2.5 times as long, 8 rows 1.2 times;
+    # two runs of one shape differ by a few per cent.
+    assert sweep_ms(simulation(64, shape)) <= 1.1 * sweep_ms(simulation(64))
+
+
+def test_members_with_other_stored_shapes_share_batched_launches():
+    ens = Ensemble([simulation(16), simulation(16, (3, 16))], batched=True)
+    ens.step(2)
+    a, b = (s.state(device=True) for s in ens.sims)
+    assert torch.equal(a, b)
+    ens.close()
