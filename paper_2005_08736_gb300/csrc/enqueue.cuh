@@ -101,27 +101,38 @@ SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
   return a;
 }
 
-// k_sweep with a TP x TS tile.  The march along the normal carries nothing
-// from one layer to the next, so its length only sets the number of CTAs: 24
-// per SM for the three directions, down to one layer each on small grids.
+// Layers of direction d that each CTA of k_sweep or k_sweep_adj marches
+// through.  The march along the normal carries nothing from one layer to the
+// next, so its length only sets the number of CTAs: 24 per SM for the three
+// directions, down to one layer each on small grids.  No march is longer than a
+// tenth of an SM's share of all layers: in a direction of few tiles and many
+// layers it would finish long after the others (long boxes, one step: FP64
+// WENO-Z + full flux 6 x 6 x 512 21.7 -> 9.2 ms, FP32 16 x 16 x 200 269 -> 207
+// us).  An even split of all layers instead costs flat boxes, whose long
+// marches start first, 2 to 4 % (128 x 128 x 6 and x 16); cubes are not
+// concerned.
+inline int march_length(const int tiles[3], const int layers[3], int d, int sms) {
+  const long long most = 24LL * sms, all = tiles[0] + tiles[1] + tiles[2];
+  long long work = 0;
+  for (int c = 0; c < 3; ++c) work += (long long)tiles[c] * layers[c];
+  const long long chunks = (most + all - 1) / all, tenth = (work + 10LL * sms - 1) / (10LL * sms);
+  return int(std::min((layers[d] + chunks - 1) / chunks, tenth));
+}
+
+// k_sweep with a TP x TS tile.
 template <class T, int TP, int TS>
 SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   SweepArgs3<T> a = sweep_common(e, q);
-  int tiles = 0;
+  int tiles[3];
   for (int d = 0; d < 3; ++d) {
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
     a.gx[d] = (e.n[P] + TP - 1) / TP;
     a.gy[d] = (e.n[S] + TS - 1) / TS;
-    tiles += a.gx[d] * a.gy[d];
+    tiles[d] = a.gx[d] * a.gy[d];
   }
   for (int d = 0; d < 3; ++d) {
-    int chunk = std::min(e.sweep_chunk, a.layers[d]);
-    if (chunk <= 0) {
-      const int want_chunks = (24 * e.sms + tiles - 1) / tiles;
-      chunk = (a.layers[d] + want_chunks - 1) / want_chunks;
-    }
-    a.chunk[d] = chunk;
-    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * ((a.layers[d] + chunk - 1) / chunk);
+    a.chunk[d] = e.sweep_chunk > 0 ? std::min(e.sweep_chunk, a.layers[d]) : march_length(tiles, a.layers, d, e.sms);
+    a.start[d + 1] = a.start[d] + tiles[d] * ((a.layers[d] + a.chunk[d] - 1) / a.chunk[d]);
   }
   return a;
 }
@@ -377,20 +388,19 @@ cudaError_t launch_adjoint_sweeps(const Engine& e, const T* q, const T* wL, cons
   a.g = g;
   a.gas = gas_of<T>(e.cfg);
   a.start[0] = 0;
-  int tiles = 0;
+  int tiles[3];
   for (int d = 0; d < 3; ++d) {
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
     a.w[d] = static_cast<const T*>(e.w[d]);
     a.gx[d] = (g.n[P] + TP - 1) / TP;
     a.gy[d] = (g.n[S] + TS - 1) / TS;
-    tiles += a.gx[d] * a.gy[d];
+    tiles[d] = a.gx[d] * a.gy[d];
   }
-  // A layer takes tens of microseconds and shares nothing with the next, so
-  // the chunks are short: 24 CTAs per SM keep the tail under a few per cent.
-  const int want_chunks = (24 * e.sms + tiles - 1) / tiles;
+  // A layer takes tens of microseconds and shares nothing with the next:
+  // march_length's 24 CTAs per SM keep the tail under a few per cent.
   for (int d = 0; d < 3; ++d) {
-    a.chunk[d] = std::max(1, (g.n[d] + want_chunks - 1) / want_chunks);
-    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * ((g.n[d] + a.chunk[d] - 1) / a.chunk[d]);
+    a.chunk[d] = march_length(tiles, g.n, d, e.sms);
+    a.start[d + 1] = a.start[d] + tiles[d] * ((g.n[d] + a.chunk[d] - 1) / a.chunk[d]);
   }
   kern<<<a.start[3], NT, smem, e.stream>>>(a);
   err = cudaGetLastError();

@@ -7,7 +7,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 from paper_2005_08736_gb300 import inputs  # noqa: E402
-from paper_2005_08736_gb300.solver import Ensemble, Simulation, taylor_green_config  # noqa: E402
+from paper_2005_08736_gb300.solver import Config, Ensemble, Simulation, taylor_green_config  # noqa: E402
 
 
 def simulation(n, shape=(0, 0)):
@@ -27,6 +27,20 @@ def test_stored_shapes_cost_no_more_than_the_automatic_one(shape):
     # 64^3: 64 rows a block made the sweeps 2.5 times as long, 8 rows 1.2 times;
     # two runs of one shape differ by a few per cent.
     assert sweep_ms(simulation(64, shape)) <= 1.1 * sweep_ms(simulation(64))
+
+
+@pytest.mark.parametrize("n", [(6, 6, 256), (6, 256, 6), (256, 6, 6), (16, 16, 200)])
+def test_long_boxes_are_split_evenly(n):
+    # One layer per CTA is the shortest march; the automatic split may be
+    # longer where that saves start-ups, never much slower.  The long axis's
+    # few tiles once marched up to 18 layers each: 1.3 to 2.7 times as long.
+    ms = []
+    for chunk in (0, 1):
+        sim = Simulation(Config(*n, prec=1, recon=2, flux=1, tau_num_C=1.0, mu_ref=5e-3, p_ref=1.0))
+        sim._call(sim.lib.hgks_set_sweep_shape(sim.h, 0, chunk))
+        sim.init_primitive(inputs.random_smooth(n, seed=3, amp=0.1, kmax=1))
+        ms.append(sweep_ms(sim))
+    assert ms[0] <= 1.15 * ms[1]
 
 
 def test_members_with_other_stored_shapes_share_batched_launches():
