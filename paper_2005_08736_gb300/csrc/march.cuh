@@ -114,7 +114,7 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
     // A, B: point pair (layers f, f + 1; column hp).  Columns past the grid's
     // halo repeat the last one (their results are not used).
     const int v = tid / HP, hp = tid % HP, f = f0 + 2 * v;
-    const bool live = tid < NPT;
+    const bool live = tid < NPT && f < layers;
     float2 r6;
     {
       const int fa = min(f, nd), fb = min(f + 1, nd);
@@ -122,30 +122,30 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
                        1.f / (6.f * (a.wn[fb - 1 + kGhost] + a.wn[fb + kGhost])));
     }
     // Cells f0-3 .. f0+LAYERS+1 along n of the CTA's columns, one row ahead:
-    // thread (variable v, column hp) copies its PLANES cells asynchronously.
-    // Planes past the ghost cells repeat the last one: only layers that do not
-    // exist read them, but such a layer shares its pair with face n (walls, an
-    // even number of cells), and the two choose their compatibility rule
-    // together.
+    // thread (variable v, column hp) copies its cells asynchronously, all that
+    // the pairs with a layer that exists read.  The plane past the ghost cells
+    // (walls, an even number of cells) repeats the last one: only a layer that
+    // does not exist reads it, but that layer shares its pair with face n, and
+    // the two choose their compatibility rule together.
     const int gvv = v == 0 ? 0 : (v == 1 ? 1 + d : (v == 2 ? 1 + P : (v == 3 ? 1 + S : 4)));
     const float* src = a.q + gvv * g.P + (long long)f0 * sn + (min(p0 - 2 + hp, nP + 1) + kGhost) * sp +
                        (long long)kGhost * ss;
     const unsigned dst = (unsigned)__cvta_generic_to_shared(cells + v * (March::PLANES * HP) + hp);
-    const int planes = v < 5 ? min(March::PLANES, nd + 6 - f0) : 0;
+    const int planes = v < 5 ? min(March::PLANES, (layers - f0 + 1) / 2 * 2 + 5) : 0, last = nd + 5 - f0;
     auto stage = [&](int row) {
       const float* q = src + (long long)row * ss;
       const unsigned to = dst + (row & 1) * (March::CELLS * 4);
       auto copy = [&](int j) {
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + j * (HP * 4)), "l"(q) : "memory");
       };
-      if (planes == March::PLANES) {
+      if (planes == March::PLANES && last >= March::PLANES - 1) {
 #pragma unroll
         for (int j = 0; j < March::PLANES; ++j, q += sn) copy(j);
-      } else if (planes > 0) {
-#pragma unroll 1
+      } else {
+#pragma unroll
         for (int j = 0; j < March::PLANES; ++j) {
-          copy(j);
-          if (j + 1 < planes) q += sn;
+          if (j < planes) copy(j);
+          if (j < last) q += sn;
         }
       }
     };
