@@ -62,6 +62,9 @@ struct Engine {
   // Face layers each CTA of k_sweep marches through (set by hgks_autotune or
   // hgks_set_sweep_shape); 0: automatic.
   int sweep_chunk = 0;
+  // Rows each block of k_march takes (set while an ensemble is captured, whose
+  // members share the SMs); 0: an even split of the grid's rows over all SMs.
+  int march_share = 0;
 };
 
 // Turbulence statistics (turbulence.cuh): raw sums, each the sum over cells
@@ -141,6 +144,8 @@ template <class T> cudaError_t enqueue_from_fp64(const Engine& e, const double* 
 template <class T> cudaError_t enqueue_to_fp64(const Engine& e, double* dst);
 // Whether the sweeps run in k_march (march.cuh), else in k_sweep (sweep_tile.cuh).
 bool sweeps_march(const hgks_config& c);
+// Rows per block of k_march for grids that run at the same time.
+int march_share(const std::vector<Engine*>& members);
 // Adjoint of one S2O4 step at the state e.q with the step dt already in
 // e.scal[0]: adj_out = (dQ^{n+1}/dQ^n)^T adj_in (FP64 device arrays, [5][N]).
 template <class T> cudaError_t enqueue_adjoint_step(const Engine& e, const double* adj_in,

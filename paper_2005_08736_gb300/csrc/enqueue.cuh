@@ -137,14 +137,29 @@ SweepArgs3<T> sweep_args(const Engine& e, const T* q) {
   return a;
 }
 
-// k_march: every block takes the same number of rows of the sequence of all
-// tiles' rows (march_block), so that the blocks, one per SM, finish together;
-// at least two rows, since each stretch repeats four rows of face fields (a
-// quarter of a row's work each).  This is the only launch shape: shorter
-// stretches repeat more and longer ones leave SMs idle (256^3: 8.55 ms a step,
-// 8.56 to 8.88 with 526 to 64 rows a block instead of 1,051, 10.2 with 8;
-// 128 x 128 x 96 with walls 0.93, 1.00 with 16; 32^3 77 us, 97 with 8).
-inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks) {
+// Rows per block of k_march for grids of so many rows that run at the same
+// time: every block takes the same number of rows of the sequence of all
+// tiles' rows (march_block), and the blocks are no more than the SMs, one each,
+// so that they finish together; at least two rows, since each stretch repeats
+// four rows of face fields (a quarter of a row's work each).  This is the only
+// launch shape: shorter stretches repeat more and longer ones leave SMs idle
+// (256^3: 8.55 ms a step, 8.56 to 8.88 with 526 to 64 rows a block instead of
+// 1,051, 10.2 with 8; 128 x 128 x 96 with walls 0.93, 1.00 with 16; 32^3 77 us,
+// 97 with 8).
+inline int march_share_of(const std::vector<long long>& rows, int sms) {
+  long long all = 0;
+  for (const long long r : rows) all += r;
+  const auto blocks = [&](long long share) {
+    long long n = 0;
+    for (const long long r : rows) n += (r + share - 1) / share;
+    return n;
+  };
+  long long share = std::max(2LL, (all + sms - 1) / sms);
+  while (share < all && blocks(share) > sms) ++share;
+  return int(share);
+}
+
+inline SweepArgs3<float> march_args(const Engine& e, const float* q) {
   SweepArgs3<float> a = sweep_common(e, q);
   for (int d = 0; d < 3; ++d) {
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
@@ -153,21 +168,19 @@ inline SweepArgs3<float> march_args(const Engine& e, const float* q, int& blocks
     a.chunk[d] = 0;
     a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[S];
   }
-  const int rows = a.start[3];
-  a.share = std::max(2, (rows + e.sms - 1) / e.sms);
-  blocks = (rows + a.share - 1) / a.share;
+  a.share = e.march_share > 0 ? e.march_share : march_share_of({a.start[3]}, e.sms);
   return a;
 }
+inline int march_blocks(const SweepArgs3<float>& a) { return (a.start[3] + a.share - 1) / a.share; }
 
 template <class T, int MODE, int FLUX, int STAGE>
 cudaError_t launch_sweep(const Engine& e, const T* q) {
   if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
-    int blocks;
-    const SweepArgs3<float> a = march_args(e, q, blocks);
+    const SweepArgs3<float> a = march_args(e, q);
     const cudaError_t err = cudaFuncSetAttribute(k_march<STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)March::SMEM);
     if (err != cudaSuccess) return err;
-    k_march<STAGE><<<blocks, March::THREADS, March::SMEM, e.stream>>>(a);
+    k_march<STAGE><<<march_blocks(a), March::THREADS, March::SMEM, e.stream>>>(a);
     return cudaGetLastError();
   } else {
     constexpr int TP = SweepTile<T, FLUX>::TP, TS = SweepTile<T, FLUX>::TS;
@@ -497,9 +510,8 @@ cudaError_t batched_sweeps(const std::vector<Engine*>& ms, int stage, cudaStream
   if constexpr (std::is_same<T, float>::value && MODE == RECON_LINEAR && FLUX == FLUX_SMOOTH) {
     std::vector<MarchJob<STAGE>> jobs;
     for (Engine* e : ms) {
-      int nb;
-      jobs.push_back({march_args(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs), nb)});
-      blocks.push_back(nb);
+      jobs.push_back({march_args(*e, static_cast<const T*>(stage == 1 ? e->q : e->qs))});
+      blocks.push_back(march_blocks(jobs.back().a));
     }
     return launch_batched(jobs, blocks, March::SMEM, s);
   } else {

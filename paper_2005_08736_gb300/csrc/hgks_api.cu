@@ -1013,10 +1013,16 @@ static hgks_status capture_ensemble(hgks_ensemble* en, hgks_ensemble::Slot& sl, 
     return HGKS_E_CUDA;
   }
   const int n = (int)en->members.size();
+  // Members that march share the SMs: each alone would fill them all.
+  std::vector<hgks::Engine*> ms, marching;
+  for (hgks_ctx* c : en->members) {
+    ms.push_back(&c->e);
+    if (hgks::sweeps_march(c->e.cfg)) marching.push_back(&c->e);
+  }
+  const int share = marching.empty() ? 0 : hgks::march_share(marching);
+  for (hgks::Engine* e : marching) e->march_share = share;
   if (en->batched) {
     // One launch per phase over all members, on the first member's stream.
-    std::vector<hgks::Engine*> ms;
-    for (hgks_ctx* c : en->members) ms.push_back(&c->e);
     err = en->members[0]->e.cfg.prec == HGKS_FP32 ? hgks::enqueue_batched_step<float>(ms, dt_fixed, s0)
                                                    : hgks::enqueue_batched_step<double>(ms, dt_fixed, s0);
   } else {
@@ -1031,6 +1037,7 @@ static hgks_status capture_ensemble(hgks_ensemble* en, hgks_ensemble::Slot& sl, 
       if (err == cudaSuccess) err = cudaStreamWaitEvent(s0, en->events[i + 1], 0);
     }
   }
+  for (hgks::Engine* e : marching) e->march_share = 0;
   const cudaError_t end = cudaStreamEndCapture(s0, &g);
   if (err == cudaSuccess) err = end;
   if (err == cudaSuccess) err = cudaGraphInstantiate(&sl.graph, g, 0);
