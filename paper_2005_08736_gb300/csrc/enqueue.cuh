@@ -159,14 +159,23 @@ inline int march_share_of(const std::vector<long long>& rows, int sms) {
   return int(share);
 }
 
+// P is the transverse axis that is contiguous in memory, unless the grid is so
+// thin along it that the other one gives at most two fifths of the rows: a row
+// costs the same whatever part of its 32 faces exists.  Between two fifths and
+// two thirds the strided loads cost what the fewer rows save (one step, P
+// contiguous / exchanged: 6 x 128 x 128 294 / 169 us, 8 x 200 x 50 207 / 148,
+// 12 x 64 x 64 112 / 96; but 16 x 128 x 128 292 / 287, 128 x 16 x 128 243 / 259,
+// 20 x 100 x 160 332 / 382, 16 x 24 x 64 78 / 104).
 inline SweepArgs3<float> march_args(const Engine& e, const float* q) {
   SweepArgs3<float> a = sweep_common(e, q);
   for (int d = 0; d < 3; ++d) {
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
-    a.gx[d] = (e.n[P] + March::TP - 1) / March::TP;
+    const auto tiles = [&](int p) { return (e.n[p] + March::TP - 1) / March::TP; };
+    a.swap[d] = 5LL * tiles(S) * e.n[P] <= 2LL * tiles(P) * e.n[S];
+    a.gx[d] = tiles(a.swap[d] ? S : P);
     a.gy[d] = (a.layers[d] + March::LAYERS - 1) / March::LAYERS;
     a.chunk[d] = 0;
-    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[S];
+    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[a.swap[d] ? P : S];
   }
   a.share = e.march_share > 0 ? e.march_share : march_share_of({a.start[3]}, e.sms);
   return a;

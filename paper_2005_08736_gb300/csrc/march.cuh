@@ -3,8 +3,8 @@
 // TRANSVERSE axis.
 //
 // A CTA owns 10 face layers along the normal n and 32 faces along P (the
-// transverse axis that is contiguous in memory) and marches row by row along
-// S, the other transverse axis.  Per row s:
+// transverse axis that is contiguous in memory, but for very thin grids,
+// march_args) and marches row by row along S, the other transverse axis.  Per row s:
 //   A  face fields (WENO5 end values, compatibility state Q0, normal slope)
 //      of row s + 2 at 32 + 4 points of P, from the row's cells, which were
 //      copied to shared memory asynchronously a row ahead;
@@ -95,7 +95,9 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
   float* cells = reinterpret_cast<float*>(outb + 2 * March::NOUT * NPT);  // [2][5][PLANES][HP], rows in turn
   const SweepArgs<float> a = sweep_of(sweeps, row >= sweeps.start[2] ? 2 : (row >= sweeps.start[1] ? 1 : 0));
   const GridDev& g = a.g;
-  const int d = a.d, P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
+  const int d = a.d;
+  const bool swap = d == 0 ? sweeps.swap[0] : (d == 1 ? sweeps.swap[1] : sweeps.swap[2]);
+  const int P = swap ? (d == 2 ? 1 : 2) : (d == 0 ? 1 : 0), S = 3 - d - P;
   const int nd = sweeps.g.n[d], nP = sweeps.g.n[P], nS = sweeps.g.n[S];
   const int layers = sweeps.layers[d];
   const int rel = row - sweeps.start[d], tile = rel / nS, tiles = sweeps.gx[d];
@@ -105,10 +107,11 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
   // Strides of the state the sweep reads, per axis, and of its variables.
   const long long sx = a.xt ? (long long)g.p[2] * g.p[1] : 1LL, sy = a.xt ? 1LL : (long long)g.p[0],
                   sz = a.xt ? (long long)g.p[1] : (long long)g.p[0] * g.p[1];
-  const long long sn = d == 0 ? sx : (d == 1 ? sy : sz), sp = P == 0 ? sx : sy, ss = S == 1 ? sy : sz;
+  const auto stride = [&](int axis) { return axis == 0 ? sx : (axis == 1 ? sy : sz); };
+  const long long sn = stride(d), sp = stride(P), ss = stride(S);
   const int gv[5] = {0, 1 + d, 1 + P, 1 + S, 4};
-  const float* wP = d == 1 ? a.wt2 : a.wt1;  // t1 = P for the x and z sweeps, S for the y sweep
-  const float* wS = d == 1 ? a.wt1 : a.wt2;
+  const bool t1P = P == (d + 1) % 3;
+  const float *wP = t1P ? a.wt1 : a.wt2, *wS = t1P ? a.wt2 : a.wt1;
 
   if (tid < March::MAKERS) {
     // A, B: point pair (layers f, f + 1; column hp).  Columns past the grid's
@@ -217,9 +220,11 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
     const long long FS = (long long)(g.n[0] + (d == 0)) * (g.n[1] + (d == 1)) * (g.n[2] + (d == 2));
     // Face-flux layout: x fastest for the y and z faces, y fastest ([z][x][y])
     // for the x faces.
-    const long long fstep = d == 0 ? g.n[1] : (d == 1 ? (long long)g.n[0] : (long long)g.n[0] * g.n[1]);
-    const long long rstep = d == 0 ? (long long)(g.n[0] + 1) * g.n[1]
-                                   : (d == 1 ? (long long)g.n[0] * (g.n[1] + 1) : (long long)g.n[0]);
+    const long long ox = d == 0 ? (long long)g.n[1] : 1LL, oy = d == 0 ? 1LL : (long long)g.n[0],
+                    oz = (long long)(g.n[0] + (d == 0)) * (g.n[1] + (d == 1));
+    const auto ostride = [&](int axis) { return axis == 0 ? ox : (axis == 1 ? oy : oz); };
+    const long long fstep = ostride(d), rstep = ostride(S);
+    long long fi = (long long)s0 * rstep + (long long)(fo + m) * fstep + (p0 + ip) * ostride(P);
     __syncthreads();
 #pragma unroll 1
     for (int r = s0 - 2; r <= s1 + 2; ++r) {
@@ -250,7 +255,6 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
         }
         flux_smooth_x2<STAGE == 1>(pt[0], a.gas, Fs);
         flux_smooth_x2<STAGE == 1>(pt[1], a.gas, Fs);
-        const long long fi = (long long)s * rstep + (long long)(fo + m) * fstep + p0 + ip;
 #pragma unroll
         for (int k = STAGE == 1 ? 0 : 1; k < 2; ++k) {
           // The second stage needs dF only (Eq. (6)); its F planes are not written.
@@ -263,6 +267,7 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
             if (face && fo + m == 0 && layers == nd) out[nd * fstep] = sum;  // periodic: face n is face 0
           }
         }
+        fi += rstep;
       }
       __syncthreads();
     }

@@ -41,6 +41,7 @@ struct SweepArgs3 {
   GridDev g;
   int gx[3], gy[3], chunk[3], start[4];
   int share;           // k_march: rows per block (start counts rows)
+  int swap[3];         // k_march: P and S exchanged
   int layers[3];       // face layers to compute: n + 1, or n where face n is face 0
   Gas<T> gas;
 };
