@@ -28,7 +28,7 @@
 namespace hgks {
 
 // Whether the midpoint rule applies to the jump dd about the mean dm (FP32).
-__device__ __forceinline__ bool compat_small_jump(const float dm[5], const float dd[5], const Gas<float>& g) {
+HGKS_HD bool compat_small_jump(const float dm[5], const float dd[5], const Gas<float>& g) {
   const float rho = g.rho_r + dm[0];
   const float ke2 = (dm[1] * dm[1] + dm[2] * dm[2] + dm[3] * dm[3]) / rho;
   const float p = g.p_r + g.gm1 * (dm[4] - 0.5f * ke2);
@@ -78,8 +78,7 @@ HGKS_HD void compat_state(const T dql[5], const T dqr[5], const Gas<T>& g, T dq0
 // Returns false, with Q0 undefined, if the rule does not apply to both points
 // (compat_small_jump: its density, sound-speed and pressure scales are
 // formed from the same reciprocals).
-__device__ __forceinline__ bool compat_jump_x2(const float2 dm[5], const float2 dd[5], const Gas<float>& g,
-                                               float2 Q0[5]) {
+HGKS_HD bool compat_jump_x2(const float2 dm[5], const float2 dd[5], const Gas<float>& g, float2 Q0[5]) {
   const float2 rho = add2(bc2(g.rho_r), dm[0]);
   const float2 inv = rcp2(rho);
   const float2 U = mul2(dm[1], inv), V = mul2(dm[2], inv), W = mul2(dm[3], inv);
@@ -148,9 +147,8 @@ __device__ __forceinline__ bool compat_jump_x2(const float2 dm[5], const float2 
 // and the jump keeps its relative precision.  The compatibility state by the
 // midpoint rule in pair arithmetic when both points' jumps are small, else
 // per point.
-__device__ __forceinline__ void face_fields_smooth_linear_x2(const float2 qk[5][6], float2 r6,
-                                                             const Gas<float>& g, float2 Q0[5],
-                                                             float2 D0[5]) {
+HGKS_HD void face_fields_smooth_linear_x2(const float2 qk[5][6], float2 r6, const Gas<float>& g, float2 Q0[5],
+                                          float2 D0[5]) {
   float2 dm[5], dd[5];
   const float2 r84 = mul2(bc2(14.f), r6), mr6 = mul2(bc2(-1.f), r6);
 #pragma unroll

@@ -63,15 +63,15 @@ struct March {
 // low-Mach flow are what is left over).
 struct DerivCoef {
   float2 a, b;
-  __device__ __forceinline__ explicit DerivCoef(float w) {
+  HGKS_HD explicit DerivCoef(float w) {
     a = bc2(1.f / (6.f * (w + w)));
     b = bc2((1.7320508075688772f / 54.f) / w);
   }
 };
 
 // tangential_linear_x2 with the derivatives per unit length.
-__device__ __forceinline__ void tangential_linear_scaled_x2(float2 f0, float2 f1, float2 f2, float2 f3, float2 f4,
-                                                            const DerivCoef& c, float2 v[2], float2 d[2]) {
+HGKS_HD void tangential_linear_scaled_x2(float2 f0, float2 f1, float2 f2, float2 f3, float2 f4, const DerivCoef& c,
+                                         float2 v[2], float2 d[2]) {
   const float sq3 = 1.7320508075688772f;
   const float2 s13 = add2(f1, f3), s04 = add2(f0, f4);
   const float2 d04 = sub2(f0, f4), d31 = sub2(f3, f1);

@@ -55,6 +55,7 @@ HGKS_HD float2 rcp2(float2 a) { return make_float2(1.f / a.x, 1.f / a.y); }
 //   rounded 719/720 would scale every face value,
 //   O = sqrt3 (7/432 (f0-f4) + 25/216 (f3-f1)),
 //   A = (f0-f4)/12 + 2(f3-f1)/3,  B = sqrt3/54 (13 (f1+f3) - 24 f2 - (f0+f4)).
+// The host checks alone call it: k_march takes tangential_linear_scaled_x2.
 HGKS_HD void tangential_linear_x2(float2 f0, float2 f1, float2 f2, float2 f3,
                                                      float2 f4, float2 v[2], float2 d[2]) {
   const float sq3 = 1.7320508075688772f;
