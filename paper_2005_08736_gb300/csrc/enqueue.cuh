@@ -171,11 +171,11 @@ inline SweepArgs3<float> march_args(const Engine& e, const float* q) {
   for (int d = 0; d < 3; ++d) {
     const int P = d == 0 ? 1 : 0, S = d == 2 ? 1 : 2;
     const auto tiles = [&](int p) { return (e.n[p] + March::TP - 1) / March::TP; };
-    a.swap[d] = 5LL * tiles(S) * e.n[P] <= 2LL * tiles(P) * e.n[S];
-    a.gx[d] = tiles(a.swap[d] ? S : P);
+    const bool exchange = 5LL * tiles(S) * e.n[P] <= 2LL * tiles(P) * e.n[S];
+    a.gx[d] = tiles(exchange ? S : P);
     a.gy[d] = (a.layers[d] + March::LAYERS - 1) / March::LAYERS;
-    a.chunk[d] = 0;
-    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[a.swap[d] ? P : S];
+    a.chunk[d] = exchange ? 1 : 0;
+    a.start[d + 1] = a.start[d] + a.gx[d] * a.gy[d] * e.n[exchange ? P : S];
   }
   a.share = e.march_share > 0 ? e.march_share : march_share_of({a.start[3]}, e.sms);
   return a;

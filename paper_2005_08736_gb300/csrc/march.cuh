@@ -19,7 +19,7 @@
 // 700 and 600 instructions each, so both halves finish together and the FMA
 // pipe sees all sixteen warps all the time.
 //
-// Why this split: marching along the normal instead (the tiles of sweep.cuh)
+// Why this split: marching along the normal instead (the tiles of sweep_tile.cuh)
 // recomputes the face fields of a halo of two on all four sides (1.69x for a
 // 32 x 8 tile) and the first tangential pass on two (1.31x), and its passes
 // alternate over the CTA with five barriers per two layers; there the face
@@ -96,8 +96,7 @@ __device__ __forceinline__ int march_rows(const SweepArgs3<float>& sweeps, int r
   const SweepArgs<float> a = sweep_of(sweeps, row >= sweeps.start[2] ? 2 : (row >= sweeps.start[1] ? 1 : 0));
   const GridDev& g = a.g;
   const int d = a.d;
-  const bool swap = d == 0 ? sweeps.swap[0] : (d == 1 ? sweeps.swap[1] : sweeps.swap[2]);
-  const int P = swap ? (d == 2 ? 1 : 2) : (d == 0 ? 1 : 0), S = 3 - d - P;
+  const int P = a.chunk ? (d == 2 ? 1 : 2) : (d == 0 ? 1 : 0), S = 3 - d - P;
   const int nd = sweeps.g.n[d], nP = sweeps.g.n[P], nS = sweeps.g.n[S];
   const int layers = sweeps.layers[d];
   const int rel = row - sweeps.start[d], tile = rel / nS, tiles = sweeps.gx[d];

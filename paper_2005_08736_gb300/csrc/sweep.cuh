@@ -30,7 +30,8 @@ struct SweepArgs {
 // The three sweeps of a stage in one launch: block b belongs to direction d
 // with start[d] <= b < start[d + 1].  The sweeps are independent of each
 // other, so one grid fills the chip on grids where one direction cannot
-// (32^3: 24 tiles a direction) and has one tail instead of three.
+// (32^3: 8 tiles of k_sweep, 4 of k_march a direction) and has one tail
+// instead of three.
 template <class T>
 struct SweepArgs3 {
   const T* q;          // padded state
@@ -39,9 +40,9 @@ struct SweepArgs3 {
   const T* w[3];
   const double* scal;
   GridDev g;
-  int gx[3], gy[3], chunk[3], start[4];
-  int share;           // k_march: rows per block (start counts rows)
-  int swap[3];         // k_march: P and S exchanged
+  int gx[3], gy[3], chunk[3], start[4];  // k_march: chunk is whether P and S are exchanged,
+                                         // start counts rows
+  int share;           // k_march: rows per block
   int layers[3];       // face layers to compute: n + 1, or n where face n is face 0
   Gas<T> gas;
 };
