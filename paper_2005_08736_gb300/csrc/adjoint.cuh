@@ -4,9 +4,9 @@
 // buffer.  There is no counterpart in the paper (its scheme has no adjoint);
 // the step's adjoint is assembled from two such evaluations in hgks_api.cu.
 //
-// The kernel mirrors the forward sweep (sweep.cuh) tile by tile and layer by
-// layer.  For each face layer it first recomputes the face fields and the t1
-// pass into shared memory, then runs the reverse:
+// The kernel mirrors the forward sweep (sweep_tile.cuh) tile by tile and layer
+// by layer.  For each face layer it first recomputes the face fields and the
+// t1 pass into shared memory, then runs the reverse:
 //   R3  per Gauss point: the cotangent of the face flux from the divergence
 //       (Eq. (4)), the vector-Jacobian product of the flux at the point, and
 //       the transposed t2 pass, accumulated into shared memory;

@@ -3,10 +3,10 @@
 // and the update of each stage) covering every instance of the ensemble.  The
 // instance table is a kernel parameter (__grid_constant__: it stays in the
 // constant bank, no copy): instance m owns the blocks [start[m], start[m+1])
-// of the grid, and each block runs the same body as the single-instance
-// kernel (kernels.cuh, sweep.cuh) on its instance's arguments and its local
-// block coordinates.  No block waits on another: the phases are ordered by
-// the stream (and the captured graph) only.
+// of the grid, and each block runs the same body as the single-instance kernel
+// (kernels.cuh, sweep_tile.cuh, march.cuh) on its instance's arguments and its
+// local block coordinates.  No block waits on another: the phases are ordered
+// by the stream (and the captured graph) only.
 #pragma once
 
 #include "kernels.cuh"

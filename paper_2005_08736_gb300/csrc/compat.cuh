@@ -137,7 +137,7 @@ HGKS_HD bool compat_jump_x2(const float2 dm[5], const float2 dd[5], const Gas<fl
 
 // Face fields of the smooth flux (Q0 and its normal slope) at two points:
 // qk[i][k] = variable i of cell f-3+k at both points (conservative variables,
-// linear weights; face_fields_cells in sweep.cuh), r6 = 1/(6 (hl + hr)) of
+// linear weights; face_fields_cells, sweep.cuh), r6 = 1/(6 (hl + hr)) of
 // each.  With the cells' differences D_k = q_k - q_{k-1} the WENO5 end values
 // (2, -13, 47, 27, -3)/60 of both sides have the mean and the jump
 //   (Ql + Qr)/2 = q2 + D3/2 + (7 (D2 - D4) - (D1 - D5))/60,

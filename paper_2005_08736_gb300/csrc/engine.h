@@ -28,7 +28,7 @@ struct Engine {
   void* q = nullptr;     // padded state Q^n (deviation), 5 * P
   void* qs = nullptr;    // padded state Q*, then Q^{n+1}, 5 * P
   void* qx = nullptr;    // padded state with x slowest, [5][x][z][y], read by the x sweep
-                         // (null: the x sweep reads q with pair loads along x)
+                         // (null: the x sweep reads q, strided)
   void* inc = nullptr;   // stage-1 increment, 5 * N
   void* comp = nullptr;  // FP32 compensation of Q^n, 5 * N (null for FP64)
   void* comp2 = nullptr; // FP32 compensation of Q^{n+1}, 5 * N (null for FP64)

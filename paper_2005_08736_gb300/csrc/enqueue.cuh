@@ -74,9 +74,13 @@ cudaError_t enqueue_ghosts(const Engine& e, void* qbuf, bool copy, Probe* probe)
 
 // Tile of k_sweep, TP x TS faces.  FP64 is bound by its pipe, not by latency:
 // with the smooth flux one CTA of 512 threads has 1.56 points of face fields
-// per face where two of 16 x 8 faces have 1.88 (128^3: 44.3 -> 40.5 ms a step
-// against one CTA of 16 x 8).  FP32 needs the second CTA's other phase: the full
-// flux on 16 x 16 tiles, one CTA, takes 58.1 ms at 256^3, on 16 x 8 56.3.
+// per face where two of 16 x 8 faces have 1.88 (a step on 16 x 8 / 16 x 16:
+// linear 128^3 44.3 / 40.5 ms; WENO-Z 64^3 16.4 / 15.4, in characteristic
+// variables, whose 128 registers spill up to 712 bytes, 20.8 / 19.3; on grids
+// of little more than a tile the smaller one would do, 12 x 10 x 9 0.45 / 0.58
+// and 0.55 / 0.72, 40 x 36 x 20 with walls 2.54 / 2.82).  FP32 needs the second
+// CTA's other phase: the full flux on 16 x 16 tiles, one CTA, takes 58.1 ms at
+// 256^3, on 16 x 8 56.3.
 template <class T, int FLUX> struct SweepTile {
   static constexpr int TP = 16, TS = sizeof(T) == 8 && FLUX == FLUX_SMOOTH ? 16 : 8;
 };

@@ -5,8 +5,8 @@
 // rho W, rho E) of (nx+6)(ny+6)(nz+6) cells, x fastest, 3 ghost layers on
 // every side, holding deviations from the reference state at rest.
 //
-// Per stage, the fused sweep kernel (sweep.cuh) writes the face fluxes of
-// each direction; k_update then forms L = -(1/|Omega|) sum F (Eq. (4)) and
+// Per stage, the fused sweep kernels (sweep_tile.cuh, march.cuh) write the
+// face fluxes of each direction; k_update then forms L = -(1/|Omega|) sum F (Eq. (4)) and
 // the S2O4 stage (Eq. (6)).  Ghost fills, the CFL and diagnostic reductions
 // and the state conversions are here too.
 #pragma once
@@ -30,34 +30,13 @@ __host__ __device__ __forceinline__ long long pad_index(const GridDev& g, int x,
   return ((long long)(z + kGhost) * g.p[1] + (y + kGhost)) * g.p[0] + (x + kGhost);
 }
 
-// Extents and offsets of the face-field box of direction d: faces 0..n_d
-// along d, tangential rows -2..n+1 along the two other axes.
-struct FaceBox {
-  int r[3], o[3];
-  long long size;
-};
-__host__ __device__ __forceinline__ FaceBox face_box(const GridDev& g, int d, int tang_halo) {
-  FaceBox b;
-  for (int c = 0; c < 3; ++c) {
-    if (c == d) {
-      b.r[c] = g.n[c] + 1;
-      b.o[c] = 0;
-    } else {
-      b.r[c] = g.n[c] + 2 * tang_halo;
-      b.o[c] = -tang_halo;
-    }
-  }
-  b.size = (long long)b.r[0] * b.r[1] * b.r[2];
-  return b;
-}
-
 // ------------------------------------------------------------- ghost cells ---
 
 // The ghost fill and the CFL reduction are bodies over explicit block
-// coordinates (device functions) with thin __global__ wrappers; the update
-// and the sweep keep their bodies in the kernels, as included texts
-// (update_body.inc).  The ensemble's batched launches
-// (batch.cuh) run the same bodies for many instances in one grid.
+// coordinates (device functions) with thin __global__ wrappers, as the sweeps
+// are; the update keeps its body in the kernel, as an included text
+// (update_body.inc).  The ensemble's batched launches (batch.cuh) run the same
+// bodies for many instances in one grid.
 
 // Ghost cells of the padded state q and, if qx is not null, the copy of the
 // padded state with x slowest, qx[v][x][z][y] (ghosts included), that the x

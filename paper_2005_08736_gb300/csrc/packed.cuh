@@ -1,14 +1,13 @@
-// Packed FP32 pairs for the sweep kernel: one instruction applies an add,
+// Packed FP32 pairs for the sweep kernels: one instruction applies an add,
 // multiply or fused multiply-add to both halves of a float2 (__fadd2_rn /
-// __fmul2_rn / __ffma2_rn, sm_100 and later).  The sweep kernel is bound by
-// instruction issue, not by the FMA pipe, so evaluating two points in the
-// halves of one float2 halves the issue slots of their arithmetic.
+// __fmul2_rn / __ffma2_rn, sm_100 and later).  The FP32 sweeps are bound by
+// instruction issue before the FMA pipe, so evaluating two reconstructions in
+// the halves of one float2 halves the issue slots of their arithmetic.
 //
-// In the last phase the two halves are the two t1 Gauss abscissae of one
-// face; the shared-memory layout of the t1 pass keeps them adjacent, so one
-// 64-bit load fetches both.  In the face-field phase they are two adjacent
-// points of a face layer (compat.cuh).  The formulas are those of recon.cuh (linear tangential
-// reconstruction) and physics.cuh (smooth flux), evaluated pairwise; only the
+// In k_march (march.cuh) the halves are two adjacent face layers, from the
+// cells to the flux; in k_sweep (sweep_tile.cuh) and the adjoint two fields of
+// one point, in its face fields the two cells of a face.  The formulas are
+// those of recon.cuh, compat.cuh and physics.cuh, evaluated pairwise; only the
 // rounding of the fused operations can differ from the scalar code.
 #pragma once
 

@@ -21,12 +21,12 @@
 // Why by groups: the full flux's three at once need 90 planes of t1-pass values
 // and three point states in registers (FP32: 210 KB and 246 registers, 8 warps
 // per SM, FMA pipe 54 % active).  One group needs 30 planes and one point
-// state: 111 KB and 128 registers without spills, 16 warps per SM in two CTAs
-// whose phases overlap.  In FP64 the tile grows from 8 x 8 to 16 x 8 (face
+// state: 111 KB and 128 registers (16 bytes of spills at most), 16 warps per SM
+// in two CTAs whose phases overlap.  In FP64 the tile grows from 8 x 8 to 16 x 8 (face
 // fields at 1.9 points per face instead of 2.25), and every reconstruction of
 // the pass along t2 serves both abscissae.
 // Measured (GB300, one step): FP32 WENO-Z + full flux 256^3 73.4 -> 59.9 ms
-// (56.3 with the strides as constants and shorter chunks); in characteristic
+// (56.3 with the strides as constants and shorter marches); in characteristic
 // variables 90x75x67 2.59 -> 2.24 ms; eight boxes of 32^3 to 96^3 11.4 -> 8.92
 // ms; FP64 WENO-Z + full flux 64^3 71.1 -> 46.0 ms.
 // Bound by the FMA pipe and instruction issue (FP32), the FP64 pipe (FP64).
