@@ -9,13 +9,12 @@
 // by the stream (and the captured graph) only.
 #pragma once
 
+#include "engine.h"
 #include "kernels.cuh"
 #include "march.cuh"
 #include "sweep_tile.cuh"
 
 namespace hgks {
-
-constexpr int kBatchMax = 32;  // instances per batched launch
 
 template <class Job>
 struct BatchTable {

@@ -142,6 +142,8 @@ template <class T> cudaError_t enqueue_sweep_only(const Engine& e);
 template <class T> cudaError_t enqueue_diag(const Engine& e);
 template <class T> cudaError_t enqueue_from_fp64(const Engine& e, const double* src, int conservative);
 template <class T> cudaError_t enqueue_to_fp64(const Engine& e, double* dst);
+constexpr int kBatchMax = 32;  // members per batched launch
+
 // Whether the sweeps run in k_march (march.cuh), else in k_sweep (sweep_tile.cuh).
 bool sweeps_march(const hgks_config& c);
 // Rows per block of k_march for grids that run at the same time.

@@ -1013,14 +1013,23 @@ static hgks_status capture_ensemble(hgks_ensemble* en, hgks_ensemble::Slot& sl, 
     return HGKS_E_CUDA;
   }
   const int n = (int)en->members.size();
-  // Members that march share the SMs: each alone would fill them all.
+  // Members that march at the same time share the SMs, each alone would fill
+  // them all: those of one batched launch, and about eight branches (64 boxes
+  // of 32^3, us a step: alone 2165, four 1658, eight 1602, sixteen 1615, all 32
+  // of a device queue 1814; 24 of 12^3 262, 262, 237, 251, 268).  A branch of
+  // sixteen rows per SM or more gains nothing (three of 96^3 1420 alone, 1448).
   std::vector<hgks::Engine*> ms, marching;
   for (hgks_ctx* c : en->members) {
     ms.push_back(&c->e);
-    if (hgks::sweeps_march(c->e.cfg)) marching.push_back(&c->e);
+    if (hgks::sweeps_march(c->e.cfg) && (en->batched || hgks::march_share({&c->e}) < 16)) marching.push_back(&c->e);
   }
-  const int share = marching.empty() ? 0 : hgks::march_share(marching);
-  for (hgks::Engine* e : marching) e->march_share = share;
+  const size_t group = en->batched ? hgks::kBatchMax : 8;
+  for (size_t i0 = 0; i0 < marching.size(); i0 += group) {
+    const std::vector<hgks::Engine*> together(marching.begin() + i0,
+                                              marching.begin() + std::min(marching.size(), i0 + group));
+    const int share = hgks::march_share(together);
+    for (hgks::Engine* e : together) e->march_share = share;
+  }
   if (en->batched) {
     // One launch per phase over all members, on the first member's stream.
     err = en->members[0]->e.cfg.prec == HGKS_FP32 ? hgks::enqueue_batched_step<float>(ms, dt_fixed, s0)

@@ -51,9 +51,10 @@ def test_members_with_other_stored_shapes_share_batched_launches():
     ens.close()
 
 
-def test_members_of_a_batch_share_the_chip():
-    # 24 boxes of 32^3 in one launch against one box of as many cells: 1.6
-    # times as long; with every member split over all SMs 2.1 times.
+@pytest.mark.parametrize("batched", [True, False])
+def test_members_of_an_ensemble_share_the_chip(batched):
+    # 24 boxes of 32^3 against one box of as many cells: 1.6 times as long
+    # (1.4 as branches); with every member split over all SMs 2.1 (1.9) times.
     def step_ms(step, stream):
         step()
         ms = []
@@ -69,7 +70,7 @@ def test_members_of_a_batch_share_the_chip():
     n = (64, 96, 128)
     one = Simulation(Config(*n, prec=1))
     one.init_primitive(inputs.random_smooth(n, seed=1, amp=0.05, p0=100 / 1.4))
-    ens = Ensemble([simulation(32) for _ in range(24)], batched=True)
+    ens = Ensemble([simulation(32) for _ in range(24)], batched=batched)
     batch = step_ms(lambda: ens.step(4, 1e-4, sync=False), ens.sims[0].stream)
     single = step_ms(lambda: one.step(4, 1e-4, sync=False), one.stream)
     assert batch <= 1.8 * single, (batch, single)
