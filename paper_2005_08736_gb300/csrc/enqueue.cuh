@@ -108,7 +108,10 @@ SweepArgs3<T> sweep_common(const Engine& e, const T* q) {
 // Layers of direction d that each CTA of k_sweep or k_sweep_adj marches
 // through.  The march along the normal carries nothing from one layer to the
 // next, so its length only sets the number of CTAs: 24 per SM for the three
-// directions, down to one layer each on small grids.  No march is longer than a
+// directions, down to one layer each on small grids (24 / 48 / 96 per SM, one
+// step: FP32 WENO-Z + full flux 256^3 55.2 / 54.2 / 54.0 ms and 96^3 2.92 / 2.93 /
+// 2.95, WENO-JS + smooth 100x83x77 0.946 / 0.944 / 0.964, FP64 linear 128^3 40.4 /
+// 40.7 / 40.8; hgks_autotune finds what suits a grid).  No march is longer than a
 // tenth of an SM's share of all layers: in a direction of few tiles and many
 // layers it would finish long after the others (long boxes, one step: FP64
 // WENO-Z + full flux 6 x 6 x 512 21.7 -> 9.2 ms, FP32 16 x 16 x 200 269 -> 207
