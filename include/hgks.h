@@ -117,6 +117,12 @@ hgks_status hgks_init_conservative(hgks_ctx* ctx, const double* cons, int is_hos
  * is_host != 0. */
 hgks_status hgks_get_state(hgks_ctx* ctx, double* cons_out, int is_host);
 
+/* Copy the conservative state out to a DEVICE buffer that belongs to another
+ * stream (a cudaStream_t of the context's device): the copy runs on that
+ * stream, after the work already enqueued on the context's, whose later work
+ * waits for it.  Does not synchronise. */
+hgks_status hgks_get_state_on(hgks_ctx* ctx, double* cons_out, void* stream);
+
 /* Set the simulated time and the step counter (both reset to 0 by
  * hgks_init_state / hgks_init_conservative): with hgks_get_state and
  * hgks_init_conservative this checkpoints and resumes a run.  step >= 0

@@ -20,7 +20,7 @@ STATUS_NAMES = {0: "OK", 1: "E_INVAL", 2: "E_NOMEM", 3: "E_CUDA", 4: "E_NONPHYSI
 
 # Entry points declared in include/hgks.h.
 EXPORTS = ["hgks_default_config", "hgks_create", "hgks_destroy", "hgks_init_state",
-           "hgks_init_conservative", "hgks_get_state", "hgks_step", "hgks_diagnostics",
+           "hgks_init_conservative", "hgks_get_state", "hgks_get_state_on", "hgks_step", "hgks_diagnostics",
            "hgks_adjoint_step", "hgks_profile_step", "hgks_step_noalloc", "hgks_last_error",
            "hgks_ensemble_create", "hgks_ensemble_step", "hgks_ensemble_destroy",
            "hgks_ensemble_last_error", "hgks_autotune", "hgks_set_sweep_shape",
@@ -114,6 +114,7 @@ def load(path: str | None = None):
         L.hgks_init_state.argtypes = [vp, vp, i]
         L.hgks_init_conservative.argtypes = [vp, vp, i]
         L.hgks_get_state.argtypes = [vp, vp, i]
+        L.hgks_get_state_on.argtypes = [vp, vp, vp]
         L.hgks_step.argtypes = [vp, i, d, i, pd]
         L.hgks_diagnostics.argtypes = [vp, ctypes.POINTER(HgksDiag)]
         L.hgks_turbulence_stats.argtypes = [vp, ctypes.POINTER(HgksTurbulence)]

@@ -21,6 +21,7 @@ struct hgks_ctx {
   double graph_dt[2] = {0.0, 0.0};
   void* buf0 = nullptr;  // the state buffer allocated first
   int device = 0;
+  cudaEvent_t order[2] = {nullptr, nullptr};  // of hgks_get_state_on: before and after the copy
   // Host mirror of the device step counter: steps enqueued since the state
   // was set (init_steps: the counter when it was set).  Used to find the last
   // good state after a non-physical one.
@@ -382,6 +383,8 @@ hgks_status hgks_destroy(hgks_ctx* c) {
   cudaStreamSynchronize(c->e.stream);
   drop_graphs(c);
   free_all(c->e);
+  for (cudaEvent_t ev : c->order)
+    if (ev) cudaEventDestroy(ev);
   if (c->own_stream) cudaStreamDestroy(c->e.stream);
   delete c;
   return HGKS_OK;
@@ -431,6 +434,22 @@ hgks_status hgks_get_state(hgks_ctx* c, double* out, int is_host) {
     HGKS_CHECK(c, cudaMemcpyAsync(out, e.io, 5 * e.N * sizeof(double), cudaMemcpyDeviceToHost, e.stream));
     HGKS_CHECK(c, cudaStreamSynchronize(e.stream));
   }
+  return HGKS_OK;
+}
+
+hgks_status hgks_get_state_on(hgks_ctx* c, double* out, void* stream) {
+  if (!c || !out) return fail(c, HGKS_E_INVAL, "null argument");
+  hgks::Engine on = c->e;
+  on.stream = static_cast<cudaStream_t>(stream);
+  if (on.stream == c->e.stream) return hgks_get_state(c, out, 0);
+  for (cudaEvent_t& ev : c->order)
+    if (!ev) HGKS_CHECK(c, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  HGKS_CHECK(c, cudaEventRecord(c->order[0], c->e.stream));
+  HGKS_CHECK(c, cudaStreamWaitEvent(on.stream, c->order[0], 0));
+  HGKS_CHECK(c, on.cfg.prec == HGKS_FP32 ? hgks::enqueue_to_fp64<float>(on, out)
+                                          : hgks::enqueue_to_fp64<double>(on, out));
+  HGKS_CHECK(c, cudaEventRecord(c->order[1], on.stream));
+  HGKS_CHECK(c, cudaStreamWaitEvent(c->e.stream, c->order[1], 0));
   return HGKS_OK;
 }
 

@@ -178,10 +178,13 @@ class Simulation:
             self._call(self.lib.hgks_get_state(self.h, ctypes.c_void_p(out.data_ptr()), 1))
             return out
         if device:
+            # Written on the current stream, whose memory it is: work queued
+            # there may still read what was freed to make it.  (The simulation's
+            # stream writing after a wait for that work ran the members of an
+            # ensemble one after another, 1 to 2 % of a step with its output.)
             out = torch.empty(self.cfg.shape, dtype=torch.float64, device=self.device)
-            self._call(self.lib.hgks_get_state(self.h, ctypes.c_void_p(out.data_ptr()), 0))
-            out.record_stream(self.stream)
-            torch.cuda.current_stream(self.device).wait_stream(self.stream)
+            current = torch.cuda.current_stream(self.device).cuda_stream
+            self._call(self.lib.hgks_get_state_on(self.h, ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(current)))
             return out
         out = np.empty(self.cfg.shape)
         self._call(self.lib.hgks_get_state(self.h, ctypes.c_void_p(out.ctypes.data), 1))
