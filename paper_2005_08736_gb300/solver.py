@@ -116,7 +116,11 @@ class Simulation:
             raise RuntimeError("a CUDA device is required")
         self.cfg = cfg
         self.device = torch.device("cuda", torch.cuda.current_device())
-        self.stream = stream if stream is not None else torch.cuda.Stream(self.device)
+        # The default stream cannot be captured: like no stream, it stands for
+        # one of the simulation's own, with which every caller's stream is
+        # ordered (the library's own choice would be unknown here).
+        own = stream is None or stream.cuda_stream == 0
+        self.stream = torch.cuda.Stream(self.device) if own else stream
         self._c = cfg.c_struct()
         h = ctypes.c_void_p()
         _lib.check(self.lib.hgks_create(ctypes.byref(self._c), ctypes.c_void_p(self.stream.cuda_stream),
@@ -152,12 +156,17 @@ class Simulation:
         return ctypes.c_void_p(arr.ctypes.data), 1, arr
 
     def init_primitive(self, prim) -> None:
+        """Set the state from primitive cell values (rho, u, v, w, p).  A device
+        tensor is read on the simulation's stream, after the work queued on the
+        current one; the call does not wait for it, so write the tensor again
+        only after a call that does (state, step with sync)."""
         p, host, keep = self._fp64_arg(prim)
         self._call(self.lib.hgks_init_state(self.h, p, host))
         if not host:
             keep.record_stream(self.stream)
 
     def init_conservative(self, cons) -> None:
+        """Set the state from conservative averages (as init_primitive)."""
         p, host, keep = self._fp64_arg(cons)
         self._call(self.lib.hgks_init_conservative(self.h, p, host))
         if not host:
