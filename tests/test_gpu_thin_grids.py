@@ -44,10 +44,14 @@ def test_thin_grids_match_the_oracle(n, walls):
 def test_a_thin_grid_costs_no_more_than_half_again_along_another_axis():
     # 6 x 128 x 128 once took 2.5 times as long as 128 x 128 x 6 (and longer
     # than the kernels before); now 1.5 times, of the whole step.
-    ms = []
+    sims = []
     for n in ((6, 128, 128), (128, 128, 6)):
         sim = Simulation(Config(*n, prec=1))
         sim.init_primitive(inputs.random_smooth(n, seed=2, amp=0.05, p0=100 / 1.4))
-        sim.step(2)
-        ms.append(min(sim.profile_step()["flux_stage1"] for _ in range(5)))
+        sim.step(20)
+        sims.append(sim)
+    ms = [1e30, 1e30]
+    for _ in range(8):
+        for k, sim in enumerate(sims):
+            ms[k] = min(ms[k], sim.profile_step()["flux_stage1"])
     assert ms[0] <= 1.9 * ms[1], ms
